@@ -1645,6 +1645,18 @@ struct KTimer {
   }
 };
 
+// An on-chip solve's steps in C chunks of L.  prop: every chunk's propagator is computed
+// (all chunks side by side) and the states and co-states at the chunk boundaries follow by
+// products; otherwise one serial pass each writes them.  par: the gradient's chunks run
+// side by side, R per launch; otherwise one after the other, the co-state handed on.
+struct OcChunks {
+  bool prop = false, par = false;
+  int L = 1, C = 1, R = 1;
+  int G = 1, NG = 1;              // prop: chunks per group of the two-level product, groups
+  double2 *ck = nullptr, *lam = nullptr;   // states before, co-states after each chunk
+  double2 *U = nullptr, *P = nullptr;      // chunk and group propagators
+};
+
 struct Solve {
   KTimer kt;
   Setup s;
@@ -1673,13 +1685,17 @@ struct Solve {
   const double2* adj_tab = nullptr;
   const float2* adj_tab32 = nullptr;
   double* J_dev = nullptr;        // coupling strengths (batched on-chip adjoint launches)
-  // the generic gather kernels only: their cross-densities read the forward rows
-  // (xa.tabrow) while the apply reads adj_tab; the tiled and on-chip adjoints contract
-  // the coupling cross-densities with the rows they apply
-  bool force_gather = false;
+  // the co-state is pulled back with rows of its own (adj_tab); no_tiled: and the coupling
+  // cross-densities are wanted too, which the gather and on-chip kernels contract with the
+  // forward rows but the tiled adjoint with the rows it applies
+  bool two_rows = false, no_tiled = false;
+  // on-chip: the solve's chunks of steps (plan_chunks)
+  OnchipPlan* ocp = nullptr;      // propagator plan (D columns)
+  OcChunks ch;
   ~Solve() {
     slab_plan_destroy(slab);
     onchip_plan_destroy(oc);
+    onchip_plan_destroy(ocp);
   }
   // the on-chip kernels evolve this solve (gradient solves need the adjoint to fit too)
   bool onchip(bool grad) const { return oc && (grad ? onchip_adjoint_ok(oc) : onchip_forward_ok(oc)); }
@@ -1734,9 +1750,9 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
   // plans first: they upload their offset tables, and every host-to-device copy of
   // a solve goes before its first kernel (see dcopy)
   sv.mixed = o->precision == SG_MIXED;
-  const int pc = sv.force_gather ? 2 : path_choice();
-  if (pc == 0) sv.oc = onchip_plan_create(s.p, sv.mixed, s.K, s.sumd, st);
-  if (pc <= 1 && !(sv.oc && onchip_adjoint_ok(sv.oc))) sv.slab = slab_plan_create(s.p, sv.mixed, st);
+  const int pc = path_choice();
+  if (pc == 0) sv.oc = onchip_plan_create(s.p, sv.mixed, s.K, s.sumd, st, sv.two_rows);
+  if (pc <= 1 && !sv.no_tiled && !(sv.oc && onchip_adjoint_ok(sv.oc))) sv.slab = slab_plan_create(s.p, sv.mixed, st);
   // mixed precision on the on-chip kernels reads only FP32 tables
   const bool f32only = sv.mixed && sv.onchip(grad);
   sv.drives_dev = sv.ar.get<DriveDev>(std::max(1, s.K));
@@ -1908,6 +1924,169 @@ void dcopy(double2* dst, const double2* src, long long n, cudaStream_t st) {
   k_cast<double><<<grid_for(n), kT, 0, st>>>(src, dst, n, 1.0);
 }
 
+// --- on-chip solves in chunks of steps -----------------------------------------------
+// The step maps are linear, so a chunk's propagator does not depend on the state it
+// starts from: with D small, every chunk evolves the identity side by side, and products
+// give the states at the chunk boundaries (App. A's product of short-time propagators,
+// over longer pieces).  The co-states follow with the adjoints in reverse order.  Then
+// every chunk has its start state and its end co-state, and all chunks recompute and pull
+// back side by side.  A serial evolution keeps one CTA per column group busy for all N
+// steps (the D = 25 pair: one CTA of 152 SMs).
+//
+// kPropCtas: the propagators cost a chunk ctas(D columns) CTAs where the serial pass costs
+// ctas(S columns), so they pay as long as enough chunks fit side by side: up to 32 CTAs a
+// chunk (D <= 256 at the level counts here), at least 4 chunks at once.  Beyond that the
+// boundary states come from one serial pass each way.
+constexpr int kPropCtas = 32;
+constexpr int kMinChunk = 4;      // steps: below this the products outweigh the steps saved
+constexpr size_t kSegBytes = 1ull << 30;
+
+void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
+  Setup& s = sv.s;
+  OcChunks& c = sv.ch;
+  c = OcChunks{};
+  const int N = s.N;
+  c.L = N;
+  const long long simg = onchip_state_elems(sv.oc);
+  const size_t stage = (size_t)onchip_stage_elems(sv.oc) * (sv.mixed ? sizeof(float2) : sizeof(double2));
+  const int ncta = onchip_ctas(sv.oc);
+  // gradient chunks that run at once
+  const int slots = grad ? std::max(1, 152 * onchip_adj_resident(sv.oc) / ncta) : 1;
+  const size_t accb = (size_t)ncta * onchip_acc_doubles(sv.oc) * sizeof(double);
+  auto bytes = [&](int C, int L, int R, size_t nprop) {
+    return 2 * (size_t)C * simg * sizeof(double2) + (size_t)R * L * 4 * stage + (size_t)R * accb +
+           (size_t)C * nprop * sizeof(double2);
+  };
+  auto fit_rounds = [&](int C, int L) {                 // chunks per launch within the segment store
+    const size_t per = std::max<size_t>(1, (size_t)L * 4 * stage);
+    long long R = std::max<long long>(1, (long long)(kSegBytes / per));
+    if (R > slots) R = R / slots * slots;               // whole waves
+    return (int)std::min<long long>(R, C);
+  };
+  if (s.D <= 256 && N >= 2 * kMinChunk) {
+    KPlan pd = s.p;
+    pd.S = (int)s.D;
+    sv.ocp = onchip_plan_create(pd, sv.mixed, s.K, s.sumd, sv.ar.st, false, true);
+    const int nD = sv.ocp && onchip_forward_ok(sv.ocp) ? onchip_ctas(sv.ocp) : 0;
+    const int most = nD ? 152 * onchip_fwd_resident(sv.ocp) / nD : 0;
+    if (nD && nD <= kPropCtas && most >= 4) {
+      c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + most - 1) / most);
+      c.C = (N + c.L - 1) / c.L;
+      c.prop = c.par = c.C > 1;
+      c.R = grad ? fit_rounds(c.C, c.L) : 1;
+      // The product's order.  One level: C dependent matrix-times-column products.  Two: the
+      // C - 1 products of every group with D columns (over the SMs), then C/G + G dependent ones.
+      const double D = (double)s.D, one = c.C;
+      int G = std::max(1, (int)std::lround(std::sqrt((double)c.C)));
+      const double two = c.C * D / 152.0 + 2.0 * G + c.C / (double)G;
+      c.G = c.C;
+      if (two < one) c.G = G;
+      c.NG = (c.C + c.G - 1) / c.G;
+      const size_t nprop = (size_t)s.D * onchip_columns(sv.ocp) + (c.NG > 1 ? (size_t)s.D * s.D / c.G + 1 : 0);
+      if (c.prop && bytes(grad ? c.C : 0, c.L, grad ? c.R : 0, 0) + c.C * nprop * sizeof(double2) <= work_limit) return;
+      c = OcChunks{};
+      c.L = N;
+    }
+  }
+  if (!grad) return;
+  // boundary states by serial passes; segments of L steps
+  if (slots > 1 && N > kMinChunk) {
+    if (ckpt > 0) {
+      c.L = std::min(ckpt, N);
+    } else {
+      const size_t most = std::max<size_t>(1, kSegBytes / (4 * stage * slots));   // steps per chunk that fit
+      const long long waves = (N + (long long)(most * slots) - 1) / (long long)(most * slots);
+      c.L = std::max<int>(kMinChunk, (int)((N + slots * waves - 1) / (slots * waves)));
+    }
+    c.C = (N + c.L - 1) / c.L;
+    c.R = fit_rounds(c.C, c.L);
+    c.par = c.C > 1;
+    if (!c.par || bytes(c.C, c.L, c.R, 0) <= work_limit) return;
+    c = OcChunks{};
+  }
+  c.L = ckpt > 0 ? ckpt : std::max(1, (int)std::lround(std::sqrt((double)N)));
+  c.L = std::min(c.L, N);
+  c.C = (N + c.L - 1) / c.L;
+  c.R = 1;
+}
+
+// A gradient solve's chunks and the states before them.
+sg_status alloc_chunks(sg_ctx* ctx, Solve& sv, int ckpt) {
+  plan_chunks(sv, true, ckpt, ctx->work_limit);
+  sv.ch.ck = sv.ar.get<double2>((size_t)sv.ch.C * onchip_state_elems(sv.oc));
+  if (!sv.ch.ck) return sg_fail(ctx, SG_E_NOMEM, "device allocation of checkpoints failed");
+  return SG_OK;
+}
+
+// The chunk propagators' products: columns `start` (a state image) through all chunks.
+// states: the columns before (adjoint: after) every chunk; last: the final columns.
+void chunk_products(Solve& sv, const double2* start, double2* states, double2* last, double2* groups, bool adjoint,
+                    cudaStream_t st) {
+  const Setup& s = sv.s;
+  OcChunks& c = sv.ch;
+  const long long simg = onchip_state_elems(sv.oc), DD = (long long)s.D * s.D;
+  const int cols = onchip_columns(sv.oc);
+  OnchipChain a;
+  a.D = (int)s.D;
+  a.adjoint = adjoint;
+  a.state_stride = simg;
+  if (c.NG > 1) {
+    a.U = c.P; a.u_stride = DD; a.C = a.G = c.NG;
+    a.start = start; a.states = states ? groups : nullptr; a.last = last;
+    sv.launches += onchip_chain(a, cols, 1, st);
+    if (!states) return;
+    a.start = groups; a.start_stride = simg;
+  } else {
+    a.start = start;
+    a.last = last;
+  }
+  a.U = c.U; a.u_stride = (long long)onchip_columns(sv.ocp) * s.D; a.C = c.C; a.G = c.G;
+  a.states = states;
+  if (c.NG > 1) a.last = nullptr;
+  sv.launches += onchip_chain(a, cols, c.NG, st);
+}
+
+// sv.psi evolved in place; with sv.ch.ck, the states before every chunk kept.
+template <typename R>
+sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
+  sg_ctx* ctx = sys->ctx;
+  cudaStream_t st = ctx->stream;
+  Setup& s = sv.s;
+  OcChunks& c = sv.ch;
+  OnchipForward f;
+  f.tab = sizeof(R) == 4 ? (const void*)sv.tab32 : (const void*)sv.tab;
+  if (!c.prop) {
+    f.psi_api = f.psi_out = sv.psi;
+    f.ck_out = c.ck;
+    f.K = c.L;
+    sv.launches += onchip_forward(sv.oc, f, 0, s.N, s.N, s.dt, st);
+    SG_CUDA_TRY(ctx, cudaGetLastError());
+    return SG_OK;
+  }
+  const long long simg = onchip_state_elems(sv.oc), DD = (long long)s.D * s.D;
+  const long long uimg = (long long)onchip_columns(sv.ocp) * s.D;
+  c.U = sv.ar.get<double2>((size_t)c.C * uimg);
+  c.P = sv.ar.get<double2>(c.NG > 1 ? (size_t)c.NG * DD : 1);
+  double2* img = sv.ar.get<double2>(2 * (size_t)simg);
+  double2* groups = sv.ar.get<double2>((size_t)c.NG * simg);
+  if (!c.U || !c.P || !img || !groups) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the chunk propagators failed");
+  onchip_to_image(sv.oc, sv.psi, img, st);
+  f.ident = true;
+  f.img_out = c.U;
+  sv.launches += 1 + onchip_forward(sv.ocp, f, 0, s.N, c.L, s.dt, st);
+  if (c.NG > 1) {
+    OnchipChain a;
+    a.U = c.U; a.u_stride = uimg; a.D = (int)s.D; a.C = c.C; a.G = c.G;
+    a.last = c.P; a.last_stride = DD;
+    sv.launches += onchip_chain(a, (int)s.D, c.NG, st);
+  }
+  chunk_products(sv, img, c.ck, img + simg, groups, false, st);
+  onchip_from_image(sv.oc, img + simg, sv.psi, st);
+  ++sv.launches;
+  SG_CUDA_TRY(ctx, cudaGetLastError());
+  return SG_OK;
+}
+
 template <typename R>
 sg_status run_forward(sg_system* sys, Solve& sv, const long long* cols_dev, bool init_from_psi,
                       int ckpt_every, std::vector<double2*>* ckpts) {
@@ -1920,15 +2099,7 @@ sg_status run_forward(sg_system* sys, Solve& sv, const long long* cols_dev, bool
     k_init_cols<<<grid_for(n), kT, 0, st>>>(sv.psi, s.D, s.S, cols_dev);
     ++sv.launches;
   }
-  // on-chip: the whole evolution in one launch, checkpoints as state images
-  // (ckpts[c] = ckpts[0] + c * onchip_state_elems)
-  if (sv.onchip(ckpts != nullptr)) {
-    const void* tab = sizeof(R) == 4 ? (const void*)sv.tab32 : (const void*)sv.tab;
-    sv.launches += onchip_forward(sv.oc, tab, sv.psi, nullptr, sv.psi, ckpts ? (*ckpts)[0] : nullptr,
-                                  ckpt_every, 0, s.N, s.dt, nullptr, st);
-    SG_CUDA_TRY(ctx, cudaGetLastError());
-    return SG_OK;
-  }
+  if (sv.onchip(ckpts != nullptr)) return run_forward_onchip<R>(sys, sv);
   C* X = sv.ar.get<C>(n);
   C* Xo = sv.ar.get<C>(n);
   C* Dacc = sv.ar.get<C>(n);
@@ -2000,15 +2171,17 @@ XArgs make_xargs(const Solve& sv, GradAcc acc) {
   return xa;
 }
 
-// Adjoint on the on-chip kernels: per checkpoint segment one recompute launch that
-// stores every stage input, one adjoint launch; per-CTA accumulators summed at the end.
+// Adjoint on the on-chip kernels: the co-states after every chunk (products with the chunk
+// propagators' adjoints, or one serial pull-back), then per launch pair R chunks: a recompute
+// that stores every stage input, and the pull-back with its cross-densities; the
+// accumulators of all blocks are summed at the end.
 template <typename R>
-sg_status run_backward_onchip(sg_system* sys, Solve& sv, std::vector<double2*>& ckpts, int K,
-                              double2* pbar, GradAcc acc) {
+sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc acc) {
   typedef typename CT<R>::T C;
   sg_ctx* ctx = sys->ctx;
   cudaStream_t st = ctx->stream;
   Setup& s = sv.s;
+  OcChunks& c = sv.ch;
   const OnchipPlan* oc = sv.oc;
   const XArgs xa = make_xargs(sv, acc);
   const long long ns = onchip_state_elems(oc);
@@ -2016,23 +2189,26 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, std::vector<double2*>& 
   const int ncta = onchip_ctas(oc);
   const long long nst = 3ll * s.N;
   const int Kd = std::max(1, s.K);
+  const size_t naccd = (size_t)c.R * ncta * onchip_acc_doubles(oc);
   double2* pimg = sv.ar.get<double2>(ns);
-  C* segY = sv.ar.get<C>((size_t)4 * K * nstage);
+  C* segY = sv.ar.get<C>((size_t)4 * c.R * c.L * nstage);
   double* gFc = sv.ar.get<double>((size_t)ncta * nst * Kd);
-  double* accc = sv.ar.get<double>((size_t)ncta * onchip_acc_doubles(oc));
+  double* accc = sv.ar.get<double>(naccd);
   int* err = sv.ar.get<int>(1);
-  void* colow = onchip_colow_global(oc) ? (void*)sv.ar.get<float2>(ns) : nullptr;
-  if (!pimg || !segY || !gFc || !accc || !err || (onchip_colow_global(oc) && !colow))
+  void* colow = onchip_colow_global(oc) ? (void*)sv.ar.get<float2>((size_t)c.R * ns) : nullptr;
+  c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
+  double2* groups = c.prop ? sv.ar.get<double2>((size_t)c.NG * ns) : pimg;
+  if (!pimg || !segY || !gFc || !accc || !err || (onchip_colow_global(oc) && !colow) || !c.lam || !groups)
     return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
   SG_CUDA_TRY(ctx, cudaMemsetAsync(gFc, 0, (size_t)ncta * nst * Kd * sizeof(double), st));
-  SG_CUDA_TRY(ctx, cudaMemsetAsync(accc, 0, (size_t)ncta * onchip_acc_doubles(oc) * sizeof(double), st));
+  SG_CUDA_TRY(ctx, cudaMemsetAsync(accc, 0, naccd * sizeof(double), st));
   SG_CUDA_TRY(ctx, cudaMemsetAsync(err, 0, sizeof(int), st));
   onchip_to_image(oc, pbar, pimg, st);
   ++sv.launches;
   const void* tab = sizeof(R) == 4 ? (const void*)sv.tab32 : (const void*)sv.tab;
   const void* atab = sizeof(R) == 4 ? (sv.adj_tab32 ? (const void*)sv.adj_tab32 : tab)
                                     : (sv.adj_tab ? (const void*)sv.adj_tab : tab);
-  OnchipTables tb{atab, sv.coef, sv.ph, sv.opd_dev};
+  OnchipTables tb{tab, atab, sv.coef, sv.ph, sv.opd_dev};
   if (sizeof(R) == 4) {
     // FP32 tables (k_tables32) and an FP32 copy of the operators
     const long long nop = 2 * (long long)s.opdflat.size();
@@ -2040,16 +2216,31 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, std::vector<double2*>& 
     if (!op32 || !sv.coef32 || !sv.ph32) return sg_fail(ctx, SG_E_NOMEM, "FP32 tables missing");
     onchip_to_f32(reinterpret_cast<const double*>(sv.opd_dev), op32, nop, st);
     ++sv.launches;
-    tb = OnchipTables{atab, sv.coef32, sv.ph32, op32};
+    tb = OnchipTables{tab, atab, sv.coef32, sv.ph32, op32};
   }
-  const int nseg = (int)ckpts.size();
-  for (int c = nseg - 1; c >= 0; --c) {
-    const int n0 = c * K, n1 = std::min(s.N, n0 + K);
-    sv.launches += onchip_forward(oc, tab, nullptr, ckpts[c], nullptr, nullptr, K, n0, n1, s.dt, segY, st);
-    sv.launches += onchip_adjoint(oc, tb, segY, pimg, n0, n1, s.dt, xa, (int)nst, gFc, accc, err, colow, st);
+  if (c.prop) {
+    chunk_products(sv, pimg, c.lam, nullptr, groups, true, st);
+  } else if (c.par) {
+    OnchipForward b;
+    b.tab = atab;
+    b.img_in = pimg;
+    b.rev = true;
+    b.ck_out = c.lam;
+    b.K = c.L;
+    sv.launches += onchip_forward(oc, b, 0, s.N, s.N, s.dt, st);
+  }
+  for (int c1 = c.C; c1 > 0; c1 -= c.R) {
+    const int c0 = std::max(0, c1 - c.R), n0 = c0 * c.L, n1 = std::min(s.N, c1 * c.L);
+    OnchipForward f;
+    f.tab = tab;
+    f.img_in = c.ck + (size_t)c0 * ns;
+    f.segY = segY;
+    sv.launches += onchip_forward(oc, f, n0, n1, c.L, s.dt, st);
+    sv.launches += onchip_adjoint(oc, tb, segY, c.par ? c.lam + (size_t)c0 * ns : pimg, n0, n1, c.L, s.dt, xa,
+                                  (int)nst, gFc, accc, err, colow, st);
   }
   onchip_batcher_release();                       // the solve's last on-chip launch is issued
-  onchip_reduce(oc, gFc, accc, nst, s.K, s.p.n1, s.p.ne, acc, st);
+  onchip_reduce(oc, gFc, accc, c.R * ncta, nst, s.K, s.p.n1, s.p.ne, acc, st);
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
   int herr = 0;
@@ -2068,7 +2259,7 @@ sg_status run_backward(sg_system* sys, Solve& sv, std::vector<double2*>& ckpts, 
   cudaStream_t st = ctx->stream;
   Setup& s = sv.s;
   const long long n = s.D * s.S;
-  if (sv.onchip(true)) return run_backward_onchip<R>(sys, sv, ckpts, K, pbar, acc);
+  if (sv.onchip(true)) return run_backward_onchip<R>(sys, sv, pbar, acc);
   const bool slab = sv.slab != nullptr;
   // buffers of the gather path only (the slab path keeps a segment store instead)
   C* X = slab ? nullptr : sv.ar.get<C>(n);
@@ -2205,6 +2396,29 @@ sg_status run_backward(sg_system* sys, Solve& sv, std::vector<double2*>& ckpts, 
 
 }  // namespace
 
+size_t sg_chunk_bytes(const sg_system* sys, const sg_evolve_opts* o, bool grad) {
+  double D = 1;
+  for (const HostMode& m : sys->modes) D *= m.d;
+  if (o->solver != SG_SOLVER_RK4 || D > 4096 || sys->modes.size() < 2 || !(o->dt > 0.0)) return 0;
+  const int d = sys->modes[0].d;
+  const double N = o->T / o->dt, S = o->ncols, cs = o->precision == SG_MIXED ? 8 : 16;
+  const double image = D * (S + 16) * sizeof(double2);
+  const double seg = grad ? 4 * N * D * (S + 16) * 1.13 * cs : 0.0;      // every stage input
+  double b = 0.0, C = 0.0;
+  if (D <= 256) {
+    C = std::min(N / kMinChunk + 1, 152.0 * 32 / std::max(1.0, D * D / (d * d) / 256));
+    b += C * D * (D + 32) * 2 * sizeof(double2);
+  }
+  if (grad) {
+    const double waves = 1 + seg / kSegBytes;
+    C = std::max(C, std::min(N / kMinChunk + 1, 152.0 * 8 * waves / std::max(1.0, S * D / (d * d) / 256)));
+    const double blocks = 152.0 * 32 * std::max(1.0, S * D / (d * d) / 128);
+    const double acc = 8.0 * (130.0 * sys->drives.size() + 290.0 * sys->couplings.size() + 10.0 * sys->modes.size());
+    b += 2 * C * image + std::min(seg, 1.5 * (double)kSegBytes) + std::min(N, blocks) * acc;
+  }
+  return (size_t)(1.25 * b) + (32u << 20);
+}
+
 // Q2 evolution (on-chip) of the solve's columns, lab frame, in place in sv.psi.
 sg_status run_q2(sg_system* sys, Solve& sv, const long long* cols_dev, bool init_from_psi) {
   sg_ctx* ctx = sys->ctx;
@@ -2305,7 +2519,7 @@ sg_status run_backward_q2(sg_system* sys, Solve& sv, double2* pbar, GradAcc acc)
   if (rc != SG_OK)
     return sg_fail(ctx, rc, "the Q2 gradient needs 2..16 modes, <= 32 couplings, <= 16 drives and its buffers "
                             "in shared memory");
-  onchip_reduce(sv.oc, gFc, nullptr, nst, s.K, s.p.n1, s.p.ne, acc, st);
+  onchip_reduce(sv.oc, gFc, nullptr, 0, nst, s.K, s.p.n1, s.p.ne, acc, st);
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
   return SG_OK;
@@ -2337,6 +2551,7 @@ sg_status sg_evolve_impl(sg_system* sys, const sg_evolve_opts* o, void* psi_dev)
   rc = upload_and_tables(sys, o, sv, false);
   if (rc != SG_OK) return rc;
   sv.psi = static_cast<double2*>(psi_dev);
+  if (!s.q2 && sv.onchip(false)) plan_chunks(sv, false, 0, ctx->work_limit);
   if (s.q2) rc = run_q2(sys, sv, cols_dev, !o->col_index);
   else rc = o->precision == SG_MIXED ? run_forward<float>(sys, sv, cols_dev, !o->col_index, 0, nullptr)
                                      : run_forward<double>(sys, sv, cols_dev, !o->col_index, 0, nullptr);
@@ -2486,16 +2701,15 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
   // checkpoints
   int K = 0;
   std::vector<double2*> ckpts;
+  if (!grad && !s.q2 && sv.onchip(false)) plan_chunks(sv, false, 0, ctx->work_limit);
   if (grad && !s.q2) {             // the Q2 adjoint recomputes the states by inverse factors
     K = ckpt > 0 ? ckpt : std::max(1, (int)std::lround(std::sqrt((double)s.N)));
     K = std::min(K, s.N);
     const int nck = (s.N + K - 1) / K;
     if (sv.onchip(true)) {
-      // one block of state images, ckpts[c] = ckpts[0] + c * image size
-      const long long ns = onchip_state_elems(sv.oc);
-      double2* p = sv.ar.get<double2>((size_t)nck * ns);
-      if (!p) return sg_fail(ctx, SG_E_NOMEM, "device allocation of checkpoints failed");
-      for (int c = 0; c < nck; ++c) ckpts.push_back(p + (size_t)c * ns);
+      rc = alloc_chunks(ctx, sv, ckpt);
+      if (rc != SG_OK) return rc;
+      K = sv.ch.L;
     } else {
       for (int c = 0; c < nck; ++c) {
         double2* p = sv.ar.get<double2>(n);
@@ -2748,9 +2962,10 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
   sv.ar.st = sva.ar.st = ctx->stream;
   sv.want_ham = sva.want_ham = grad_ham != nullptr;
   // the Hamiltonian gradient contracts the coupling and energy terms with the forward
-  // rows of the non-Hermitian generator: the gather kernels keep them apart from the
-  // applied (conjugate-transposed) rows
-  sv.force_gather = sva.force_gather = grad_ham != nullptr;
+  // rows of the non-Hermitian generator: the on-chip and gather kernels keep them apart
+  // from the applied (conjugate-transposed) rows
+  sv.two_rows = sva.two_rows = true;
+  sv.no_tiled = sva.no_tiled = grad_ham != nullptr;
   rc = build_setup(&dsys, &od, sv.s);
   if (rc != SG_OK) return rc;
   rc = build_setup(&dadj, &od, sva.s);
@@ -2787,10 +3002,9 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
   const int nck = (s.N + K - 1) / K;
   std::vector<double2*> ckpts;
   if (sv.onchip(true)) {
-    const long long ns = onchip_state_elems(sv.oc);
-    double2* p = sv.ar.get<double2>((size_t)nck * ns);
-    if (!p) return sg_fail(ctx, SG_E_NOMEM, "device allocation of checkpoints failed");
-    for (int c = 0; c < nck; ++c) ckpts.push_back(p + (size_t)c * ns);
+    rc = alloc_chunks(ctx, sv, ckpt);
+    if (rc != SG_OK) return rc;
+    K = sv.ch.L;
   } else {
     for (int c = 0; c < nck; ++c) {
       double2* p = sv.ar.get<double2>(n);

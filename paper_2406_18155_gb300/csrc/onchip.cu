@@ -162,6 +162,7 @@ struct OcArgs {
   int D, S, Sc, nbc, nbt, CS, CSP, ncta, row, K, sumd, n1, ne;
   int ent;               // Sc * D entries per CTA
   int npw;               // adjoint: phase warps (the rest compute cross-densities)
+  int two;               // adjoint: separate rows to pull back with (open systems)
   int pblo_g;            // adjoint, mixed: co-state low words in global memory (shared memory short)
   // forward shared-memory byte offsets
   int f_ys, f_ks, f_ps, f_dl, f_M;
@@ -171,7 +172,7 @@ struct OcArgs {
   // partials, then the coupling unitaries when they fit
   int b_x0, b_x1, b_x2, b_x3, b_rows, b_rowcap, b_red, b_G;
   // adjoint shared-memory byte offsets
-  int a_xs, a_ks, a_ys, a_yn, a_db, a_pb, a_M, a_cf, a_ph, a_obD, a_obL, a_obR, a_ebB, a_ebL, a_ebR,
+  int a_xs, a_ks, a_ys, a_yn, a_db, a_pb, a_M, a_W, a_cf, a_ph, a_obD, a_obL, a_obR, a_ebB, a_ebL, a_ebR,
       a_jb, a_gs, a_sq;
   int rowA, Kp, sumdA;   // row, K and sumd rounded up to even counts
   long long accd;        // doubles per CTA accumulator block (global layout)
@@ -180,20 +181,23 @@ struct OcArgs {
   int wlim, skip_first;
 };
 
-// One solve of a batched launch: its tables, buffers and step range (the fields of
-// the unbatched launch's arguments).  CTAs [b ncta, (b + 1) ncta) of a batched grid
-// run solve b.
+// One solve of a launch: its tables, buffers and chunks of steps.  A solve has C chunks
+// of L steps, chunk c covering steps [n0 + c L, min(n1, n0 + (c + 1) L)), and every chunk
+// has the plan's ncta CTAs; the CTAs of solve b of a launch start at cta0[b].
 struct OcSys {
   const void* tab;
+  const void* atab;      // adjoint: rows the co-state is pulled back with (tab: the forward
+                         // rows, which the cross-densities contract)
   const void* coef;
   const void* ph;
   const void* opd;
   const double2* psi_api;
-  const double2* img_in;
+  const double2* img_in; // start images, one per chunk
+  double2* img_out;      // forward: the chunks' final images
   double2* psi_out;
   double2* ck_out;
   void* segY;
-  double2* pbar_img;
+  double2* pbar_img;     // adjoint: the co-states at the chunks' ends, one image per chunk
   double* gF_cta;
   double* acc_cta;
   int* err;
@@ -201,12 +205,26 @@ struct OcSys {
   const double* J;       // coupling strengths of the solve (Hamiltonian-gradient contraction)
   long long nstK;
   int n0, n1, K;
+  int C, L;
+  int ident;             // forward: column j starts in basis state j (a chunk's propagator)
+  int rev;               // forward: the steps backwards (the co-state's pull-back, see k_oc_fwd)
 };
 constexpr int kOcMaxBatch = 24;
 struct OcBatch {
-  int nsys;              // 0: an unbatched launch (the kernel's own arguments)
+  int nsys;
+  int cta0[kOcMaxBatch];
   OcSys s[kOcMaxBatch];
 };
+
+// The solve, chunk and CTA within the chunk that this block works on.
+__device__ __forceinline__ const OcSys& oc_locate(const OcBatch& bt, int ncta, int& chunk, int& cta) {
+  int b = 0;
+  while (b + 1 < bt.nsys && (int)blockIdx.x >= bt.cta0[b + 1]) ++b;
+  const int rel = blockIdx.x - bt.cta0[b];
+  chunk = rel / ncta;
+  cta = rel - chunk * ncta;
+  return bt.s[b];
+}
 
 template <int DL>
 __device__ __forceinline__ int oc_pos(const OcArgs& oa, int e) {
@@ -245,27 +263,26 @@ __host__ __device__ __forceinline__ int stage_row(int s) { return s == 0 ? 0 : (
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
+// Chunks of RK4 steps, one CTA group each.  rev: y_n = R_n^dag y_{n+1}, the pull-back of
+// the co-state alone.  With A(t) = -i H(t) anti-Hermitian (or the rows of H_eff^dag for
+// the open system), the conjugate transpose of the step map 1 + h/6 (A1 + 4 A2 + A3 +
+// h (A2 A1 + A2 A2 + A3 A2) + h^2/2 (A2 A2 A1 + A3 A2 A2) + h^3/4 A3 A2 A2 A1) is the same
+// polynomial with A1 and A3 exchanged and -h for h: the RK4 step of length -h that reads
+// the stage rows in reverse order.  So the same loop pulls the co-state back exactly.
 template <typename R, int DL>
 __global__ void __launch_bounds__(kST, 1)
-k_oc_fwd(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, const double2* __restrict__ psi_api,
-         const double2* __restrict__ img_in, double2* __restrict__ psi_out, double2* __restrict__ ck_out, int K,
-         int n0, int n1, double dt, typename CT<R>::T* __restrict__ segY, const __grid_constant__ OcBatch bt) {
+k_oc_fwd(const __grid_constant__ SlabPass sp, const __grid_constant__ OcArgs oa, double dt,
+         const __grid_constant__ OcBatch bt) {
   typedef typename CT<R>::T C;
-  int cta = blockIdx.x;
-  if (bt.nsys > 0) {
-    const int b = blockIdx.x / oa.ncta;
-    cta = blockIdx.x - b * oa.ncta;
-    const OcSys& d = bt.s[b];
-    tab = static_cast<const C*>(d.tab);
-    psi_api = d.psi_api;
-    img_in = d.img_in;
-    psi_out = d.psi_out;
-    ck_out = d.ck_out;
-    K = d.K;
-    n0 = d.n0;
-    n1 = d.n1;
-    segY = static_cast<C*>(d.segY);
-  }
+  int chunk, cta;
+  const OcSys& d = oc_locate(bt, oa.ncta, chunk, cta);
+  const C* __restrict__ tab = static_cast<const C*>(d.tab);
+  const int n0 = d.n0 + chunk * d.L, n1 = min(d.n1, n0 + d.L);
+  const int nsteps = n1 - n0, rev = d.rev;
+  const size_t simg = (size_t)oa.ncta * oa.ent;          // entries of a state image
+  const double2* const img_in = d.img_in ? d.img_in + (size_t)chunk * simg : nullptr;
+  C* const segY = d.segY ? static_cast<C*>(d.segY) + (size_t)4 * chunk * d.L * oa.ncta * oa.CSP : nullptr;
+  double2* const ck_out = d.ck_out;
   extern __shared__ __align__(16) unsigned char sm[];
   C* ys = reinterpret_cast<C*>(sm + oa.f_ys);
   C* ks = reinterpret_cast<C*>(sm + oa.f_ks);
@@ -274,33 +291,39 @@ k_oc_fwd(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
   C* dl = reinterpret_cast<C*>(sm + oa.f_dl);
   C* const M0 = reinterpret_cast<C*>(sm + oa.f_M);
   C* const M1 = M0 + oa.rowA;
-  const R h = (R)dt;
+  const R h = (R)(rev ? -dt : dt);
   for (int e = threadIdx.x; e < oa.ent; e += blockDim.x) {
     const int c = e / oa.D, t = e - c * oa.D;
     const int col = cta * oa.Sc + c;
     double2 v = make_double2(0.0, 0.0);
     if (img_in) v = img_in[(size_t)cta * oa.ent + e];
-    else if (col < oa.S) v = psi_api[(size_t)t * oa.S + col];
+    else if (d.ident) v.x = col == t ? 1.0 : 0.0;
+    else if (col < oa.S) v = d.psi_api[(size_t)t * oa.S + col];
     ps.set(e, v);
     ys[oc_pos<DL>(oa, e)] = ps.hi(e);
   }
-  if (n0 < n1) issue_rows<C>(tab, oa.row, 3 * n0, M0, threadIdx.x, blockDim.x);
+  // table row of stage s of the i-th step taken
+  auto row_of = [&](int i, int s) {
+    return rev ? 3 * (n1 - 1 - i) + 2 - stage_row(s) : 3 * (n0 + i) + stage_row(s);
+  };
+  if (nsteps > 0) issue_rows<C>(tab, oa.row, row_of(0, 0), M0, threadIdx.x, blockDim.x);
   cp_wait_all();
   __syncthreads();
   int buf = 0;
-  for (int step = n0; step < n1; ++step) {
-    if (ck_out && (step - n0) % K == 0) {
-      double2* ck = ck_out + ((size_t)((step - n0) / K) * oa.ncta + cta) * oa.ent;
+  for (int i = 0; i < nsteps; ++i) {
+    // the state before every K-th step, or (rev) the co-state after it
+    if (ck_out && (rev ? (i == 0 || (nsteps - i) % d.K == 0) : i % d.K == 0)) {
+      double2* ck = ck_out + ((size_t)((rev ? nsteps - 1 - i : i) / d.K) * oa.ncta + cta) * oa.ent;
       for (int e = threadIdx.x; e < oa.ent; e += blockDim.x) ck[e] = ps.get(e);
     }
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
       C* const Mc = buf ? M1 : M0;
       // next stage's table row
-      const int nstep = s < 3 ? step : step + 1, ns = s < 3 ? s + 1 : 0;
-      if (nstep < n1) issue_rows<C>(tab, oa.row, 3 * nstep + stage_row(ns), buf ? M0 : M1, threadIdx.x, blockDim.x);
+      const int ni = s < 3 ? i : i + 1, ns = s < 3 ? s + 1 : 0;
+      if (ni < nsteps) issue_rows<C>(tab, oa.row, row_of(ni, ns), buf ? M0 : M1, threadIdx.x, blockDim.x);
       if (segY) {
-        C* g = segY + ((size_t)(4 * (step - n0) + s) * oa.ncta + cta) * oa.CSP;
+        C* g = segY + ((size_t)(4 * i + s) * oa.ncta + cta) * oa.CSP;
         for (int e = threadIdx.x; e < oa.ent; e += blockDim.x) {
           const int pos = oc_pos<DL>(oa, e);
           g[pos] = ys[pos];
@@ -334,11 +357,15 @@ k_oc_fwd(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
       buf ^= 1;
     }
   }
-  if (psi_out) {
+  if (d.img_out) {
+    double2* o = d.img_out + (size_t)chunk * simg + (size_t)cta * oa.ent;
+    for (int e = threadIdx.x; e < oa.ent; e += blockDim.x) o[e] = ps.get(e);
+  }
+  if (d.psi_out) {
     for (int e = threadIdx.x; e < oa.ent; e += blockDim.x) {
       const int c = e / oa.D, t = e - c * oa.D;
       const int col = cta * oa.Sc + c;
-      if (col < oa.S) psi_out[(size_t)t * oa.S + col] = ps.get(e);
+      if (col < oa.S) d.psi_out[(size_t)t * oa.S + col] = ps.get(e);
     }
   }
 }
@@ -468,35 +495,26 @@ __device__ __forceinline__ void oc_contract(const XArgs& xa, const double* Jb, c
 
 template <typename R, int DL, bool PARX>
 __global__ void __launch_bounds__(kST, 1)
-k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, const R* __restrict__ coef,
-         const typename CT<R>::T* __restrict__ ph, const typename CT<R>::T* __restrict__ opd,
-         const typename CT<R>::T* __restrict__ segY, double2* __restrict__ pbar_img, int n0, int n1, double dt,
-         XArgs xa, double* __restrict__ gF_cta, double* __restrict__ acc_cta, long long nstK,
-         int* __restrict__ err, float2* __restrict__ pblo, const __grid_constant__ OcBatch bt) {
+k_oc_adj(const __grid_constant__ SlabPass sp, const __grid_constant__ OcArgs oa, double dt,
+         const __grid_constant__ XArgs xa, const __grid_constant__ OcBatch bt) {
   typedef typename CT<R>::T C;
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbar;
-  int cta = blockIdx.x;
-  const double* Jb = nullptr;                           // the solve's couplings (batched), else xa.J
-  if (bt.nsys > 0) {
-    const int b = blockIdx.x / oa.ncta;
-    cta = blockIdx.x - b * oa.ncta;
-    const OcSys& d = bt.s[b];
-    tab = static_cast<const C*>(d.tab);
-    coef = static_cast<const R*>(d.coef);
-    ph = static_cast<const C*>(d.ph);
-    opd = static_cast<const C*>(d.opd);
-    segY = static_cast<const C*>(d.segY);
-    pbar_img = d.pbar_img;
-    n0 = d.n0;
-    n1 = d.n1;
-    gF_cta = d.gF_cta;
-    acc_cta = d.acc_cta;
-    nstK = d.nstK;
-    err = d.err;
-    pblo = static_cast<float2*>(d.pblo);
-    Jb = d.J;
-  }
+  int chunk, cta;
+  const OcSys& dd = oc_locate(bt, oa.ncta, chunk, cta);
+  const C* __restrict__ tab = static_cast<const C*>(dd.tab);
+  const C* __restrict__ atab = static_cast<const C*>(dd.atab);
+  const bool two = atab != tab;                          // separate rows to pull back with
+  const R* __restrict__ coef = static_cast<const R*>(dd.coef);
+  const C* __restrict__ ph = static_cast<const C*>(dd.ph);
+  const C* __restrict__ opd = static_cast<const C*>(dd.opd);
+  const C* __restrict__ segY = static_cast<const C*>(dd.segY) + (size_t)4 * chunk * dd.L * oa.ncta * oa.CSP;
+  const size_t simg = (size_t)oa.ncta * oa.ent;
+  double2* __restrict__ pbar_img = dd.pbar_img + (size_t)chunk * simg;
+  const int n0 = dd.n0 + chunk * dd.L, n1 = min(dd.n1, n0 + dd.L);
+  double* __restrict__ acc_cta = dd.acc_cta + (size_t)chunk * oa.ncta * oa.accd;
+  int* __restrict__ err = dd.err;
+  float2* __restrict__ pblo = dd.pblo ? static_cast<float2*>(dd.pblo) + (size_t)chunk * simg : nullptr;
   (void)pblo;
   C* xs = reinterpret_cast<C*>(sm + oa.a_xs);
   C* ks = reinterpret_cast<C*>(sm + oa.a_ks);
@@ -512,6 +530,8 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
   }
   C* const M0 = reinterpret_cast<C*>(sm + oa.a_M);
   C* const M1 = M0 + oa.rowA;
+  C* const W0 = two ? reinterpret_cast<C*>(sm + oa.a_W) : M0;      // rows the phase warps apply
+  C* const W1 = two ? W0 + oa.rowA : M1;
   R* const cf0 = reinterpret_cast<R*>(sm + oa.a_cf);
   R* const cf1 = cf0 + oa.Kp;
   C* const ph0 = reinterpret_cast<C*>(sm + oa.a_ph);
@@ -527,7 +547,7 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
   A.gs = reinterpret_cast<R*>(sm + oa.a_gs);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nphase = oa.npw * 32;                      // phase threads: [0, nphase)
-  const int nxw = kST / 32 - oa.npw;                   // density warps: [npw, 8)
+  const int nxw = blockDim.x / 32 - oa.npw;            // density warps: [npw, nw)
   R* sq = reinterpret_cast<R*>(sm + oa.a_sq) + warp * 32;
   const R h = (R)dt;
   const int DD = DL * DL;
@@ -546,13 +566,14 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
   }
   __syncthreads();
   const unsigned img_bytes = (unsigned)(oa.CSP * sizeof(C));
-  double* gFc = gF_cta + (size_t)cta * nstK;
+  double* gFc = dd.gF_cta + (size_t)cta * dd.nstK;
   // prefetch of stage s of step n: its input into ydst, its rows into buffer b
   auto issue = [&](int n, int s, C* ydst, int b, bool skip) {
     if (threadIdx.x == 0 && !skip)
       bulk_load(ydst, segY + ((size_t)(4 * (n - n0) + s) * oa.ncta + cta) * oa.CSP, img_bytes, &mbar);
     const int q = 3 * n + stage_row(s);
     issue_rows<C>(tab, oa.row, q, b ? M1 : M0, threadIdx.x, blockDim.x);
+    if (two) issue_rows<C>(atab, oa.row, q, b ? W1 : W0, threadIdx.x, blockDim.x);
     issue_rows<R>(coef, oa.K, q, b ? cf1 : cf0, threadIdx.x, blockDim.x);
     issue_rows<C>(ph, oa.sumd, q, b ? ph1 : ph0, threadIdx.x, blockDim.x);
   };
@@ -571,7 +592,7 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
   };
   bool ok0 = true;
   if (n0 < n1) {
-    issue(n1 - 1, 3, ys, 0, oa.skip_first != 0 && cta == 0);
+    issue(n1 - 1, 3, ys, 0, oa.skip_first != 0 && blockIdx.x == 0);
     cp_wait_all();
     ok0 = mb_wait_for(&mbar, parity, oa.wlim);
     parity ^= 1;
@@ -590,7 +611,7 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
       if (more) issue(pn, psn, yn, buf ^ 1, aborted);
       if (warp < oa.npw) {
         // phase warps: ks = H kbar_s, then the adjoint epilogue
-        oc_apply<DL>(sp, oa, Mc, xs, ks, nphase, 1);
+        oc_apply<DL>(sp, oa, buf ? W1 : W0, xs, ks, nphase, 1);
         for (int e = threadIdx.x; e < oa.ent; e += nphase) {
           const int pos = oc_pos<DL>(oa, e);
           const C a = ks[pos];
@@ -646,7 +667,7 @@ k_oc_adj(SlabPass sp, OcArgs oa, const typename CT<R>::T* __restrict__ tab, cons
             for (int b = 0; b < DL; ++b)
               if ((!PARX || ((a + b) & 1)) && lane == a * DL + b) mine = acc[xd_i<DL, PARX>(a, b)];
           const C w = cmk<C>(mine.y, -mine.x);             // W = -i C
-          oc_contract<DL, R>(xa, Jb, opd, sp.x_gslot[slot], w, lane, Mc, cfs, phs, tq, q, s, A, sq, gFc);
+          oc_contract<DL, R>(xa, dd.J, opd, sp.x_gslot[slot], w, lane, Mc, cfs, phs, tq, q, s, A, sq, gFc);
         }
       }
       bool ok = true;
@@ -968,16 +989,106 @@ __global__ void k_oc_image(OcArgs oa, const double2* __restrict__ api, double2* 
   }
 }
 
+// state image -> API layout
+__global__ void k_oc_api(OcArgs oa, const double2* __restrict__ img, double2* __restrict__ api) {
+  const long long total = (long long)oa.S * oa.D;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (long long)gridDim.x * blockDim.x) {
+    const long long t = e / oa.S, col = e - t * oa.S;
+    api[e] = img[col * oa.D + t];
+  }
+}
+
 // FP64 -> FP32 copy of the per-stage phase and coefficient tables and the operators.
 __global__ void k_oc_f32(const double* __restrict__ src, float* __restrict__ dst, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     dst[i] = __double2float_rn(src[i]);
 }
 
+// u x + v, or v for x = 0: a column that an unstable step (|E dt| > 2.8 in the lab frame) blows
+// up to infinity must not reach columns that have no amplitude on its level.
+__device__ __forceinline__ double2 chain_fma(double2 u, double2 x, double2 v) {
+  return x.x != 0.0 || x.y != 0.0 ? cfma(u, x, v) : v;
+}
+
+// Products of chunk propagators with columns, FP64: block (s, g) takes column s through the
+// propagators of group g's chunks in order, or (ADJ) through their adjoints in reverse
+// order.  A matrix times one column has D^2 complex multiply-adds against D^2 entries
+// read once from L2, and the next one waits for its result, so a chunk costs a load round
+// trip plus two barriers: the D rows get `parts` threads each, with independent loads, and the
+// two-level order of the callers keeps the chain short.  ADJ reads the same column-major
+// image along its columns (a warp per output, lanes along the column), forward across
+// them, so both are coalesced.  Measured with the whole solve: the D = 16 pair's 10,000 FP64
+// steps go from 546 ms in one serial CTA to 1.40 ms (chunks 0.9 ms, products 0.1 ms), the
+// D = 25 gradient (10,000 mixed steps) from 254 to 4.6 ms.
+struct OcChainArgs {
+  OnchipChain a;
+  int ncols, rows, parts;
+};
+template <bool ADJ>
+__global__ void k_oc_chain(const __grid_constant__ OcChainArgs k) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const OnchipChain& a = k.a;
+  const int D = a.D, s = blockIdx.x, g = blockIdx.y;
+  double2* const x = reinterpret_cast<double2*>(sm);
+  double2* const part = x + D;
+  const int c0 = g * a.G, c1 = min(a.C, c0 + a.G);
+  for (int t = threadIdx.x; t < D; t += blockDim.x) {
+    double2 v = make_double2(0.0, 0.0);
+    if (a.start) v = a.start[(size_t)g * a.start_stride + (size_t)s * D + t];
+    else v.x = s == t ? 1.0 : 0.0;
+    x[t] = v;
+  }
+  __syncthreads();
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = c0; i < c1; ++i) {
+    const int c = ADJ ? c1 - 1 - (i - c0) : i;
+    const double2* __restrict__ U = a.U + (size_t)c * a.u_stride;
+    if (a.states)
+      for (int t = threadIdx.x; t < D; t += blockDim.x) a.states[(size_t)c * a.state_stride + (size_t)s * D + t] = x[t];
+    if (ADJ) {
+      for (int j = warp; j < D; j += nw) {
+        double2 v = make_double2(0.0, 0.0);
+        for (int t = lane; t < D; t += 32) v = chain_fma(cconj(U[(size_t)j * D + t]), x[t], v);
+        double re = v.x, im = v.y;
+        for (int o = 16; o > 0; o >>= 1) {
+          re += __shfl_xor_sync(0xffffffffu, re, o);
+          im += __shfl_xor_sync(0xffffffffu, im, o);
+        }
+        if (lane == 0) part[j] = make_double2(re, im);
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < D; t += blockDim.x) x[t] = part[t];
+    } else {
+      const int p = threadIdx.x / k.rows;
+      if (p < k.parts) {
+        for (int t = threadIdx.x - p * k.rows; t < D; t += k.rows) {
+          double2 v = make_double2(0.0, 0.0);
+#pragma unroll 4
+          for (int j = p; j < D; j += k.parts) v = chain_fma(U[(size_t)j * D + t], x[j], v);
+          part[p * k.rows + t] = v;
+        }
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < D; t += blockDim.x) {
+        double2 v = part[t];
+        for (int q = 1; q < k.parts; ++q) {
+          v.x += part[q * k.rows + t].x;
+          v.y += part[q * k.rows + t].y;
+        }
+        x[t] = v;
+      }
+    }
+    __syncthreads();
+  }
+  if (a.last)
+    for (int t = threadIdx.x; t < D; t += blockDim.x) a.last[(size_t)g * a.last_stride + (size_t)s * D + t] = x[t];
+}
+
 // Fixed-order sum over CTAs of the per-CTA gradient blocks.
 struct RedArgs {
   long long nstK, accd;
-  int ncta, K, n1, ne;
+  int ncta, nacc, K, n1, ne;
   GradAcc acc;
 };
 __global__ void k_oc_reduce(RedArgs r, const double* __restrict__ gF_cta, const double* __restrict__ acc_cta) {
@@ -992,7 +1103,8 @@ __global__ void k_oc_reduce(RedArgs r, const double* __restrict__ gF_cta, const 
       continue;
     }
     long long j = i - r.nstK;
-    for (int c = 0; c < r.ncta; ++c) s += acc_cta[(size_t)c * r.accd + j];
+#pragma unroll 8
+    for (int c = 0; c < r.nacc; ++c) s += acc_cta[(size_t)c * r.accd + j];
     const long long nD = 2 * r.K * MD2, nE = 2 * r.ne * MD2;
     if (j < nD) { reinterpret_cast<double*>(r.acc.obD)[j] += s; continue; }
     j -= nD;
@@ -1022,6 +1134,7 @@ struct OnchipPlan {
   OcArgs oa{};
   bool mixed = false, adj_ok = false, fwd_ok = false;
   size_t sm_fwd = 0, sm_adj = 0, limit = 0;
+  int fthreads = kST;             // forward kernel: a thread per block, whole warps
   // everything the plan is built from (the structure of the Kronecker-sum plan,
   // precision, drive count, energy-row length): plans with equal signatures are
   // equal, so their solves can share batched launches
@@ -1075,6 +1188,7 @@ void layout(OcArgs& a, int DL, size_t cs, size_t& fwd, size_t& adj) {
   a.a_db = take((size_t)a.ent * cs);
   a.a_pb = take((size_t)a.ent * (a.pblo_g ? 8 : 16));
   a.a_M = take(2 * (size_t)a.rowA * cs);
+  a.a_W = a.two ? take(2 * (size_t)a.rowA * cs) : a.a_M;
   a.a_cf = take(2 * (size_t)a.Kp * rs);
   a.a_ph = take(2 * (size_t)a.sumdA * cs);
   const int DD = DL * DL;
@@ -1093,8 +1207,8 @@ void layout(OcArgs& a, int DL, size_t cs, size_t& fwd, size_t& adj) {
 }  // namespace
 
 namespace {
-std::vector<long long> plan_signature(const KPlan& p, bool mixed, int K, int sumd) {
-  std::vector<long long> v = {mixed ? 1 : 0, K, sumd, p.nq, p.S, p.D, p.n1, p.ne, p.row, p.dl, (long long)p.par1,
+std::vector<long long> plan_signature(const KPlan& p, bool mixed, int K, int sumd, int kind) {
+  std::vector<long long> v = {mixed ? 1 : 0, kind, K, sumd, p.nq, p.S, p.D, p.n1, p.ne, p.row, p.dl, (long long)p.par1,
                               (long long)p.parL, (long long)p.parR};
   for (int i = 0; i < p.nq; ++i) { v.push_back(p.dims[i]); v.push_back(p.st[i]); }
   for (int u = 0; u < p.n1; ++u) { v.push_back(p.s1_mode[u]); v.push_back(p.s1_off[u]); }
@@ -1105,7 +1219,8 @@ std::vector<long long> plan_signature(const KPlan& p, bool mixed, int K, int sum
 }
 }  // namespace
 
-OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st) {
+OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st, bool two_rows,
+                               bool fwd_only) {
   if (p.nq < 2 || p.nq > SG_MAXQ) return nullptr;
   SlabPlanHost* h = slab_plan_create(p, mixed, st, true);
   if (!h) return nullptr;
@@ -1123,7 +1238,7 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const size_t limit = (size_t)std::max(0, optin - 1024);
   OnchipPlan* oc = new OnchipPlan();
-  oc->sig = plan_signature(p, mixed, K, sumd);
+  oc->sig = plan_signature(p, mixed, K, sumd, (two_rows ? 1 : 0) + (fwd_only ? 2 : 0));
   oc->h = h;
   oc->mixed = mixed;
   OcArgs& a = oc->oa;
@@ -1135,6 +1250,7 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
   a.sumd = sumd;
   a.n1 = p.n1;
   a.ne = p.ne;
+  a.two = two_rows ? 1 : 0;
   const size_t cs = mixed ? sizeof(float2) : sizeof(double2);
   // Columns per CTA: as many as give every thread one block per phase, within shared
   // memory (fewer CTAs per solve amortise the per-stage barriers and contractions).
@@ -1148,7 +1264,7 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
       a.Sc = sc;
       layout(a, DL, cs, fwd, adj);
       if (!best_fwd && fwd <= limit) best_fwd = sc;
-      if (!best_adj && adj <= limit) { best_adj = sc; break; }
+      if (fwd_only ? best_fwd != 0 : adj <= limit) { best_adj = sc; break; }
     }
     if (best_adj) break;
   }
@@ -1167,11 +1283,12 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
   a.ncta = (p.S + sc - 1) / sc;
   a.Sc = (p.S + a.ncta - 1) / a.ncta;
   layout(a, DL, cs, fwd, adj);
-  oc->adj_ok = adj <= limit;
+  oc->adj_ok = !fwd_only && adj <= limit;
   oc->fwd_ok = fwd <= limit;
   oc->sm_fwd = fwd;
   oc->sm_adj = adj;
   oc->limit = limit;
+  oc->fthreads = std::min(kST, (a.nbt + 31) / 32 * 32);
   // Adjoint warp split from the complex multiply-adds per stage: a phase block costs
   // 2 d^3 per edge and d^3 per 1-body term, a slot's cross-density d^3 (1-body) or
   // 2 d^3 (edge side); parity-odd operators halve both.  SG_OC_PW overrides (1..7).
@@ -1230,27 +1347,43 @@ void smem_limit_once() {
   (void)done;
 }
 
-const OcBatch& no_batch() {
-  static const OcBatch b{};
-  return b;
+// CTAs of one kernel that an SM holds at once (0 if the launch cannot run).
+template <auto kern>
+int resident(int threads, size_t smem) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// CTA ranges of a launch's solves; returns the grid.
+int lay_out(OcBatch& bt, int ncta) {
+  int g = 0;
+  for (int b = 0; b < bt.nsys; ++b) {
+    bt.cta0[b] = g;
+    g += bt.s[b].C * ncta;
+  }
+  return g;
 }
 
 template <typename R, int DL>
-int fwd_t(const OnchipPlan* oc, const void* tab, const double2* psi_api, const double2* img_in, double2* psi_out,
-          double2* ck_out, int K, int n0, int n1, double dt, void* segY, cudaStream_t st) {
-  typedef typename CT<R>::T C;
-  auto kern = k_oc_fwd<R, DL>;
+int fwd_t(const OnchipPlan* oc, OcBatch& bt, double dt, cudaStream_t st) {
   smem_limit_once<k_oc_fwd<R, DL>>();
-  kern<<<oc->oa.ncta, kST, oc->sm_fwd, st>>>(oc->h->pass[0], oc->oa, (const C*)tab, psi_api, img_in, psi_out,
-                                             ck_out, std::max(1, K), n0, n1, dt, (C*)segY, no_batch());
+  const int grid = lay_out(bt, oc->oa.ncta);
+  if (grid > 0) k_oc_fwd<R, DL><<<grid, oc->fthreads, oc->sm_fwd, st>>>(oc->h->pass[0], oc->oa, dt, bt);
   return 1;
 }
 
 template <typename R, int DL>
-int adj_t(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* pbar_img, int n0, int n1,
-          double dt, const XArgs& xa, int nst, double* gF_cta, double* acc_cta, int* err, void* pblo,
-          cudaStream_t st) {
-  typedef typename CT<R>::T C;
+int fwd_resident_t(const OnchipPlan* oc) {
+  smem_limit_once<k_oc_fwd<R, DL>>();
+  return resident<k_oc_fwd<R, DL>>(oc->fthreads, oc->sm_fwd);
+}
+
+template <typename R, int DL>
+int adj_t(const OnchipPlan* oc, OcBatch& bt, double dt, const XArgs& xa, cudaStream_t st) {
   auto kern = oc->h->allpar ? k_oc_adj<R, DL, true> : k_oc_adj<R, DL, false>;
   smem_limit_once<k_oc_adj<R, DL, true>>();
   smem_limit_once<k_oc_adj<R, DL, false>>();
@@ -1259,35 +1392,9 @@ int adj_t(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double
   oa.wlim = 1 << 22;
   if (const char* e = std::getenv("SG_TEST_WAIT_LIMIT")) oa.wlim = std::max(1, atoi(e));
   const char* sk = std::getenv("SG_TEST_SKIP_BULK");
-  oa.skip_first = sk && sk[0] == '1';
-  kern<<<oa.ncta, kST, oc->sm_adj, st>>>(oc->h->pass[0], oa, (const C*)tb.tab, (const R*)tb.coef,
-                                             (const C*)tb.ph, (const C*)tb.opd, (const C*)segY, pbar_img, n0, n1,
-                                             dt, xa, gF_cta, acc_cta, (long long)nst * std::max(1, oc->oa.K), err,
-                                             (float2*)pblo, no_batch());
-  return 1;
-}
-
-// Batched launches: bt.nsys solves of oc's plan shape, CTAs [b ncta, (b + 1) ncta)
-// running solve b.
-template <typename R, int DL>
-int fwd_batch_t(const OnchipPlan* oc, const OcBatch& bt, double dt, cudaStream_t st) {
-  smem_limit_once<k_oc_fwd<R, DL>>();
-  k_oc_fwd<R, DL><<<bt.nsys * oc->oa.ncta, kST, oc->sm_fwd, st>>>(oc->h->pass[0], oc->oa, nullptr, nullptr, nullptr,
-                                                                  nullptr, nullptr, 1, 0, 0, dt, nullptr, bt);
-  return 1;
-}
-
-template <typename R, int DL>
-int adj_batch_t(const OnchipPlan* oc, const OcBatch& bt, double dt, const XArgs& xa, cudaStream_t st) {
-  auto kern = oc->h->allpar ? k_oc_adj<R, DL, true> : k_oc_adj<R, DL, false>;
-  smem_limit_once<k_oc_adj<R, DL, true>>();
-  smem_limit_once<k_oc_adj<R, DL, false>>();
-  OcArgs oa = oc->oa;
-  oa.wlim = 1 << 22;
-  if (const char* e = std::getenv("SG_TEST_WAIT_LIMIT")) oa.wlim = std::max(1, atoi(e));
-  oa.skip_first = 0;
-  kern<<<bt.nsys * oa.ncta, kST, oc->sm_adj, st>>>(oc->h->pass[0], oa, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                   nullptr, 0, 0, dt, xa, nullptr, nullptr, 0, nullptr, nullptr, bt);
+  oa.skip_first = bt.nsys == 1 && sk && sk[0] == '1';
+  const int grid = lay_out(bt, oa.ncta);
+  if (grid > 0) kern<<<grid, kST, oc->sm_adj, st>>>(oc->h->pass[0], oa, dt, xa, bt);
   return 1;
 }
 
@@ -1340,11 +1447,11 @@ bool oc_compatible(const OcPending& a, const OcPending& b) {
 }
 
 template <typename R, int DL>
-int batch_launch_t(const OnchipPlan* oc, int kind, const OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
-  return kind == 0 ? fwd_batch_t<R, DL>(oc, bt, dt, st) : adj_batch_t<R, DL>(oc, bt, dt, *xa, st);
+int launch_t(const OnchipPlan* oc, int kind, OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
+  return kind == 0 ? fwd_t<R, DL>(oc, bt, dt, st) : adj_t<R, DL>(oc, bt, dt, *xa, st);
 }
-int batch_launch(const OnchipPlan* oc, int kind, const OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
-  OC_DISPATCH(batch_launch_t, oc, kind, bt, dt, xa, st);
+int oc_launch(const OnchipPlan* oc, int kind, OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
+  OC_DISPATCH(launch_t, oc, kind, bt, dt, xa, st);
 }
 
 }  // namespace
@@ -1375,7 +1482,7 @@ struct OcBatcher {
         cudaStreamWaitEvent(st, grp[b]->ready, 0);
         bt.s[b] = grp[b]->d;
       }
-      batch_launch(grp[0]->oc, grp[0]->kind, bt, grp[0]->dt, grp[0]->xa, st);
+      oc_launch(grp[0]->oc, grp[0]->kind, bt, grp[0]->dt, grp[0]->xa, st);
       for (OcPending* m : grp) cudaEventRecord(m->done, st);
       ++launches;
       members += bt.nsys;
@@ -1452,55 +1559,84 @@ void onchip_batcher_stats(const OcBatcher* b, long long* launches, long long* me
   if (members) *members = m->members;
 }
 
-int onchip_forward(const OnchipPlan* oc, const void* tab, const double2* psi_api, const double2* img_in,
-                   double2* psi_out, double2* ck_out, int K, int n0, int n1, double dt, void* segY,
-                   cudaStream_t st) {
-  if (tl_batcher) {
-    OcPending p{};
-    p.kind = 0;
-    p.oc = oc;
-    p.dt = dt;
-    p.d.tab = tab;
-    p.d.psi_api = psi_api;
-    p.d.img_in = img_in;
-    p.d.psi_out = psi_out;
-    p.d.ck_out = ck_out;
-    p.d.segY = segY;
-    p.d.K = std::max(1, K);
-    p.d.n0 = n0;
-    p.d.n1 = n1;
-    return tl_batcher->submit(p, st);
-  }
-  OC_DISPATCH(fwd_t, oc, tab, psi_api, img_in, psi_out, ck_out, K, n0, n1, dt, segY, st);
+namespace {
+
+// One launch, through the thread's batcher when it has one.
+int submit(const OcPending& p, cudaStream_t st) {
+  if (tl_batcher) return tl_batcher->submit(p, st);
+  OcBatch bt{};
+  bt.nsys = 1;
+  bt.s[0] = p.d;
+  bt.s[0].J = nullptr;               // the launch's own XArgs hold this solve's couplings
+  return oc_launch(p.oc, p.kind, bt, p.dt, p.xa, st);
 }
 
-int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* pbar_img, int n0,
-                   int n1, double dt, const XArgs& xa, int nst, double* gF_cta, double* acc_cta, int* err,
-                   void* colow, cudaStream_t st) {
-  if (tl_batcher) {
-    OcPending p{};
-    p.kind = 1;
-    p.oc = oc;
-    p.dt = dt;
-    p.xa = &xa;
-    p.d.tab = tb.tab;
-    p.d.coef = tb.coef;
-    p.d.ph = tb.ph;
-    p.d.opd = tb.opd;
-    p.d.segY = const_cast<void*>(segY);
-    p.d.pbar_img = pbar_img;
-    p.d.gF_cta = gF_cta;
-    p.d.acc_cta = acc_cta;
-    p.d.err = err;
-    p.d.pblo = colow;
-    p.d.J = xa.Jdev;
-    p.d.nstK = (long long)nst * std::max(1, oc->oa.K);
-    p.d.n0 = n0;
-    p.d.n1 = n1;
-    return tl_batcher->submit(p, st);
-  }
-  OC_DISPATCH(adj_t, oc, tb, segY, pbar_img, n0, n1, dt, xa, nst, gF_cta, acc_cta, err, colow, st);
+}  // namespace
+
+int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st) {
+  OcPending p{};
+  p.kind = 0;
+  p.oc = oc;
+  p.dt = dt;
+  p.d.tab = f.tab;
+  p.d.psi_api = f.psi_api;
+  p.d.img_in = f.img_in;
+  p.d.img_out = f.img_out;
+  p.d.psi_out = f.psi_out;
+  p.d.ck_out = f.ck_out;
+  p.d.segY = f.segY;
+  p.d.K = std::max(1, f.K);
+  p.d.n0 = n0;
+  p.d.n1 = n1;
+  p.d.L = std::max(1, L);
+  p.d.C = (n1 - n0 + p.d.L - 1) / p.d.L;
+  p.d.ident = f.ident ? 1 : 0;
+  p.d.rev = f.rev ? 1 : 0;
+  return submit(p, st);
 }
+
+int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* lam, int n0, int n1,
+                   int L, double dt, const XArgs& xa, int nst, double* gF_cta, double* acc_cta, int* err,
+                   void* colow, cudaStream_t st) {
+  OcPending p{};
+  p.kind = 1;
+  p.oc = oc;
+  p.dt = dt;
+  p.xa = &xa;
+  p.d.tab = tb.tab;
+  p.d.atab = tb.atab;
+  p.d.coef = tb.coef;
+  p.d.ph = tb.ph;
+  p.d.opd = tb.opd;
+  p.d.segY = const_cast<void*>(segY);
+  p.d.pbar_img = lam;
+  p.d.gF_cta = gF_cta;
+  p.d.acc_cta = acc_cta;
+  p.d.err = err;
+  p.d.pblo = colow;
+  p.d.J = xa.Jdev;
+  p.d.nstK = (long long)nst * std::max(1, oc->oa.K);
+  p.d.n0 = n0;
+  p.d.n1 = n1;
+  p.d.L = std::max(1, L);
+  p.d.C = (n1 - n0 + p.d.L - 1) / p.d.L;
+  return submit(p, st);
+}
+
+namespace {
+
+template <typename R, int DL>
+int adj_resident_t(const OnchipPlan* oc) {
+  smem_limit_once<k_oc_adj<R, DL, true>>();
+  smem_limit_once<k_oc_adj<R, DL, false>>();
+  return oc->h->allpar ? resident<k_oc_adj<R, DL, true>>(kST, oc->sm_adj)
+                       : resident<k_oc_adj<R, DL, false>>(kST, oc->sm_adj);
+}
+
+}  // namespace
+
+int onchip_fwd_resident(const OnchipPlan* oc) { OC_DISPATCH(fwd_resident_t, oc); }
+int onchip_adj_resident(const OnchipPlan* oc) { OC_DISPATCH(adj_resident_t, oc); }
 
 namespace {
 
@@ -1652,16 +1788,41 @@ void onchip_to_image(const OnchipPlan* oc, const double2* api, double2* img, cud
   k_oc_image<<<grid_of(onchip_state_elems(oc)), 256, 0, st>>>(oc->oa, api, img);
 }
 
+void onchip_from_image(const OnchipPlan* oc, const double2* img, double2* api, cudaStream_t st) {
+  k_oc_api<<<grid_of((long long)oc->oa.S * oc->oa.D), 256, 0, st>>>(oc->oa, img, api);
+}
+
+int onchip_columns(const OnchipPlan* oc) { return oc->oa.ncta * oc->oa.Sc; }
+
+int onchip_chain(const OnchipChain& a, int ncols, int ngroups, cudaStream_t st) {
+  OcChainArgs k{};
+  k.a = a;
+  k.ncols = ncols;
+  const int D = a.D;
+  // threads: D rows (padded to whole warps) times parts of the sum
+  int rows = (D + 31) / 32 * 32;
+  if (D <= 16) rows = 16;
+  k.rows = rows;
+  k.parts = std::max(1, std::min(256 / rows, (D + 3) / 4));
+  const int threads = (rows * k.parts + 31) / 32 * 32;
+  const size_t smem = (size_t)(D + rows * k.parts) * sizeof(double2);
+  const dim3 grid(ncols, ngroups);
+  if (a.adjoint) k_oc_chain<true><<<grid, threads, smem, st>>>(k);
+  else k_oc_chain<false><<<grid, threads, smem, st>>>(k);
+  return 1;
+}
+
 void onchip_to_f32(const double* src, float* dst, long long n, cudaStream_t st) {
   k_oc_f32<<<grid_of(n), 256, 0, st>>>(src, dst, n);
 }
 
-void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, long long nst, int K,
+void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, int nblk, long long nst, int K,
                    int n1, int ne, GradAcc acc, cudaStream_t st) {
   RedArgs r{};
   r.nstK = nst * std::max(1, K);
   r.accd = acc_cta ? oc->oa.accd : 0;   // no per-CTA accumulator blocks: dF/df only
   r.ncta = oc->oa.ncta;
+  r.nacc = nblk;
   r.K = K;
   r.n1 = n1;
   r.ne = ne;

@@ -17,8 +17,10 @@ struct OnchipPlan;   // opaque
 // mode has the same level count (2..5) and at least one column fits in shared memory
 // for the Q2 kernel (onchip_forward_ok / onchip_adjoint_ok tell whether the RK4
 // kernels fit too).  K drives and sumd = sum of level counts size the adjoint's
-// per-stage buffers.
-OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st);
+// per-stage buffers.  two_rows: the adjoint pulls back with rows of its own (open systems).
+// fwd_only: the columns per CTA are those of the forward kernel (propagators).
+OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st, bool two_rows = false,
+                               bool fwd_only = false);
 void onchip_plan_destroy(OnchipPlan* oc);
 // The adjoint kernel fits too (gradient solves may use the on-chip path).
 bool onchip_adjoint_ok(const OnchipPlan* oc);
@@ -30,14 +32,48 @@ int onchip_ctas(const OnchipPlan* oc);
 // doubles of one CTA's operator/energy/coupling accumulators (GradAcc layout minus gF).
 long long onchip_acc_doubles(const OnchipPlan* oc);
 
-// Forward RK4 steps n0 .. n1-1.  The start state is img_in (state image) when
-// non-null, else psi_api (D x S, column innermost).  Writes the state before step
-// n0 + c K to ck_out + c * state_elems when ck_out is non-null, the final state to
-// psi_out (API layout) when non-null, and every stage input of every step to
-// segY (stage images, slot 4 (step - n0) + stage) when non-null.  Returns launches.
-int onchip_forward(const OnchipPlan* oc, const void* tab, const double2* psi_api, const double2* img_in,
-                   double2* psi_out, double2* ck_out, int K, int n0, int n1, double dt, void* segY,
-                   cudaStream_t st);
+// RK4 steps n0 .. n1-1 in chunks of L steps, all chunks side by side in one launch (L >=
+// n1 - n0: one chunk, the serial evolution).  Every chunk starts from its image of img_in
+// (chunk-major state images), from the identity (ident: column j in basis state j), or from
+// psi_api (D x S, column innermost).  Outputs, where non-null: img_out, the chunks' final
+// images; psi_out (API layout, one chunk); ck_out, one chunk, the state before step
+// n0 + c K at ck_out + c * state_elems; segY, every stage input of every step (stage images,
+// slot 4 (step - n0) + stage).  rev: the steps backwards with their adjoint maps (one
+// chunk pulls a co-state from after step n1-1 to before step n0, and ck_out + c *
+// state_elems is the co-state after the last step of segment c).  Returns launches.
+struct OnchipForward {
+  const void* tab = nullptr;
+  const double2* psi_api = nullptr;
+  const double2* img_in = nullptr;
+  double2* img_out = nullptr;
+  double2* psi_out = nullptr;
+  double2* ck_out = nullptr;
+  int K = 1;
+  void* segY = nullptr;
+  bool ident = false, rev = false;
+};
+int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st);
+// CTAs of the forward (adjoint) launch that one SM holds at once.
+int onchip_fwd_resident(const OnchipPlan* oc);
+int onchip_adj_resident(const OnchipPlan* oc);
+// Columns of a state image, padding included.
+int onchip_columns(const OnchipPlan* oc);
+void onchip_from_image(const OnchipPlan* oc, const double2* img, double2* api, cudaStream_t st);
+// Columns through groups of G consecutive chunk propagators (FP64).  U: C column-major D x D
+// matrices, u_stride entries apart.  Group g starts from column image start + g start_stride
+// (null: the identity) and, in chunk order (adjoint: reverse order, with U^dag), writes the
+// columns before (adjoint: after) chunk c to states + c state_stride and the result to
+// last + g last_stride.
+struct OnchipChain {
+  const double2* U = nullptr;
+  const double2* start = nullptr;
+  double2* states = nullptr;
+  double2* last = nullptr;
+  long long u_stride = 0, start_stride = 0, state_stride = 0, last_stride = 0;
+  int D = 0, C = 0, G = 1;
+  bool adjoint = false;
+};
+int onchip_chain(const OnchipChain& a, int ncols, int ngroups, cudaStream_t st);
 // API layout -> state image (columns past S are zero).
 void onchip_to_image(const OnchipPlan* oc, const double2* api, double2* img, cudaStream_t st);
 // Per-stage tables the adjoint reads, in the stage precision (complex64 / float in
@@ -45,21 +81,21 @@ void onchip_to_image(const OnchipPlan* oc, const double2* api, double2* img, cud
 // coefficients (3N x K), frame phases (3N x sumd) and the flat truncated operators.
 struct OnchipTables {
   const void* tab;
+  const void* atab;      // rows the co-state is pulled back with (tab unless the plan has two_rows)
   const void* coef;
   const void* ph;
   const void* opd;
 };
-// Adjoint of steps n1-1 .. n0 from the stage inputs in segY: pbar_img (state image
-// of the co-state before the segment's last step) is pulled back in place; the
-// cross-densities of every stage are contracted into gF_cta (CTA-major, 3N x K
-// each, one store per stage slot) and acc_cta (CTA-major, onchip_acc_doubles
-// each, added to).  *err is set when a bounded wait on a bulk copy gives up.
-// Returns launches.
+// Adjoint of steps n0 .. n1-1 in chunks of L steps, side by side in one launch, from the
+// stage inputs in segY: chunk c pulls its co-state image lam + c * state_elems (the co-state
+// after its last step) back in place; the cross-densities of every stage are contracted into
+// gF_cta (CTA-major, 3N x K each, one store per stage slot) and acc_cta (chunk- and
+// CTA-major, onchip_acc_doubles each, added to).  *err is set when a bounded wait on a bulk
+// copy gives up.  Returns launches.
 // colow: when onchip_colow_global(oc), a device buffer of onchip_state_elems complex64
-// entries that holds the low words of the float-float co-state across the segments
-// of one backward sweep (contents undefined before the first segment); else null.
-int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* pbar_img, int n0,
-                   int n1, double dt, const XArgs& xa, int nst, double* gF_cta, double* acc_cta, int* err,
+// entries per chunk for the low words of the float-float co-state; else null.
+int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* lam, int n0, int n1,
+                   int L, double dt, const XArgs& xa, int nst, double* gF_cta, double* acc_cta, int* err,
                    void* colow, cudaStream_t st);
 bool onchip_colow_global(const OnchipPlan* oc);
 
@@ -69,8 +105,8 @@ bool onchip_forward_ok(const OnchipPlan* oc);
 // Element-wise FP64 -> FP32 copy (tables for the mixed-precision adjoint).
 void onchip_to_f32(const double* src, float* dst, long long n, cudaStream_t st);
 bool onchip_mixed(const OnchipPlan* oc);
-// acc += sum over CTAs (in CTA order) of the per-CTA accumulators.
-void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, long long nst, int K,
+// acc += sums in block order: of gF_cta over the plan's CTAs, of acc_cta over nblk blocks.
+void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, int nblk, long long nst, int K,
                    int n1, int ne, GradAcc acc, cudaStream_t st);
 
 // Suzuki-Trotter evolution (Sec. 2.3, App. A) of N Q2 sub-steps, lab frame, from psi_in

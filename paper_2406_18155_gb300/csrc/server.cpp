@@ -37,7 +37,8 @@ struct Req {
   std::vector<double> target;
   int kind = SG_FID_AVG;
   int want_grad = 1;
-  size_t mem = 0;
+  size_t mem = 0;                // device memory: what the solve needs, plus
+  size_t chunk_mem = 0;          // what it may take to compute its chunks side by side
   int state = 0;                 // 0 queued, 1 running, 2 done, 3 cancelled
   sg_status status = SG_OK;
   double F[2] = {0, 0};
@@ -123,6 +124,7 @@ struct sg_server {
     if (bt) onchip_batcher_bind(bt);
     sg_ctx* saved = r->sys->ctx;
     r->sys->ctx = c;
+    c->work_limit = r->chunk_mem;
     sg_status rc = SG_OK;
     if (!r->sys->prepared) rc = sg_prepare_impl(r->sys);
     int np = 0, nh = 0;
@@ -329,6 +331,9 @@ sg_status sg_server_submit(sg_server* srv, const sg_request* req, uint64_t* tick
     ++srv->rejected;
     return sg_fail(srv->ctx, SG_E_NOMEM_RETRY, "request alone exceeds the memory budget");
   }
+  // a budget too small for the chunks side by side leaves them to run one after the other
+  r->chunk_mem = std::min(sg_chunk_bytes(req->sys, &r->opts, req->want_grad != 0), srv->budget - r->mem);
+  r->mem += r->chunk_mem;
   srv->inflight[req->sys] = 1;
   r->ticket = srv->next_ticket++;
   r->submit_s = now_s(srv->t0);

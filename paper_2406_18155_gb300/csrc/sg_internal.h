@@ -52,6 +52,9 @@ struct sg_ctx {
   cudaStream_t stream = nullptr;
   std::string last_error;
   std::mutex mu;
+  // bytes that a solve may take for computing its chunks of steps side by side, beyond what
+  // one chunk after the other needs (a server's requests: their share of the budget)
+  size_t work_limit = ~size_t(0);
 };
 
 struct StageTables;  // defined in evolve.cu
@@ -117,6 +120,9 @@ void launch_open_frame_ebar(const double2* psi, const double2* bar, const long l
                             double T, double* ebar_d, cudaStream_t st);
 void launch_open_fold(int nq, const double2* opbar_d, const double* ebar_d, double2* opbar, double* ebar,
                       cudaStream_t st);
+// Upper estimate of the device memory that a solve takes for computing its chunks of steps
+// side by side (sg_ctx::work_limit), from the sizes alone.
+size_t sg_chunk_bytes(const sg_system* sys, const sg_evolve_opts* o, bool grad);
 sg_status sg_evolve_batch_impl(sg_system* const* systems, int B, const sg_evolve_opts* o, void* psi_dev);
 // red (nullable): the column-sharded solve's all-reduce (sg_fidelity_grad_sharded).
 sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double* target,

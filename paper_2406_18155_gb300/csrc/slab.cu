@@ -678,7 +678,9 @@ SlabPlanHost* slab_plan_create(const KPlan& p, bool mixed, cudaStream_t st, bool
       if (P.offB >= 0) ok = ok && add(1, P.gB);
       if (!ok) { delete h; return nullptr; }
     }
-    // offsets of the tile entries
+    // offsets of the tile entries (the on-chip kernels, which read a plan's tiles and phases
+    // only, go without)
+    if (metadata_only) continue;
     std::vector<int> off(sp.T);
     for (int t = 0; t < sp.T; ++t) {
       long long o = 0;
@@ -712,7 +714,7 @@ SlabPlanHost* slab_plan_create(const KPlan& p, bool mixed, cudaStream_t st, bool
   h->grid_fwd = (int)std::min<long long>(ntiles, 152ll * (mixed ? 3 : 1));
   h->grid_zfwd = (int)std::min<long long>(ntiles, 152ll * (mixed ? 2 : 1));
   h->grid_adj = (int)std::min<long long>(ntiles, 152ll * (mixed ? 2 : 1));
-  cudaStreamSynchronize(st);
+  if (!metadata_only) cudaStreamSynchronize(st);
   return h;
 }
 
