@@ -19,9 +19,11 @@ constexpr int kThreads = 256;
 // on the diagonal, unsorted) and V holds the eigenvectors in columns.  Rotations
 // of one round act on disjoint index pairs (round-robin tournament ordering), so
 // their row and column updates run in parallel.  Symmetric 2x2 Schur rotations.
-__device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs) {
+// (start: V holds orthonormal columns whose rotations the solver continues, A their matrix.)
+__device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs, bool start = false) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < M * M; i += nt) V[i] = (i / M == i % M) ? 1.0 : 0.0;
+  if (!start)
+    for (int i = tid; i < M * M; i += nt) V[i] = (i / M == i % M) ? 1.0 : 0.0;
   const int Mp = (M + 1) & ~1;           // even number of players; index M is a dummy when M is odd
   const int npair = Mp / 2;
   __shared__ double red[kThreads];
@@ -44,6 +46,9 @@ __device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs
     double dia_tot = red[0];
     __syncthreads();
     if (off_tot <= 1e-32 * dia_tot || off_tot == 0.0) break;
+    // entries too small to keep the test above from passing (M^2 of them add up to less than
+    // a third of its bound) are not rotated: where parity splits the matrix that is half of them
+    const double small = 1e-18 * sqrt(dia_tot);
     for (int round = 0; round < Mp - 1; ++round) {
       // pairing of this round (circle method): position 0 holds player 0,
       // position i >= 1 holds 1 + (i - 1 + round) mod (Mp - 1)
@@ -57,7 +62,7 @@ __device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs
         double c = 1.0, s = 0.0;
         if (q < M) {
           double apq = A[p * M + q];
-          if (apq != 0.0) {
+          if (fabs(apq) > small) {
             double app = A[p * M + p], aqq = A[q * M + q];
             double tau = (aqq - app) / (2.0 * apq);
             double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
@@ -73,8 +78,8 @@ __device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs
       for (int i = tid; i < npair * M; i += nt) {
         int k = i / M, col = i % M;
         int p = pairs[2 * k], q = pairs[2 * k + 1];
-        if (q >= M) continue;
         double c = cs[2 * k], s = cs[2 * k + 1];
+        if (s == 0.0) continue;
         double ap = A[p * M + col], aq = A[q * M + col];
         A[p * M + col] = c * ap - s * aq;
         A[q * M + col] = s * ap + c * aq;
@@ -84,8 +89,8 @@ __device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs
       for (int i = tid; i < npair * M; i += nt) {
         int k = i / M, row = i % M;
         int p = pairs[2 * k], q = pairs[2 * k + 1];
-        if (q >= M) continue;
         double c = cs[2 * k], s = cs[2 * k + 1];
+        if (s == 0.0) continue;
         double ap = A[row * M + p], aq = A[row * M + q];
         A[row * M + p] = c * ap - s * aq;
         A[row * M + q] = s * ap + c * aq;
@@ -129,16 +134,211 @@ __device__ void sort_and_gauge(const double* A, const double* V, int M, double* 
   __syncthreads();
 }
 
-// C = A * diag(g) * A^T for real M x M A (row-major), all in the given buffers.
-__device__ void adiag_at(const double* A, const double* g, int M, double* C) {
+// Nodes x_k and eigenvectors of the oscillator's X = (a + a^dag)/sqrt2 truncated to M states,
+// a thread per node: X is the Jacobi matrix of the orthonormal Hermite functions, so the
+// eigenvalues are the zeros of p_M in p_{j+1} = (x p_j - sqrt(j/2) p_{j-1}) / sqrt((j+1)/2)
+// (Golub and Welsch), found by bisection on the number of sign changes of p_0..p_M (its
+// Sturm sequence), and the eigenvector of x is (p_0(x), ..., p_{M-1}(x)) normalised.  W gets
+// the eigenvectors in columns.  A FP64 Jacobi solve of the same matrix took 2.3 ms (M = 50: twelve
+// sweeps of 49 rounds at 2 FP64 multiply-adds per clock), this 0.1 ms.
+__device__ void hermite_nodes(int M, double* x_out, double* W, double* beta, double* inv) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < M * M; i += nt) {
-    int r = i / M, c = i % M;
-    double acc = 0.0;
-    for (int k = 0; k < M; ++k) acc += A[r * M + k] * g[k] * A[c * M + k];
-    C[i] = acc;
+  for (int j = tid; j <= M; j += nt) {
+    beta[j] = sqrt(0.5 * j);
+    inv[j] = j ? 1.0 / sqrt(0.5 * j) : 0.0;
   }
   __syncthreads();
+  for (int k = tid; k < M; k += nt) {
+    // node k, ascending: the point below which k zeros of p_M lie
+    double lo = -sqrt(2.0 * M + 1.0), hi = -lo;
+    for (int it = 0; it < 64; ++it) {
+      const double x = 0.5 * (lo + hi);
+      if (x <= lo || x >= hi) break;
+      double p0 = 0.0, p1 = 1.0;
+      int changes = 0;                            // = zeros of p_M above x
+      for (int j = 0; j < M; ++j) {
+        const double p2 = (x * p1 - beta[j] * p0) * inv[j + 1];
+        changes += (p2 < 0.0) != (p1 < 0.0) ? 1 : 0;
+        p0 = p1;
+        p1 = p2;
+      }
+      if (M - changes > k) hi = x;
+      else lo = x;
+    }
+    const double x = 0.5 * (lo + hi);
+    x_out[k] = x;
+    double p0 = 0.0, p1 = 1.0, nn = 1.0;
+    for (int j = 0; j + 1 < M; ++j) {
+      const double p2 = (x * p1 - beta[j] * p0) * inv[j + 1];
+      p0 = p1;
+      p1 = p2;
+      nn += p1 * p1;
+    }
+    const double r = 1.0 / sqrt(nn);
+    p0 = 0.0;
+    p1 = 1.0;
+    for (int j = 0; j < M; ++j) {
+      W[j * M + k] = p1 * r;
+      const double p2 = (x * p1 - beta[j] * p0) * inv[j + 1];
+      p0 = p1;
+      p1 = p2;
+    }
+  }
+  __syncthreads();
+}
+
+// C1 = W diag(g1) W^T, C2 = W diag(g2) W^T (symmetric, half computed), W in shared memory.
+__device__ void wdw(const double* W, const double* g1, const double* g2, int M, double* C1, double* C2) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int i = tid; i < M * (M + 1) / 2; i += nt) {
+    int r = (int)((sqrt(8.0f * i + 1.0f) - 1.0f) * 0.5f);
+    while (r * (r + 1) / 2 > i) --r;
+    while ((r + 1) * (r + 2) / 2 <= i) ++r;
+    const int c = i - r * (r + 1) / 2;
+    double a1 = 0.0, a2 = 0.0;
+    for (int k = 0; k < M; ++k) {
+      const double w = W[r * M + k] * W[c * M + k];
+      a1 += w * g1[k];
+      a2 += w * g2[k];
+    }
+    C1[r * M + c] = C1[c * M + r] = a1;
+    C2[r * M + c] = C2[c * M + r] = a2;
+  }
+  __syncthreads();
+}
+
+// C = op(A) B for M x M matrices (TA: A^T); SYM: the product is symmetric, half computed.
+template <bool TA, bool SYM>
+__device__ void matmul(const double* A, const double* B, int M, double* C) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int n = SYM ? M * (M + 1) / 2 : M * M;
+  for (int i = tid; i < n; i += nt) {
+    int r, c;
+    if (SYM) {
+      r = (int)((sqrt(8.0f * i + 1.0f) - 1.0f) * 0.5f);
+      while (r * (r + 1) / 2 > i) --r;
+      while ((r + 1) * (r + 2) / 2 <= i) ++r;
+      c = i - r * (r + 1) / 2;
+    } else {
+      r = i / M;
+      c = i - r * M;
+    }
+    double a0 = 0.0, a1 = 0.0;
+    int k = 0;
+    for (; k + 1 < M; k += 2) {
+      a0 += (TA ? A[k * M + r] : A[r * M + k]) * B[k * M + c];
+      a1 += (TA ? A[(k + 1) * M + r] : A[r * M + k + 1]) * B[(k + 1) * M + c];
+    }
+    if (k < M) a0 += (TA ? A[k * M + r] : A[r * M + k]) * B[k * M + c];
+    C[r * M + c] = a0 + a1;
+    if (SYM) C[c * M + r] = a0 + a1;
+  }
+  __syncthreads();
+}
+
+// Jacobi sweeps in FP32 on A (overwritten), V from the identity: a fixed number of sweeps at
+// most, stopping at FP32's own level.
+__device__ void jacobi_f32(float* A, float* V, int M, float* cs, int* pairs) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int Mp = (M + 1) & ~1, npair = Mp / 2;
+  __shared__ float red[2][kThreads / 32];
+  for (int i = tid; i < M * M; i += nt) V[i] = (i / M == i % M) ? 1.f : 0.f;
+  __syncthreads();
+  for (int sweep = 0; sweep < 14; ++sweep) {
+    float off = 0.f, dia = 0.f;
+    for (int i = tid; i < M * M; i += nt) {
+      const float v = A[i];
+      if (i / M != i % M) off += v * v;
+      else dia += v * v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      dia += __shfl_xor_sync(0xffffffffu, dia, o);
+    }
+    if ((tid & 31) == 0) { red[0][tid >> 5] = off; red[1][tid >> 5] = dia; }
+    __syncthreads();
+    off = dia = 0.f;
+    for (int w = 0; w < nt / 32; ++w) { off += red[0][w]; dia += red[1][w]; }
+    __syncthreads();
+    if (off <= 1e-13f * dia) break;
+    for (int round = 0; round < Mp - 1; ++round) {
+      for (int k = tid; k < npair; k += nt) {
+        const int pa = k == 0 ? 0 : 1 + ((k - 1 + round) % (Mp - 1));
+        const int pb = 1 + ((Mp - 2 - k + round) % (Mp - 1));
+        const int p = min(pa, pb), q = max(pa, pb);
+        pairs[2 * k] = p;
+        pairs[2 * k + 1] = q;
+        float c = 1.f, s = 0.f;
+        if (q < M) {
+          const float apq = A[p * M + q];
+          if (apq != 0.f) {
+            const float tau = (A[q * M + q] - A[p * M + p]) / (2.f * apq);
+            const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+            c = 1.f / sqrtf(1.f + t * t);
+            s = t * c;
+          }
+        }
+        cs[2 * k] = c;
+        cs[2 * k + 1] = s;
+      }
+      __syncthreads();
+      for (int i = tid; i < npair * M; i += nt) {
+        const int k = i / M, col = i - k * M, p = pairs[2 * k], q = pairs[2 * k + 1];
+        const float c = cs[2 * k], s = cs[2 * k + 1];
+        if (s == 0.f) continue;
+        const float ap = A[p * M + col], aq = A[q * M + col];
+        A[p * M + col] = c * ap - s * aq;
+        A[q * M + col] = s * ap + c * aq;
+      }
+      __syncthreads();
+      for (int i = tid; i < npair * M; i += nt) {
+        const int k = i / M, row = i - k * M, p = pairs[2 * k], q = pairs[2 * k + 1];
+        const float c = cs[2 * k], s = cs[2 * k + 1];
+        if (s == 0.f) continue;
+        const float ap = A[row * M + p], aq = A[row * M + q];
+        A[row * M + p] = c * ap - s * aq;
+        A[row * M + q] = s * ap + c * aq;
+        const float vp = V[row * M + p], vq = V[row * M + q];
+        V[row * M + p] = c * vp - s * vq;
+        V[row * M + q] = s * vp + c * vq;
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Eigenpairs of the symmetric A (M x M, shared memory; on return diagonal) into V.  FP64 runs
+// at 2 multiply-adds per clock and SM, 1/64 of FP32, and a Jacobi solve needs about twelve
+// sweeps from scratch: so the first ones run in FP32, their eigenvectors are made orthonormal in
+// FP64 (two Newton-Schulz steps V <- V (3 - V^T V) / 2, 1e-6 -> 1e-12 -> 1e-24), and the FP64
+// Jacobi solve starts from V^T A V, whose off-diagonal is at FP32's rounding: two sweeps.  The
+// FP64 solver and its stopping test decide the result, as before.  B, C: M x M scratch (global).
+// M = 50 with the nodes above: k_build_modes 4.72 -> 1.67 ms.
+__device__ void eigen(double* A, double* V, int M, double* cs, int* pairs, double* B, double* C) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  // FP32 copies share V's place (M x M doubles hold two M x M float matrices)
+  float* Af = reinterpret_cast<float*>(V);
+  float* Vf = Af + M * M;
+  for (int i = tid; i < M * M; i += nt) Af[i] = (float)A[i];
+  __syncthreads();
+  jacobi_f32(Af, Vf, M, reinterpret_cast<float*>(cs), pairs);
+  for (int i = tid; i < M * M; i += nt) B[i] = (double)Vf[i];
+  __syncthreads();
+  for (int i = tid; i < M * M; i += nt) V[i] = B[i];
+  __syncthreads();
+  for (int it = 0; it < 2; ++it) {
+    matmul<true, true>(V, V, M, B);
+    for (int i = tid; i < M * M; i += nt) B[i] = (i / M == i % M ? 1.5 : 0.0) - 0.5 * B[i];
+    __syncthreads();
+    matmul<false, false>(V, B, M, C);
+    for (int i = tid; i < M * M; i += nt) V[i] = C[i];
+    __syncthreads();
+  }
+  matmul<false, false>(A, V, M, B);
+  matmul<true, true>(V, B, M, C);
+  for (int i = tid; i < M * M; i += nt) A[i] = C[i];
+  __syncthreads();
+  jacobi_eigen(A, V, M, cs, pairs, true);
 }
 
 struct BuildArgs {
@@ -146,7 +346,7 @@ struct BuildArgs {
   int kind[SG_MAXQ], M[SG_MAXQ], d[SG_MAXQ];
   double ej[SG_MAXQ], ec[SG_MAXQ], el[SG_MAXQ], ng[SG_MAXQ], phi_ext[SG_MAXQ];
   ModeDev md[SG_MAXQ];
-  double* scratch;   // per mode 4 * SG_MAXM^2 doubles
+  double* scratch;   // per mode 6 * SG_MAXM^2 doubles
 };
 
 // Builds H, operators and their parameter derivatives for one mode, diagonalises
@@ -162,12 +362,14 @@ __global__ void __launch_bounds__(kThreads) k_build_modes(BuildArgs a) {
   double* Vs = sm + M * M;        // M*M
   double* cs = Vs + M * M;        // 2*SG_MAXM
   int* pairs = reinterpret_cast<int*>(cs + 2 * SG_MAXM);   // 2*SG_MAXM
-  double* scr = a.scratch + (size_t)q * 4 * SG_MAXM * SG_MAXM;
-  double* W = scr;                       // X eigenvectors (fluxonium)
-  double* cosm = scr + M * M;
-  double* sinx = scr + 2 * M * M;
-  double* gvec = scr + 3 * M * M;        // M entries
-  double* gvec2 = gvec + M;              // M entries
+  double* scr = a.scratch + (size_t)q * 6 * SG_MAXM * SG_MAXM;
+  double* cosm = scr;
+  double* sinx = scr + M * M;
+  double* mm1 = scr + 2 * M * M;
+  double* mm2 = scr + 3 * M * M;
+  double* gvec = scr + 4 * M * M;        // M entries each
+  double* gvec2 = gvec + SG_MAXM;
+  double* node = gvec2 + SG_MAXM;
   const double ej = a.ej[q], ec = a.ec[q], el = a.el[q];
   double2* n_full = md.ops;
   double2* phi_full = md.ops + M * M;
@@ -191,29 +393,19 @@ __global__ void __launch_bounds__(kThreads) k_build_modes(BuildArgs a) {
     __syncthreads();
   } else {
     const double phe = a.phi_ext[q];
-    // X = (a + a^dag)/sqrt2, tridiagonal
-    for (int i = tid; i < M * M; i += nt) {
-      int r = i / M, c = i % M;
-      double x = 0.0;
-      if (c == r + 1) x = sqrt((double)(r + 1)) * M_SQRT1_2;
-      if (r == c + 1) x = sqrt((double)(c + 1)) * M_SQRT1_2;
-      A[i] = x;
-    }
-    __syncthreads();
-    jacobi_eigen(A, Vs, M, cs, pairs);
-    // nodes x_k = A_kk, eigenvectors W = Vs (order irrelevant for W f(x) W^T)
-    for (int i = tid; i < M * M; i += nt) W[i] = Vs[i];
+    // the eigenvectors of X = (a + a^dag)/sqrt2 in Vs (the recurrence's 2 (M + 1) coefficients
+    // take cs and the start of pairs)
+    hermite_nodes(M, node, Vs, cs, cs + M + 1);
     const double po = pow(8.0 * ec / el, 0.25);
     const double wp = sqrt(8.0 * ec * el);
     for (int k = tid; k < M; k += nt) {
-      double x = A[k * M + k];
+      double x = node[k];
       double arg = po * x - phe;
       gvec[k] = cos(arg);
       gvec2[k] = sin(arg) * x;
     }
     __syncthreads();
-    adiag_at(W, gvec, M, cosm);
-    adiag_at(W, gvec2, M, sinx);
+    wdw(Vs, gvec, gvec2, M, cosm, sinx);
     const double dpo[3] = {0.0, po / (4.0 * ec), -po / (4.0 * el)};
     const double dwp[3] = {0.0, wp / (2.0 * ec), wp / (2.0 * el)};
     for (int i = tid; i < M * M; i += nt) {
@@ -237,25 +429,33 @@ __global__ void __launch_bounds__(kThreads) k_build_modes(BuildArgs a) {
     }
     __syncthreads();
   }
-  jacobi_eigen(A, Vs, M, cs, pairs);
+  eigen(A, Vs, M, cs, pairs, mm1, mm2);
   sort_and_gauge(A, Vs, M, md.w, md.V);
-  // truncated energies and operators
+  // truncated energies and operators, V_d^T (O V_d)
   for (int k = tid; k < d; k += nt) md.E[k] = md.w[k] - md.w[0];
+  double2* T = reinterpret_cast<double2*>(mm1);                 // 2 x M x d
+  for (int i = tid; i < 2 * M * d; i += nt) {
+    const int op = i / (M * d), kb = i - op * M * d, k = kb / d, b = kb - k * d;
+    const double2* O = md.ops + op * M * M + k * M;
+    double2 t = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int l = 0; l < M; ++l) {
+      const double v = md.V[l * M + b];
+      t.x += O[l].x * v;
+      t.y += O[l].y * v;
+    }
+    T[i] = t;
+  }
+  __syncthreads();
   for (int i = tid; i < 2 * d * d; i += nt) {
-    int op = i / (d * d), ab = i % (d * d), ia = ab / d, ib = ab % d;
-    const double2* O = md.ops + op * M * M;
+    const int op = i / (d * d), ab = i - op * d * d, ia = ab / d, ib = ab - ia * d;
     double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
     for (int k = 0; k < M; ++k) {
-      double vk = md.V[k * M + ia];
-      if (vk == 0.0) continue;
-      double2 t = make_double2(0.0, 0.0);
-      for (int l = 0; l < M; ++l) {
-        double vl = md.V[l * M + ib];
-        t.x += O[k * M + l].x * vl;
-        t.y += O[k * M + l].y * vl;
-      }
-      acc.x += vk * t.x;
-      acc.y += vk * t.y;
+      const double v = md.V[k * M + ia];
+      const double2 t = T[(op * M + k) * d + ib];
+      acc.x += v * t.x;
+      acc.y += v * t.y;
     }
     md.opd[i] = acc;
   }
@@ -315,26 +515,30 @@ __global__ void __launch_bounds__(kThreads) k_chain(ChainArgs a) {
     double dE = hv[b * d + b] - hv[0];
     part += a.ebar[q * SG_MAXD + b] * dE;
   }
-  // operators
-  for (int i = tid; i < 2 * d * d; i += nt) {
-    int op = i / (d * d), ab = i % (d * d), ia = ab / d, ib = ab % d;
-    double2 ob = a.opbar[(q * 2 + op) * SG_MAXD * SG_MAXD + ia * SG_MAXD + ib];
-    if (ob.x == 0.0 && ob.y == 0.0) continue;
-    const double2* O = md.ops + (size_t)op * M * M;
-    const double2* dO = md.dops + ((size_t)op * 3 + p) * M * M;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k = 0; k < M; ++k) {
-      double vka = md.V[k * M + ia], dvka = dv[k * d + ia];
-      for (int l = 0; l < M; ++l) {
-        double vlb = md.V[l * M + ib], dvlb = dv[l * d + ib];
-        double2 o = O[k * M + l], dd = dO[k * M + l];
-        double w1 = dvka * vlb + vka * dvlb;
-        double w2 = vka * vlb;
-        acc.x += w1 * o.x + w2 * dd.x;
-        acc.y += w1 * o.y + w2 * dd.y;
-      }
+  // operators: for every (k, b) the three products (O V)_kb, (O dv)_kb, (dO V)_kb, then their
+  // contraction with column k of dv, V and the co-gradient; the M x d products are spread over
+  // the threads (one thread per (a, b) with M^2 terms each took 0.96 ms at M = 50, d = 5, this 0.10)
+  for (int i = tid; i < 2 * M * d; i += nt) {
+    const int op = i / (M * d), kb = i - op * M * d, k = kb / d, b = kb - k * d;
+    const double2* O = md.ops + (size_t)op * M * M + (size_t)k * M;
+    const double2* dO = md.dops + ((size_t)op * 3 + p) * M * M + (size_t)k * M;
+    double2 ov = make_double2(0.0, 0.0), odv = ov, dov = ov;
+#pragma unroll 4
+    for (int l = 0; l < M; ++l) {
+      const double v = md.V[l * M + b], w = dv[l * d + b];
+      const double2 o = O[l], dd = dO[l];
+      ov.x += o.x * v;
+      ov.y += o.y * v;
+      odv.x += o.x * w;
+      odv.y += o.y * w;
+      dov.x += dd.x * v;
+      dov.y += dd.y * v;
     }
-    part += ob.x * acc.x + ob.y * acc.y;        // Re(conj(ob) * acc)
+    for (int ia = 0; ia < d; ++ia) {
+      const double2 ob = a.opbar[(q * 2 + op) * SG_MAXD * SG_MAXD + ia * SG_MAXD + b];
+      const double va = md.V[k * M + ia], da = dv[k * d + ia];
+      part += ob.x * (da * ov.x + va * (odv.x + dov.x)) + ob.y * (da * ov.y + va * (odv.y + dov.y));   // Re(conj(ob) .)
+    }
   }
   red[tid] = part;
   __syncthreads();
@@ -570,7 +774,7 @@ sg_status sg_prepare_impl(sg_system* sys) {
   per_mode += SG_MAXD * sizeof(double);                 // E
   per_mode += 2 * SG_MAXD * SG_MAXD * sizeof(double2);  // opd
   per_mode = (per_mode + 255) & ~(size_t)255;
-  const size_t scratch_bytes = (size_t)nq * 4 * MM * sizeof(double);
+  const size_t scratch_bytes = (size_t)nq * 6 * MM * sizeof(double);
   const size_t total = per_mode * nq + scratch_bytes;
   if (sys->mode_block && sys->mode_block_bytes < total) {
     cudaFree(sys->mode_block);
@@ -665,7 +869,7 @@ sg_status sg_chain_device_params(sg_system* sys, const double2* opbar_dev, const
   a.opbar = opbar_dev;
   a.ebar = ebar_dev;
   a.out = out_dev;
-  // reuse the build scratch (4*MAXM^2 doubles per mode >= 3*3*MAXM*MAXD)
+  // reuse the build scratch (6*MAXM^2 doubles per mode >= 3*3*MAXM*MAXD)
   const size_t MM = (size_t)SG_MAXM * SG_MAXM;
   size_t per_mode = 0;
   per_mode += SG_MAXM * sizeof(double) + MM * sizeof(double) + 3 * MM * sizeof(double) +
