@@ -1253,9 +1253,8 @@ __global__ void __launch_bounds__(kT) k_xdens(XArgs a, const typename CT<R>::T* 
 // J N Suzuki-Trotter sub-steps, whose gF already carries df/dtheta up to the parameter
 // indicator (k_q2_gradtabs); a PWC sub-step feeds the segment of its step's midpoint
 // (reading R8), and no carrier co-gradient is formed.
-__global__ void k_pulse_chain(const DriveDev* drives, const double* amps, const double* gF,
-                              int K, int N, double dt, const int* pulse_off, int n_pulse, double* grad_pulse,
-                              double* omega_bar, int J) {
+__global__ void k_pulse_chain(const DriveDev* drives, const double* amps, const double* gF, int K, int N, double dt,
+                              int J, double* out, int stride) {
   const int k = blockIdx.x;
   const DriveDev dr = drives[k];
   const int np = dr.kind == SG_ENV_PWC ? dr.nseg : 1;
@@ -1264,7 +1263,10 @@ __global__ void k_pulse_chain(const DriveDev* drives, const double* amps, const 
   double* mine = part + tid * (np + 1);
   for (int x = 0; x <= np; ++x) mine[x] = 0.0;
   const int per = J > 0 ? J : 3;
-  for (int q = tid; q < per * N; q += blockDim.x) {
+  // this block's share of the stage slots
+  const long long nslot = (long long)per * N;
+  const int q0 = (int)(nslot * blockIdx.y / gridDim.y), q1 = (int)(nslot * (blockIdx.y + 1) / gridDim.y);
+  for (int q = q0 + tid; q < q1; q += blockDim.x) {
     const int n = q / per, jq = q % per;
     if (J > 0) {
       // Suzuki-Trotter: the carrier and the envelope shape are already in gF (the
@@ -1300,9 +1302,23 @@ __global__ void k_pulse_chain(const DriveDev* drives, const double* amps, const 
     }
   }
   __syncthreads();
+  double* row = out + ((size_t)k * gridDim.y + blockIdx.y) * stride;
   for (int x = tid; x <= np; x += blockDim.x) {
     double s = 0.0;
     for (int y = 0; y < (int)blockDim.x; ++y) s += part[y * (np + 1) + x];
+    row[x] = s;
+  }
+}
+
+// Sum of the blocks' shares in block order: parameter gradients and carrier co-gradients.
+__global__ void k_pulse_sum(const DriveDev* drives, const double* __restrict__ in, int stride, int nblk,
+                            const int* pulse_off, int n_pulse, double* grad_pulse, double* omega_bar) {
+  const int k = blockIdx.x;
+  const int np = drives[k].kind == SG_ENV_PWC ? drives[k].nseg : 1;
+  for (int x = threadIdx.x; x <= np; x += blockDim.x) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int y = 0; y < nblk; ++y) s += in[((size_t)k * nblk + y) * stride + x];
     if (x < np) {
       const int o = pulse_off[k] + x;
       if (o >= 0 && o < n_pulse) grad_pulse[o] = s;               // offsets come from the host plan
@@ -1651,6 +1667,8 @@ struct KTimer {
 // side by side, R per launch; otherwise one after the other, the co-state handed on.
 struct OcChunks {
   bool prop = false, par = false;
+  bool direct = false;            // one chunk whose serial passes keep every stage input
+  void *segU = nullptr;           // direct: the stage inputs of all steps
   int L = 1, C = 1, R = 1;
   int G = 1, NG = 1;              // prop: chunks per group of the two-level product, groups
   double2 *ck = nullptr, *lam = nullptr;   // states before, co-states after each chunk
@@ -1692,6 +1710,9 @@ struct Solve {
   // on-chip: the solve's chunks of steps (plan_chunks)
   OnchipPlan* ocp = nullptr;      // propagator plan (D columns)
   OcChunks ch;
+  bool real_oc = false;           // terms real up to the frame phases (rterms), interaction frame
+  OcrTerms rterms;
+  void* half = nullptr;           // onchip_half_step
   ~Solve() {
     slab_plan_destroy(slab);
     onchip_plan_destroy(oc);
@@ -1751,7 +1772,20 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
   // a solve goes before its first kernel (see dcopy)
   sv.mixed = o->precision == SG_MIXED;
   const int pc = path_choice();
-  if (pc == 0) sv.oc = onchip_plan_create(s.p, sv.mixed, s.K, s.sumd, st, sv.two_rows);
+  sv.real_oc = !s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows && real_terms(sys, s, s.ta);
+  if (sv.real_oc) {
+    OcrTerms& rt = sv.rterms;
+    rt.K = s.K;
+    rt.sumd = s.sumd;
+    for (int i = 0; i < s.nq; ++i) { rt.eoff[i] = s.ta.eoff[i]; rt.opd_off[i] = s.ta.opd_off[i]; }
+    for (int u = 0; u <= s.p.n1; ++u) rt.drv_start[u] = s.ta.drv_of_slot_start[u];
+    for (int k = 0; k < s.K; ++k) { rt.drv_list[k] = s.ta.drv_list[k]; rt.drv_op[k] = s.drives[k].op; }
+    for (int e = 0; e < s.p.ne; ++e) {
+      rt.e_opa[e] = s.ta.e_opa[e]; rt.e_opb[e] = s.ta.e_opb[e]; rt.e_part[e] = s.ta.e_zpart[e];
+    }
+  }
+  if (pc == 0)
+    sv.oc = onchip_plan_create(s.p, sv.mixed, s.K, s.sumd, st, sv.real_oc ? &sv.rterms : nullptr, sv.two_rows);
   if (pc <= 1 && !sv.no_tiled && !(sv.oc && onchip_adjoint_ok(sv.oc))) sv.slab = slab_plan_create(s.p, sv.mixed, st);
   // mixed precision on the on-chip kernels reads only FP32 tables
   const bool f32only = sv.mixed && sv.onchip(grad);
@@ -1837,10 +1871,19 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
         sv.q2grad = g32;
       }
     }
-  } else if (f32only) {
-    k_tables32<<<(unsigned)nst, 64, 0, st>>>(ta, sv.coef32, sv.ph32);
   } else {
-    k_tables<<<(unsigned)nst, 64, 0, st>>>(ta);
+    // a forward evolution with real operators reads the coefficients and phases only
+    const bool real = sv.onchip(grad) && onchip_real(sv.oc);
+    TabArgs tt = ta;
+    if (real && (!grad || onchip_real_adjoint(sv.oc))) tt.p.n1 = tt.p.ne = 0;
+    if (f32only) k_tables32<<<(unsigned)nst, 64, 0, st>>>(tt, sv.coef32, sv.ph32);
+    else k_tables<<<(unsigned)nst, 64, 0, st>>>(tt);
+    if (real) {
+      sv.half = sv.ar.get<double2>((size_t)s.D);
+      if (!sv.half) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the stage tables failed");
+      onchip_half_step(sv.oc, sv.E_dev, s.dt, sv.half, st);
+      ++sv.launches;
+    }
   }
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
@@ -1933,13 +1976,14 @@ void dcopy(double2* dst, const double2* src, long long n, cudaStream_t st) {
 // back side by side.  A serial evolution keeps one CTA per column group busy for all N
 // steps (the D = 25 pair: one CTA of 152 SMs).
 //
-// kPropCtas: the propagators cost a chunk ctas(D columns) CTAs where the serial pass costs
-// ctas(S columns), so they pay as long as enough chunks fit side by side: up to 32 CTAs a
-// chunk (D <= 256 at the level counts here), at least 4 chunks at once.  Beyond that the
-// boundary states come from one serial pass each way.
-constexpr int kPropCtas = 32;
+// kMinSide: a chunk's propagator takes the CTAs of D columns where the serial pass takes
+// those of S, so propagators pay while at least 4 chunks fit on the GPU at once (D <= 256
+// at the level counts here).  Beyond that the boundary states come from one serial pass
+// each way.
+constexpr int kMinSide = 4;
 constexpr int kMinChunk = 4;      // steps: below this the products outweigh the steps saved
-constexpr size_t kSegBytes = 1ull << 30;
+constexpr size_t kSegBytes = 1ull << 30;      // stage inputs of one round of chunks
+constexpr size_t kDirectBytes = 8ull << 30;   // of a whole solve (real operators, no propagators)
 
 void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   Setup& s = sv.s;
@@ -1948,13 +1992,19 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   const int N = s.N;
   c.L = N;
   const long long simg = onchip_state_elems(sv.oc);
-  const size_t stage = (size_t)onchip_stage_elems(sv.oc) * (sv.mixed ? sizeof(float2) : sizeof(double2));
+  const size_t cs = sv.mixed ? sizeof(float2) : sizeof(double2);
+  const bool real = grad && onchip_real_adjoint(sv.oc);
+  // bytes of a stage's kept inputs (real operators: of the states and of the co-states)
+  const size_t stage = real ? 2 * simg * cs : (size_t)onchip_stage_elems(sv.oc) * cs;
   const int ncta = onchip_ctas(sv.oc);
   // gradient chunks that run at once
-  const int slots = grad ? std::max(1, 152 * onchip_adj_resident(sv.oc) / ncta) : 1;
-  const size_t accb = (size_t)ncta * onchip_acc_doubles(sv.oc) * sizeof(double);
+  const int slots = !grad ? 1
+                          : std::max(1, real ? 152 * onchip_fwd_resident(sv.oc) / onchip_fwd_ctas(sv.oc)
+                                             : 152 * onchip_adj_resident(sv.oc) / ncta);
+  const size_t accd = onchip_acc_doubles(sv.oc) * sizeof(double);
   auto bytes = [&](int C, int L, int R, size_t nprop) {
-    return 2 * (size_t)C * simg * sizeof(double2) + (size_t)R * L * 4 * stage + (size_t)R * accb +
+    return 2 * (size_t)C * simg * sizeof(double2) + (size_t)R * L * 4 * stage +
+           (real ? (size_t)ocr_blocks(onchip_real_plan(sv.oc)) : (size_t)R * ncta) * accd +
            (size_t)C * nprop * sizeof(double2);
   };
   auto fit_rounds = [&](int C, int L) {                 // chunks per launch within the segment store
@@ -1966,10 +2016,10 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   if (s.D <= 256 && N >= 2 * kMinChunk) {
     KPlan pd = s.p;
     pd.S = (int)s.D;
-    sv.ocp = onchip_plan_create(pd, sv.mixed, s.K, s.sumd, sv.ar.st, false, true);
-    const int nD = sv.ocp && onchip_forward_ok(sv.ocp) ? onchip_ctas(sv.ocp) : 0;
+    sv.ocp = onchip_plan_create(pd, sv.mixed, s.K, s.sumd, sv.ar.st, sv.real_oc ? &sv.rterms : nullptr, false, true);
+    const int nD = sv.ocp && onchip_forward_ok(sv.ocp) ? onchip_fwd_ctas(sv.ocp) : 0;
     const int most = nD ? 152 * onchip_fwd_resident(sv.ocp) / nD : 0;
-    if (nD && nD <= kPropCtas && most >= 4) {
+    if (most >= kMinSide) {
       c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + most - 1) / most);
       c.C = (N + c.L - 1) / c.L;
       c.prop = c.par = c.C > 1;
@@ -1989,6 +2039,11 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     }
   }
   if (!grad) return;
+  // real operators: the two serial passes keep all stage inputs when there is room
+  if (real && ckpt <= 0 && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
+    c.direct = true;
+    return;
+  }
   // boundary states by serial passes; segments of L steps
   if (slots > 1 && N > kMinChunk) {
     if (ckpt > 0) {
@@ -2015,6 +2070,11 @@ sg_status alloc_chunks(sg_ctx* ctx, Solve& sv, int ckpt) {
   plan_chunks(sv, true, ckpt, ctx->work_limit);
   sv.ch.ck = sv.ar.get<double2>((size_t)sv.ch.C * onchip_state_elems(sv.oc));
   if (!sv.ch.ck) return sg_fail(ctx, SG_E_NOMEM, "device allocation of checkpoints failed");
+  if (sv.ch.direct) {
+    const size_t n = (size_t)4 * sv.s.N * onchip_state_elems(sv.oc);
+    sv.ch.segU = sv.mixed ? (void*)sv.ar.get<float2>(n) : (void*)sv.ar.get<double2>(n);
+    if (!sv.ch.segU) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the stage inputs failed");
+  }
   return SG_OK;
 }
 
@@ -2048,6 +2108,17 @@ void chunk_products(Solve& sv, const double2* start, double2* states, double2* l
 
 // sv.psi evolved in place; with sv.ch.ck, the states before every chunk kept.
 template <typename R>
+OnchipRealTables real_tables(const Solve& sv) {
+  OnchipRealTables r;
+  r.coef = sizeof(R) == 4 ? (const void*)sv.coef32 : (const void*)sv.coef;
+  r.ph = sizeof(R) == 4 ? (const void*)sv.ph32 : (const void*)sv.ph;
+  r.opd = sv.opd_dev;
+  r.J = sv.J_dev;
+  r.half = sv.half;
+  return r;
+}
+
+template <typename R>
 sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
   sg_ctx* ctx = sys->ctx;
   cudaStream_t st = ctx->stream;
@@ -2055,9 +2126,11 @@ sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
   OcChunks& c = sv.ch;
   OnchipForward f;
   f.tab = sizeof(R) == 4 ? (const void*)sv.tab32 : (const void*)sv.tab;
+  f.rt = real_tables<R>(sv);
   if (!c.prop) {
     f.psi_api = f.psi_out = sv.psi;
-    f.ck_out = c.ck;
+    f.ck_out = c.direct ? nullptr : c.ck;
+    f.segY = c.segU;
     f.K = c.L;
     sv.launches += onchip_forward(sv.oc, f, 0, s.N, s.N, s.dt, st);
     SG_CUDA_TRY(ctx, cudaGetLastError());
@@ -2171,6 +2244,90 @@ XArgs make_xargs(const Solve& sv, GradAcc acc) {
   return xa;
 }
 
+// dF/d(pulse parameters) and dF/d(carriers) from dF/df at every stage.  A slot costs FP64 sines
+// and cosines (about 100 multiply-adds at 2 per clock and SM), so the slots are spread over
+// the SMs and their shares summed in block order: 0.90 ms in one block per drive (10,000
+// steps, one drive), 0.02 ms over 152.
+sg_status launch_pulse_chain(Solve& sv, const double* gF, int np_max, const int* poff, double* gpulse,
+                             double* omega_bar, int nsub) {
+  const Setup& s = sv.s;
+  cudaStream_t st = sv.ar.st;
+  const int threads = 64, stride = np_max + 1;
+  const long long slots = (long long)(nsub > 0 ? nsub : 3) * s.N;
+  const int nblk = (int)std::max<long long>(1, std::min<long long>((slots + 2 * threads - 1) / (2 * threads),
+                                                                   std::max(1, 304 / s.K)));
+  double* part = sv.ar.get<double>((size_t)s.K * nblk * stride);
+  if (!part) return SG_E_NOMEM;
+  k_pulse_chain<<<dim3(s.K, nblk), threads, threads * stride * sizeof(double), st>>>(
+      sv.drives_dev, sv.amps_dev, gF, s.K, s.N, s.dt, nsub, part, stride);
+  k_pulse_sum<<<s.K, 32, 0, st>>>(sv.drives_dev, part, stride, nblk, poff, s.n_pulse, gpulse, omega_bar);
+  sv.launches += 1;
+  return SG_OK;
+}
+
+// Gradient on the real-operator kernels: per round of R chunks the states are recomputed and
+// the co-states pulled back, each keeping its stage inputs, and one launch contracts them
+// (ocr_densities); a direct solve's serial passes kept them already.
+template <typename R>
+sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc acc) {
+  typedef typename CT<R>::T C;
+  sg_ctx* ctx = sys->ctx;
+  cudaStream_t st = ctx->stream;
+  Setup& s = sv.s;
+  OcChunks& c = sv.ch;
+  const OnchipPlan* oc = sv.oc;
+  const OcrPlan* rp = onchip_real_plan(oc);
+  const long long ns = onchip_state_elems(oc);
+  const long long nst = 3ll * s.N, nstK = nst * std::max(1, s.K);
+  const int groups = ocr_groups(rp), blocks = ocr_blocks(rp);
+  const size_t naccd = (size_t)blocks * onchip_acc_doubles(oc), nseg = (size_t)4 * c.R * c.L * ns;
+  double2* pimg = sv.ar.get<double2>(ns);
+  C* segU = c.direct ? static_cast<C*>(c.segU) : sv.ar.get<C>(nseg);
+  C* segK = sv.ar.get<C>(nseg);
+  double* gFc = sv.ar.get<double>((size_t)groups * nstK);
+  double* accc = sv.ar.get<double>(naccd);
+  c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
+  double2* gimg = c.prop ? sv.ar.get<double2>((size_t)c.NG * ns) : pimg;
+  if (!pimg || !segU || !segK || !gFc || !accc || !c.lam || !gimg)
+    return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
+  SG_CUDA_TRY(ctx, cudaMemsetAsync(gFc, 0, (size_t)groups * nstK * sizeof(double), st));
+  SG_CUDA_TRY(ctx, cudaMemsetAsync(accc, 0, naccd * sizeof(double), st));
+  onchip_to_image(oc, pbar, pimg, st);
+  ++sv.launches;
+  OnchipForward f;
+  f.rt = real_tables<R>(sv);
+  OnchipForward b = f;
+  b.rev = true;
+  if (c.prop) {
+    chunk_products(sv, pimg, c.lam, nullptr, gimg, true, st);
+  } else if (c.par) {
+    b.img_in = pimg;
+    b.ck_out = c.lam;
+    b.K = c.L;
+    sv.launches += onchip_forward(oc, b, 0, s.N, s.N, s.dt, st);
+    b.ck_out = nullptr;
+  }
+  for (int c1 = c.C; c1 > 0; c1 -= c.R) {
+    const int c0 = std::max(0, c1 - c.R), n0 = c0 * c.L, n1 = std::min(s.N, c1 * c.L);
+    if (!c.direct) {
+      f.img_in = c.ck + (size_t)c0 * ns;
+      f.segY = segU;
+      sv.launches += onchip_forward(oc, f, n0, n1, c.L, s.dt, st);
+    }
+    b.img_in = c.par ? c.lam + (size_t)c0 * ns : pimg;
+    b.img_out = c.par ? nullptr : pimg;                 // one after the other: handed on
+    b.segY = segK;
+    sv.launches += onchip_forward(oc, b, n0, n1, c.L, s.dt, st);
+    if (c0 == 0) onchip_batcher_release();              // the solve's last on-chip launch is issued
+    sv.launches += ocr_densities(rp, segU, segK, f.rt.coef, sv.opd_dev, sv.J_dev, n0, n1, s.dt, sv.want_ham, nstK, gFc,
+                                 accc, st);
+  }
+  onchip_reduce(oc, gFc, groups, accc, blocks, nst, s.K, s.p.n1, s.p.ne, acc, st);
+  ++sv.launches;
+  SG_CUDA_TRY(ctx, cudaGetLastError());
+  return SG_OK;
+}
+
 // Adjoint on the on-chip kernels: the co-states after every chunk (products with the chunk
 // propagators' adjoints, or one serial pull-back), then per launch pair R chunks: a recompute
 // that stores every stage input, and the pull-back with its cross-densities; the
@@ -2223,6 +2380,7 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc 
   } else if (c.par) {
     OnchipForward b;
     b.tab = atab;
+    b.rt = real_tables<R>(sv);
     b.img_in = pimg;
     b.rev = true;
     b.ck_out = c.lam;
@@ -2235,12 +2393,13 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc 
     f.tab = tab;
     f.img_in = c.ck + (size_t)c0 * ns;
     f.segY = segY;
+    f.rows = true;
     sv.launches += onchip_forward(oc, f, n0, n1, c.L, s.dt, st);
     sv.launches += onchip_adjoint(oc, tb, segY, c.par ? c.lam + (size_t)c0 * ns : pimg, n0, n1, c.L, s.dt, xa,
                                   (int)nst, gFc, accc, err, colow, st);
   }
   onchip_batcher_release();                       // the solve's last on-chip launch is issued
-  onchip_reduce(oc, gFc, accc, c.R * ncta, nst, s.K, s.p.n1, s.p.ne, acc, st);
+  onchip_reduce(oc, gFc, ncta, accc, c.R * ncta, nst, s.K, s.p.n1, s.p.ne, acc, st);
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
   int herr = 0;
@@ -2259,7 +2418,8 @@ sg_status run_backward(sg_system* sys, Solve& sv, std::vector<double2*>& ckpts, 
   cudaStream_t st = ctx->stream;
   Setup& s = sv.s;
   const long long n = s.D * s.S;
-  if (sv.onchip(true)) return run_backward_onchip<R>(sys, sv, pbar, acc);
+  if (sv.onchip(true))
+    return onchip_real_adjoint(sv.oc) ? run_backward_real<R>(sys, sv, pbar, acc) : run_backward_onchip<R>(sys, sv, pbar, acc);
   const bool slab = sv.slab != nullptr;
   // buffers of the gather path only (the slab path keeps a segment store instead)
   C* X = slab ? nullptr : sv.ar.get<C>(n);
@@ -2403,18 +2563,18 @@ size_t sg_chunk_bytes(const sg_system* sys, const sg_evolve_opts* o, bool grad) 
   const int d = sys->modes[0].d;
   const double N = o->T / o->dt, S = o->ncols, cs = o->precision == SG_MIXED ? 8 : 16;
   const double image = D * (S + 16) * sizeof(double2);
-  const double seg = grad ? 4 * N * D * (S + 16) * 1.13 * cs : 0.0;      // every stage input
+  const double seg = grad ? 8 * N * D * (S + 16) * cs : 0.0;             // every stage input, states and co-states
   double b = 0.0, C = 0.0;
   if (D <= 256) {
-    C = std::min(N / kMinChunk + 1, 152.0 * 32 / std::max(1.0, D * D / (d * d) / 256));
+    C = std::min(N / kMinChunk + 1, 152.0 * 32 / std::max(1.0, D * D / (d * d) / 32));
     b += C * D * (D + 32) * 2 * sizeof(double2);
   }
   if (grad) {
     const double waves = 1 + seg / kSegBytes;
     C = std::max(C, std::min(N / kMinChunk + 1, 152.0 * 8 * waves / std::max(1.0, S * D / (d * d) / 256)));
-    const double blocks = 152.0 * 32 * std::max(1.0, S * D / (d * d) / 128);
+    const double blocks = 152.0 * 32 * std::max(1.0, S * D / (d * d) / 128);      // accumulators
     const double acc = 8.0 * (130.0 * sys->drives.size() + 290.0 * sys->couplings.size() + 10.0 * sys->modes.size());
-    b += 2 * C * image + std::min(seg, 1.5 * (double)kSegBytes) + std::min(N, blocks) * acc;
+    b += 2 * C * image + std::min(seg, seg <= (double)kDirectBytes && D > 256 ? (double)kDirectBytes : 1.5 * (double)kSegBytes) + std::min(N, blocks) * acc;
   }
   return (size_t)(1.25 * b) + (32u << 20);
 }
@@ -2519,7 +2679,7 @@ sg_status run_backward_q2(sg_system* sys, Solve& sv, double2* pbar, GradAcc acc)
   if (rc != SG_OK)
     return sg_fail(ctx, rc, "the Q2 gradient needs 2..16 modes, <= 32 couplings, <= 16 drives and its buffers "
                             "in shared memory");
-  onchip_reduce(sv.oc, gFc, nullptr, 0, nst, s.K, s.p.n1, s.p.ne, acc, st);
+  onchip_reduce(sv.oc, gFc, ncta, nullptr, 0, nst, s.K, s.p.n1, s.p.ne, acc, st);
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
   return SG_OK;
@@ -2829,9 +2989,8 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
     if (s.K) {
       int np_max = 1;
       for (auto& d : s.drives) np_max = std::max(np_max, d.kind == SG_ENV_PWC ? d.nseg : 1);
-      const int pt = 64;
-      k_pulse_chain<<<s.K, pt, pt * (np_max + 1) * sizeof(double), st>>>(
-          sv.drives_dev, sv.amps_dev, acc.gF, s.K, s.N, s.dt, poff, s.n_pulse, gpulse, omega_bar, s.q2 ? s.ta.nsub : 0);
+      rc = launch_pulse_chain(sv, acc.gF, np_max, poff, gpulse, omega_bar, s.q2 ? s.ta.nsub : 0);
+    if (rc != SG_OK) return rc;
     } else {
       SG_CUDA_TRY(ctx, cudaMemsetAsync(omega_bar, 0, sizeof(double), st));
     }
@@ -3073,9 +3232,8 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
   if (s.K) {
     int np_max = 1;
     for (auto& d : s.drives) np_max = std::max(np_max, d.kind == SG_ENV_PWC ? d.nseg : 1);
-    const int pt = 64;
-    k_pulse_chain<<<s.K, pt, pt * (np_max + 1) * sizeof(double), st>>>(
-        sv.drives_dev, sv.amps_dev, acc.gF, s.K, s.N, s.dt, poff, s.n_pulse, gpulse, omega_bar, 0);
+    rc = launch_pulse_chain(sv, acc.gF, np_max, poff, gpulse, omega_bar, 0);
+    if (rc != SG_OK) return done(rc);
     ++sv.launches;
   }
   double* gdev = nullptr;

@@ -31,6 +31,8 @@
 #include "slab.h"
 #include "slab_dev.cuh"
 #include "onchip.h"
+#include "onchip_dev.cuh"
+#include "onchip_real.h"
 #include <condition_variable>
 #include <cstring>
 #include <mutex>
@@ -40,120 +42,6 @@
 #include <cstdlib>
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// asynchronous copies and barriers
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-// cp.async of 4, 8 or 16 bytes global -> shared (no registers, completes at cp_wait_all)
-__device__ __forceinline__ void cp4(void* s, const void* g) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp8(void* s, const void* g) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp16(void* s, const void* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-__device__ __forceinline__ void cpv(float2* s, const float2* g) { cp8(s, g); }
-__device__ __forceinline__ void cpv(double2* s, const double2* g) { cp16(s, g); }
-__device__ __forceinline__ void cpv(float* s, const float* g) { cp4(s, g); }
-__device__ __forceinline__ void cpv(double* s, const double* g) { cp8(s, g); }
-
-__device__ __forceinline__ void mb_init(uint64_t* mb) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mb)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-// One bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) into
-// shared memory, completing a phase of mb.  Issued by one thread.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* mb) {
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(mb)), "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(mb))
-      : "memory");
-}
-__device__ __forceinline__ bool mb_try(uint64_t* mb, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(mb)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait for the phase `parity` of mb: true once the phase has completed,
-// false after `limit` polls (about a second at the default limit).
-__device__ __forceinline__ bool mb_wait_for(uint64_t* mb, unsigned parity, int limit) {
-  for (int it = 0; it < limit; ++it) {
-    if (mb_try(mb, parity)) return true;
-    __nanosleep(64);
-  }
-  return false;
-}
-// Barrier among the first n threads of the CTA (n a multiple of 32); id 0 is __syncthreads.
-__device__ __forceinline__ void bar_sub(int id, int n) {
-  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
-}
-
-// ---------------------------------------------------------------------------
-// state: complex128, or float-float pairs in mixed precision
-// ---------------------------------------------------------------------------
-// hi + lo <- hi + lo + x with hi = fl(hi + lo) afterwards (TwoSum, then a fast
-// renormalisation); exact up to the rounding of the low word.
-__device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float bb = s - hi;
-  const float e = (hi - (s - bb)) + (x - bb);
-  const float l = lo + e;
-  const float h2 = s + l;
-  lo = l - (h2 - s);
-  hi = h2;
-}
-
-template <typename R> struct StateArr;
-template <> struct StateArr<double> {
-  double2* p;
-  __device__ void init(unsigned char* base, int n) { p = reinterpret_cast<double2*>(base); (void)n; }
-  __device__ void set(int e, double2 v) { p[e] = v; }
-  __device__ double2 get(int e) const { return p[e]; }
-  __device__ double2 hi(int e) const { return p[e]; }
-  __device__ void add(int e, double2 x) { p[e] = make_double2(p[e].x + x.x, p[e].y + x.y); }
-};
-template <> struct StateArr<float> {
-  float2 *h, *l;
-  __device__ void init(unsigned char* base, int n) {
-    h = reinterpret_cast<float2*>(base);
-    l = h + n;
-  }
-  // high words in shared memory, low words elsewhere (global memory when shared
-  // memory is short: they are touched once per step)
-  __device__ void init_split(unsigned char* base, float2* lo) {
-    h = reinterpret_cast<float2*>(base);
-    l = lo;
-  }
-  __device__ void set(int e, double2 v) {
-    const float hx = __double2float_rn(v.x), hy = __double2float_rn(v.y);
-    h[e] = make_float2(hx, hy);
-    l[e] = make_float2(__double2float_rn(v.x - (double)hx), __double2float_rn(v.y - (double)hy));
-  }
-  __device__ double2 get(int e) const {
-    return make_double2((double)h[e].x + (double)l[e].x, (double)h[e].y + (double)l[e].y);
-  }
-  __device__ float2 hi(int e) const { return h[e]; }
-  __device__ void add(int e, float2 x) {
-    float2 a = h[e], b = l[e];
-    ff_add(a.x, b.x, x.x);
-    ff_add(a.y, b.y, x.y);
-    h[e] = a;
-    l[e] = b;
-  }
-};
 
 // ---------------------------------------------------------------------------
 // plan arguments
@@ -181,51 +69,6 @@ struct OcArgs {
   int wlim, skip_first;
 };
 
-// One solve of a launch: its tables, buffers and chunks of steps.  A solve has C chunks
-// of L steps, chunk c covering steps [n0 + c L, min(n1, n0 + (c + 1) L)), and every chunk
-// has the plan's ncta CTAs; the CTAs of solve b of a launch start at cta0[b].
-struct OcSys {
-  const void* tab;
-  const void* atab;      // adjoint: rows the co-state is pulled back with (tab: the forward
-                         // rows, which the cross-densities contract)
-  const void* coef;
-  const void* ph;
-  const void* opd;
-  const double2* psi_api;
-  const double2* img_in; // start images, one per chunk
-  double2* img_out;      // forward: the chunks' final images
-  double2* psi_out;
-  double2* ck_out;
-  void* segY;
-  double2* pbar_img;     // adjoint: the co-states at the chunks' ends, one image per chunk
-  double* gF_cta;
-  double* acc_cta;
-  int* err;
-  void* pblo;
-  const double* J;       // coupling strengths of the solve (Hamiltonian-gradient contraction)
-  long long nstK;
-  int n0, n1, K;
-  int C, L;
-  int ident;             // forward: column j starts in basis state j (a chunk's propagator)
-  int rev;               // forward: the steps backwards (the co-state's pull-back, see k_oc_fwd)
-};
-constexpr int kOcMaxBatch = 24;
-struct OcBatch {
-  int nsys;
-  int cta0[kOcMaxBatch];
-  OcSys s[kOcMaxBatch];
-};
-
-// The solve, chunk and CTA within the chunk that this block works on.
-__device__ __forceinline__ const OcSys& oc_locate(const OcBatch& bt, int ncta, int& chunk, int& cta) {
-  int b = 0;
-  while (b + 1 < bt.nsys && (int)blockIdx.x >= bt.cta0[b + 1]) ++b;
-  const int rel = blockIdx.x - bt.cta0[b];
-  chunk = rel / ncta;
-  cta = rel - chunk * ncta;
-  return bt.s[b];
-}
-
 template <int DL>
 __device__ __forceinline__ int oc_pos(const OcArgs& oa, int e) {
   const int c = e / oa.D;
@@ -251,14 +94,6 @@ __device__ __forceinline__ void oc_apply(const SlabPass& sp, const OcArgs& oa, c
     else bar_sub(bar, nthr);
   }
 }
-
-template <typename V>
-__device__ __forceinline__ void issue_rows(const V* __restrict__ tab, int row, int q, V* dst, int tid, int nthr) {
-  const V* src = tab + (size_t)q * row;
-  for (int i = tid; i < row; i += nthr) cpv(dst + i, src + i);
-}
-
-__host__ __device__ __forceinline__ int stage_row(int s) { return s == 0 ? 0 : (s == 3 ? 2 : 1); }
 
 // ---------------------------------------------------------------------------
 // forward
@@ -379,16 +214,6 @@ __device__ __forceinline__ C shfl_xor_c(C v, int o) {
   v.y = __shfl_xor_sync(0xffffffffu, v.y, o);
   return v;
 }
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-template <typename C> __device__ __forceinline__ C cmulT(C a, C b) {
-  return cmk<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-template <typename C> __device__ __forceinline__ C cconjT(C a) { return cmk<C>(a.x, -a.y); }
-
 // Shared-memory accumulators of one CTA and segment (level-pair stride DL * DL, level stride DL).
 template <typename T>
 struct OcAcc {
@@ -1015,17 +840,15 @@ __device__ __forceinline__ double2 chain_fma(double2 u, double2 x, double2 v) {
 // propagators of group g's chunks in order, or (ADJ) through their adjoints in reverse
 // order.  A matrix times one column has D^2 complex multiply-adds against D^2 entries
 // read once from L2, and the next one waits for its result, so a chunk costs a load round
-// trip plus two barriers: the D rows get `parts` threads each, with independent loads, and the
-// two-level order of the callers keeps the chain short.  ADJ reads the same column-major
-// image along its columns (a warp per output, lanes along the column), forward across
-// them, so both are coalesced.  Measured with the whole solve: the D = 16 pair's 10,000 FP64
-// steps go from 546 ms in one serial CTA to 1.40 ms (chunks 0.9 ms, products 0.1 ms), the
-// D = 25 gradient (10,000 mixed steps) from 254 to 4.6 ms.
+// trip plus two barriers: the D rows get `parts` threads each with at most E entries, which
+// are loaded while the previous chunk is multiplied (E = 0: too many to hold, loaded in
+// place), and the two-level order of the callers keeps the chain short.  ADJ walks down a column per
+// thread: not coalesced, but every sector is used up by its thread's next entries.
 struct OcChainArgs {
   OnchipChain a;
   int ncols, rows, parts;
 };
-template <bool ADJ>
+template <bool ADJ, int E>
 __global__ void k_oc_chain(const __grid_constant__ OcChainArgs k) {
   extern __shared__ __align__(16) unsigned char sm[];
   const OnchipChain& a = k.a;
@@ -1040,49 +863,54 @@ __global__ void k_oc_chain(const __grid_constant__ OcChainArgs k) {
     x[t] = v;
   }
   __syncthreads();
-  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = threadIdx.x / k.rows, t = threadIdx.x - p * k.rows;
+  const bool on = p < k.parts && t < D;
+  constexpr int N = E ? E : 1;
+  double2 u[N];
+  auto fetch = [&](int c) {
+    const double2* __restrict__ U = a.U + (size_t)c * a.u_stride;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int j = p + e * k.parts;
+      if (on && j < D) u[e] = ADJ ? U[(size_t)t * D + j] : U[(size_t)j * D + t];
+    }
+  };
+  if (E && c0 < c1) fetch(ADJ ? c1 - 1 : c0);
   for (int i = c0; i < c1; ++i) {
     const int c = ADJ ? c1 - 1 - (i - c0) : i;
-    const double2* __restrict__ U = a.U + (size_t)c * a.u_stride;
     if (a.states)
-      for (int t = threadIdx.x; t < D; t += blockDim.x) a.states[(size_t)c * a.state_stride + (size_t)s * D + t] = x[t];
-    if (ADJ) {
-      for (int j = warp; j < D; j += nw) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int t = lane; t < D; t += 32) v = chain_fma(cconj(U[(size_t)j * D + t]), x[t], v);
-        double re = v.x, im = v.y;
-        for (int o = 16; o > 0; o >>= 1) {
-          re += __shfl_xor_sync(0xffffffffu, re, o);
-          im += __shfl_xor_sync(0xffffffffu, im, o);
-        }
-        if (lane == 0) part[j] = make_double2(re, im);
+      for (int r = threadIdx.x; r < D; r += blockDim.x) a.states[(size_t)c * a.state_stride + (size_t)s * D + r] = x[r];
+    double2 v = make_double2(0.0, 0.0);
+    if (E) {
+      double2 m[N];
+#pragma unroll
+      for (int e = 0; e < N; ++e) m[e] = u[e];
+      if (i + 1 < c1) fetch(ADJ ? c - 1 : c + 1);
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        const int j = p + e * k.parts;
+        if (on && j < D) v = chain_fma(ADJ ? cconj(m[e]) : m[e], x[j], v);
       }
-      __syncthreads();
-      for (int t = threadIdx.x; t < D; t += blockDim.x) x[t] = part[t];
-    } else {
-      const int p = threadIdx.x / k.rows;
-      if (p < k.parts) {
-        for (int t = threadIdx.x - p * k.rows; t < D; t += k.rows) {
-          double2 v = make_double2(0.0, 0.0);
+    } else if (on) {
+      const double2* __restrict__ U = a.U + (size_t)c * a.u_stride;
 #pragma unroll 4
-          for (int j = p; j < D; j += k.parts) v = chain_fma(U[(size_t)j * D + t], x[j], v);
-          part[p * k.rows + t] = v;
-        }
+      for (int j = p; j < D; j += k.parts)
+        v = chain_fma(ADJ ? cconj(U[(size_t)t * D + j]) : U[(size_t)j * D + t], x[j], v);
+    }
+    if (on) part[p * k.rows + t] = v;
+    __syncthreads();
+    for (int r = threadIdx.x; r < D; r += blockDim.x) {
+      double2 w = part[r];
+      for (int q = 1; q < k.parts; ++q) {
+        w.x += part[q * k.rows + r].x;
+        w.y += part[q * k.rows + r].y;
       }
-      __syncthreads();
-      for (int t = threadIdx.x; t < D; t += blockDim.x) {
-        double2 v = part[t];
-        for (int q = 1; q < k.parts; ++q) {
-          v.x += part[q * k.rows + t].x;
-          v.y += part[q * k.rows + t].y;
-        }
-        x[t] = v;
-      }
+      x[r] = w;
     }
     __syncthreads();
   }
   if (a.last)
-    for (int t = threadIdx.x; t < D; t += blockDim.x) a.last[(size_t)g * a.last_stride + (size_t)s * D + t] = x[t];
+    for (int r = threadIdx.x; r < D; r += blockDim.x) a.last[(size_t)g * a.last_stride + (size_t)s * D + r] = x[r];
 }
 
 // Fixed-order sum over CTAs of the per-CTA gradient blocks.
@@ -1131,6 +959,7 @@ int grid_of(long long n) { return (int)std::max<long long>(1, std::min<long long
 // ---------------------------------------------------------------------------
 struct OnchipPlan {
   SlabPlanHost* h = nullptr;
+  OcrPlan* real = nullptr;        // the real-operator forward kernels, where they apply
   OcArgs oa{};
   bool mixed = false, adj_ok = false, fwd_ok = false;
   size_t sm_fwd = 0, sm_adj = 0, limit = 0;
@@ -1219,8 +1048,8 @@ std::vector<long long> plan_signature(const KPlan& p, bool mixed, int K, int sum
 }
 }  // namespace
 
-OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st, bool two_rows,
-                               bool fwd_only) {
+OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st, const OcrTerms* rt,
+                               bool two_rows, bool fwd_only) {
   if (p.nq < 2 || p.nq > SG_MAXQ) return nullptr;
   SlabPlanHost* h = slab_plan_create(p, mixed, st, true);
   if (!h) return nullptr;
@@ -1308,6 +1137,11 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
     if (const char* e = std::getenv("SG_OC_PW")) a.npw = std::max(1, std::min(nw - 1, atoi(e)));
   }
   const long long MD2 = SG_MAXD * SG_MAXD;
+  // SG_TEST_SKIP_BULK tests the bounded wait of the complex-row adjoint, so it keeps those kernels
+  const char* knob = std::getenv("SG_TEST_SKIP_BULK");
+  if (rt && !(knob && knob[0] == '1')) oc->real = ocr_plan_create(p, mixed, *rt, a.ncta * a.Sc);
+  oc->sig.push_back(oc->real != nullptr);
+  if (oc->real) ocr_signature(oc->real, oc->sig);
   a.accd = 2 * (long long)K * MD2 + 4 * (long long)p.ne * MD2 + (long long)p.n1 * SG_MAXD +
            2 * (long long)p.ne * SG_MAXD + p.ne;
   return oc;
@@ -1316,6 +1150,7 @@ OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cuda
 void onchip_plan_destroy(OnchipPlan* oc) {
   if (!oc) return;
   slab_plan_destroy(oc->h);
+  ocr_plan_destroy(oc->real);
   delete oc;
 }
 
@@ -1425,7 +1260,7 @@ int adj_t(const OnchipPlan* oc, OcBatch& bt, double dt, const XArgs& xa, cudaStr
 namespace {
 
 struct OcPending {
-  int kind;                     // 0 forward, 1 adjoint
+  int kind;                     // 0 forward, 1 adjoint, 2 forward with real operators
   const OnchipPlan* oc;
   OcSys d;
   double dt;
@@ -1448,6 +1283,7 @@ bool oc_compatible(const OcPending& a, const OcPending& b) {
 
 template <typename R, int DL>
 int launch_t(const OnchipPlan* oc, int kind, OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
+  if (kind == 2) return ocr_forward(oc->real, bt, dt, st);
   return kind == 0 ? fwd_t<R, DL>(oc, bt, dt, st) : adj_t<R, DL>(oc, bt, dt, *xa, st);
 }
 int oc_launch(const OnchipPlan* oc, int kind, OcBatch& bt, double dt, const XArgs* xa, cudaStream_t st) {
@@ -1567,7 +1403,7 @@ int submit(const OcPending& p, cudaStream_t st) {
   OcBatch bt{};
   bt.nsys = 1;
   bt.s[0] = p.d;
-  bt.s[0].J = nullptr;               // the launch's own XArgs hold this solve's couplings
+  if (p.kind == 1) bt.s[0].J = nullptr;   // the launch's own XArgs hold this solve's couplings
   return oc_launch(p.oc, p.kind, bt, p.dt, p.xa, st);
 }
 
@@ -1575,10 +1411,15 @@ int submit(const OcPending& p, cudaStream_t st) {
 
 int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st) {
   OcPending p{};
-  p.kind = 0;
+  p.kind = oc->real && !f.rows ? 2 : 0;
   p.oc = oc;
   p.dt = dt;
   p.d.tab = f.tab;
+  p.d.coef = f.rt.coef;
+  p.d.ph = f.rt.ph;
+  p.d.opd64 = f.rt.opd;
+  p.d.J = f.rt.J;
+  p.d.half = f.rt.half;
   p.d.psi_api = f.psi_api;
   p.d.img_in = f.img_in;
   p.d.img_out = f.img_out;
@@ -1635,7 +1476,17 @@ int adj_resident_t(const OnchipPlan* oc) {
 
 }  // namespace
 
-int onchip_fwd_resident(const OnchipPlan* oc) { OC_DISPATCH(fwd_resident_t, oc); }
+int onchip_fwd_resident(const OnchipPlan* oc) {
+  if (oc->real) return ocr_resident(oc->real);
+  OC_DISPATCH(fwd_resident_t, oc);
+}
+int onchip_fwd_ctas(const OnchipPlan* oc) { return oc->real ? ocr_ctas(oc->real) : oc->oa.ncta; }
+bool onchip_real(const OnchipPlan* oc) { return oc->real != nullptr; }
+bool onchip_real_adjoint(const OnchipPlan* oc) { return oc->real && ocr_adjoint_ok(oc->real); }
+const OcrPlan* onchip_real_plan(const OnchipPlan* oc) { return oc->real; }
+void onchip_half_step(const OnchipPlan* oc, const double* E, double dt, void* q, cudaStream_t st) {
+  ocr_half_step(oc->real, E, dt, q, st);
+}
 int onchip_adj_resident(const OnchipPlan* oc) { OC_DISPATCH(adj_resident_t, oc); }
 
 namespace {
@@ -1800,15 +1651,17 @@ int onchip_chain(const OnchipChain& a, int ncols, int ngroups, cudaStream_t st) 
   k.ncols = ncols;
   const int D = a.D;
   // threads: D rows (padded to whole warps) times parts of the sum
-  int rows = (D + 31) / 32 * 32;
-  if (D <= 16) rows = 16;
+  const int rows = D <= 16 ? 16 : (D + 31) / 32 * 32;
   k.rows = rows;
-  k.parts = std::max(1, std::min(256 / rows, (D + 3) / 4));
+  k.parts = std::max(1, std::min((D > 64 ? 768 : 512) / rows, (D + 3) / 4));
   const int threads = (rows * k.parts + 31) / 32 * 32;
+  const int each = (D + k.parts - 1) / k.parts;
   const size_t smem = (size_t)(D + rows * k.parts) * sizeof(double2);
   const dim3 grid(ncols, ngroups);
-  if (a.adjoint) k_oc_chain<true><<<grid, threads, smem, st>>>(k);
-  else k_oc_chain<false><<<grid, threads, smem, st>>>(k);
+  auto run = [&](auto kern) { kern<<<grid, threads, smem, st>>>(k); };
+  if (each <= 4) a.adjoint ? run(k_oc_chain<true, 4>) : run(k_oc_chain<false, 4>);
+  else if (each <= 8) a.adjoint ? run(k_oc_chain<true, 8>) : run(k_oc_chain<false, 8>);
+  else a.adjoint ? run(k_oc_chain<true, 0>) : run(k_oc_chain<false, 0>);
   return 1;
 }
 
@@ -1816,12 +1669,12 @@ void onchip_to_f32(const double* src, float* dst, long long n, cudaStream_t st) 
   k_oc_f32<<<grid_of(n), 256, 0, st>>>(src, dst, n);
 }
 
-void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, int nblk, long long nst, int K,
-                   int n1, int ne, GradAcc acc, cudaStream_t st) {
+void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, int ngF, const double* acc_cta, int nblk, long long nst,
+                   int K, int n1, int ne, GradAcc acc, cudaStream_t st) {
   RedArgs r{};
   r.nstK = nst * std::max(1, K);
   r.accd = acc_cta ? oc->oa.accd : 0;   // no per-CTA accumulator blocks: dF/df only
-  r.ncta = oc->oa.ncta;
+  r.ncta = ngF;
   r.nacc = nblk;
   r.K = K;
   r.n1 = n1;

@@ -10,6 +10,7 @@
 // accumulators that one reduction sums in a fixed order.
 #pragma once
 #include "grad.cuh"
+#include "onchip_real.h"
 
 struct OnchipPlan;   // opaque
 
@@ -19,8 +20,14 @@ struct OnchipPlan;   // opaque
 // kernels fit too).  K drives and sumd = sum of level counts size the adjoint's
 // per-stage buffers.  two_rows: the adjoint pulls back with rows of its own (open systems).
 // fwd_only: the columns per CTA are those of the forward kernel (propagators).
-OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st, bool two_rows = false,
-                               bool fwd_only = false);
+// rt (nullable): the terms, when they are real up to the frame phases (interaction frame);
+// the forward evolution then runs on the real-operator kernels where they apply.
+OnchipPlan* onchip_plan_create(const KPlan& p, bool mixed, int K, int sumd, cudaStream_t st,
+                               const OcrTerms* rt = nullptr, bool two_rows = false, bool fwd_only = false);
+bool onchip_real(const OnchipPlan* oc);
+// The gradient runs on the real-operator kernels too (ocr_densities).
+bool onchip_real_adjoint(const OnchipPlan* oc);
+const OcrPlan* onchip_real_plan(const OnchipPlan* oc);
 void onchip_plan_destroy(OnchipPlan* oc);
 // The adjoint kernel fits too (gradient solves may use the on-chip path).
 bool onchip_adjoint_ok(const OnchipPlan* oc);
@@ -41,8 +48,16 @@ long long onchip_acc_doubles(const OnchipPlan* oc);
 // slot 4 (step - n0) + stage).  rev: the steps backwards with their adjoint maps (one
 // chunk pulls a co-state from after step n1-1 to before step n0, and ck_out + c *
 // state_elems is the co-state after the last step of segment c).  Returns launches.
+struct OnchipRealTables {
+  const void* coef = nullptr;     // drive coefficients (3N x K) and frame phases (3N x sumd),
+  const void* ph = nullptr;       // stage precision
+  const double2* opd = nullptr;   // flat truncated operators
+  const double* J = nullptr;      // couplings
+  const void* half = nullptr;     // onchip_half_step
+};
 struct OnchipForward {
   const void* tab = nullptr;
+  OnchipRealTables rt;            // onchip_real plans
   const double2* psi_api = nullptr;
   const double2* img_in = nullptr;
   double2* img_out = nullptr;
@@ -51,11 +66,16 @@ struct OnchipForward {
   int K = 1;
   void* segY = nullptr;
   bool ident = false, rev = false;
+  bool rows = false;              // the complex-row kernels, also where the plan is real
 };
 int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st);
 // CTAs of the forward (adjoint) launch that one SM holds at once.
 int onchip_fwd_resident(const OnchipPlan* oc);
 int onchip_adj_resident(const OnchipPlan* oc);
+// CTAs of one chunk of the forward launch.
+int onchip_fwd_ctas(const OnchipPlan* oc);
+// D entries of the stage precision: exp(-i E dt/2) of every composite level.
+void onchip_half_step(const OnchipPlan* oc, const double* E, double dt, void* q, cudaStream_t st);
 // Columns of a state image, padding included.
 int onchip_columns(const OnchipPlan* oc);
 void onchip_from_image(const OnchipPlan* oc, const double2* img, double2* api, cudaStream_t st);
@@ -105,9 +125,9 @@ bool onchip_forward_ok(const OnchipPlan* oc);
 // Element-wise FP64 -> FP32 copy (tables for the mixed-precision adjoint).
 void onchip_to_f32(const double* src, float* dst, long long n, cudaStream_t st);
 bool onchip_mixed(const OnchipPlan* oc);
-// acc += sums in block order: of gF_cta over the plan's CTAs, of acc_cta over nblk blocks.
-void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, const double* acc_cta, int nblk, long long nst, int K,
-                   int n1, int ne, GradAcc acc, cudaStream_t st);
+// acc += sums in block order: of gF_cta over ngF blocks, of acc_cta over nblk blocks.
+void onchip_reduce(const OnchipPlan* oc, const double* gF_cta, int ngF, const double* acc_cta, int nblk, long long nst,
+                   int K, int n1, int ne, GradAcc acc, cudaStream_t st);
 
 // Suzuki-Trotter evolution (Sec. 2.3, App. A) of N Q2 sub-steps, lab frame, from psi_in
 // to psi_out (API layout, may alias).  rows: (N + 1) x nq x d^2 1-body unitaries of the
