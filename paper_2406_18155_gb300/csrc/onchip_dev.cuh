@@ -28,6 +28,7 @@ struct OcSys {
   const double* J;       // coupling strengths of the solve (device)
   const double2* opd64;  // real-operator kernels: truncated operators, FP64
   const void* half;      // and the frame phases of half a step
+  int phmid;             // ph holds one row a step (its middle) instead of its three stages
   long long nstK;
   int n0, n1, K;
   int C, L;
@@ -39,6 +40,8 @@ struct OcBatch {
   int nsys;
   int cta0[kOcMaxBatch];
   OcSys s[kOcMaxBatch];
+  const OcSys* many;     // more solves than s holds: device array, `per` CTAs each
+  int per;
 };
 
 namespace {
@@ -159,6 +162,12 @@ template <> struct StateArr<float> {
 
 // The solve, chunk and CTA within the chunk that this block works on.
 __device__ __forceinline__ const OcSys& oc_locate(const OcBatch& bt, int ncta, int& chunk, int& cta) {
+  if (bt.many) {
+    const int b = blockIdx.x / bt.per, rel = blockIdx.x - b * bt.per;
+    chunk = rel / ncta;
+    cta = rel - chunk * ncta;
+    return bt.many[b];
+  }
   int b = 0;
   while (b + 1 < bt.nsys && (int)blockIdx.x >= bt.cta0[b + 1]) ++b;
   const int rel = blockIdx.x - bt.cta0[b];

@@ -175,8 +175,8 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
   const int CS = (pad(a.D - 1) + 2) / 2 * 2;
   a.Sc = std::min(cols, SC);
   a.ncta = (cols + a.Sc - 1) / a.Sc;
-  const int MS = DL * ((DL + 1) / 2), nB = p.n1 * MS;
-  if (NT > 256 || nB > 2 * NT) return give_up();
+  const int MS = DL * zrow(DL), nB = p.n1 * MS;
+  if (NT > 256 || nB > kROne * NT) return give_up();
   const size_t cs = mixed ? sizeof(float2) : sizeof(double2), zs = 8;
   const size_t img = (size_t)SC * CS * cs, own = (size_t)DL * DL * NT * cs;
   size_t at = 0;
@@ -298,6 +298,38 @@ void ocr_half_step(const OcrPlan* o, const double* E, double dt, void* q, cudaSt
   const int grid = (h.D + 63) / 64;
   if (o->mixed) k_ocr_half<float><<<grid, 64, 0, st>>>(h, (float2*)q);
   else k_ocr_half<double><<<grid, 64, 0, st>>>(h, (double2*)q);
+}
+
+namespace {
+__global__ void k_ocr_many(OcrMany m, int nsys, int N, int K, int sumd, int D, int S, OcSys* __restrict__ t) {
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nsys; b += gridDim.x * blockDim.x) {
+    OcSys d{};
+    d.coef = m.coef + (size_t)b * 3 * N * K;
+    d.ph = m.ph + (size_t)b * N * sumd;
+    d.phmid = 1;
+    d.half = m.half + (size_t)b * D;
+    d.opd64 = m.opd + (size_t)b * m.opd_n;
+    d.J = m.J + (size_t)b * m.J_n;
+    d.psi_api = d.psi_out = m.psi + (size_t)b * D * S;
+    d.K = 1;
+    d.n1 = N;
+    d.C = 1;
+    d.L = N;
+    t[b] = d;
+  }
+}
+}  // namespace
+
+size_t ocr_many_bytes(int nsys) { return (size_t)nsys * sizeof(OcSys); }
+
+cudaError_t ocr_many(const OcrPlan* o, const OcrMany& m, int nsys, int N, double dt, void* table, cudaStream_t st) {
+  k_ocr_many<<<(nsys + 63) / 64, 64, 0, st>>>(m, nsys, N, o->a.K, o->a.sumd, o->a.D, o->a.S, (OcSys*)table);
+  OcBatch bt{};
+  bt.nsys = nsys;
+  bt.many = static_cast<const OcSys*>(table);
+  bt.per = o->a.ncta;
+  ocr_forward(o, bt, dt, st);
+  return cudaGetLastError();
 }
 
 bool ocr_adjoint_ok(const OcrPlan* o) { return o->dens_ok; }

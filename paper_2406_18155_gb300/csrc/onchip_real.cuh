@@ -55,8 +55,12 @@
 #include "onchip_real.h"
 
 constexpr int kRMat = 24;         // constant matrices of a plan
+constexpr int kROne = 3;          // one-body matrix elements a thread renews per stage
 constexpr int kRBuf = 2;          // exchange images beside u and the running sum
 constexpr int kRImp = 3;          // images a phase reads
+
+// Stored row length: the most nonzeros of a row.
+__host__ __device__ constexpr int zrow(int DL) { return (DL + 1) / 2; }
 
 // Where the blocks of the kernels for NQ modes of DL levels lie: all strides are compile-time
 // constants, so a block's accesses are immediate offsets of one address per phase.  Phases
@@ -170,7 +174,6 @@ int ocr_dens_f64(const OcrPlan* o, const OcdArgs& g, const OcdJob& j, cudaStream
 #ifdef OCR_KERNELS
 namespace {
 
-__host__ __device__ constexpr int zrow(int DL) { return (DL + 1) / 2; }
 // the columns of row x that a parity-odd matrix keeps: c = zc(x, 0 .. zn(x) - 1)
 template <int DL> __host__ __device__ constexpr int zn(int x) { return x & 1 ? (DL + 1) / 2 : DL / 2; }
 __host__ __device__ constexpr int zc(int x, int j) { return 2 * j + (x & 1 ? 0 : 1); }
@@ -385,12 +388,12 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
     }
     mat[i] = zdup((R)v);
   }
-  // one-body elements that this thread keeps up to date (the plan has at most 2 a thread)
+  // one-body elements that this thread keeps up to date (the plan has at most kROne a thread)
   const int nB = a.n1 * MS;
-  R o0[2], f0[2];
-  int k0[2];
+  R o0[kROne], f0[kROne];
+  int k0[kROne];
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
+  for (int e = 0; e < kROne; ++e) {
     const int i = tid + e * nthr;
     o0[e] = f0[e] = 0;
     k0[e] = -1;
@@ -409,18 +412,19 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
   };
   auto load_f = [&](int q) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e)
+    for (int e = 0; e < kROne; ++e)
       if (k0[e] >= 0) f0[e] = coef[(size_t)q * a.K + k0[e]];
   };
   auto store_one = [&](int q, Z* to) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < kROne; ++e) {
       const int i = tid + e * nthr;
       if (i < nB) one_body<DL, R>(a, coef, d.opd64, q, i, f0[e], o0[e], to);
     }
   };
   auto mid_phases = [&](int i, C* to) {            // the phases of step i's middle, by cp.async
-    const C* src = ph + (size_t)row_of(i, 1) * a.sumd;
+    const int q = row_of(i, 1);
+    const C* src = ph + (size_t)(d.phmid ? q / 3 : q) * a.sumd;
     for (int j = tid; j < a.sumd; j += nthr) cpv(to + j, src + j);
   };
   if (on) {
@@ -514,6 +518,8 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
         __syncthreads();
         if (on) z_stage<DL, NQ, 2>(a, mat, oc, u, o, at[2]);
       }
+      // (the inner stages share one loop: the code is larger than the instruction cache's reach)
+      const R wks = s == 0 ? (R)1 : wk, c1s = s == 2 ? c1c : c1a, c2s = s == 0 ? c2a : s == 1 ? h / 2 : c2c;
       if (on) {
         // epilogue on the last phase's block
 #pragma unroll
@@ -521,23 +527,19 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
 #pragma unroll
           for (int z = 0; z < DL; ++z) {
             const int e = x * DL + z;
-            const C k = cmk<C>(sg * o[x][z].y, -sg * o[x][z].x);
+            C k = cmk<C>(sg * o[x][z].y, -sg * o[x][z].x);
             C v;
-            if (s == 0) {
-              const C q1 = cmulT(Q.get(e), k), b = bv.get(e);
-              acc.set(e, q1);
-              v = cmk<C>(c1a * b.x + c2a * q1.x, c1a * b.y + c2a * q1.y);
-            } else if (s == 1) {
-              const C b = bv.get(e), g = acc.get(e);
-              acc.set(e, cmk<C>(g.x + wk * k.x, g.y + wk * k.y));
-              v = cmk<C>(c1a * b.x + h / 2 * k.x, c1a * b.y + h / 2 * k.y);
-            } else if (s == 2) {
-              const C b = bv.get(e), g = acc.get(e);
-              acc.set(e, cmk<C>(g.x + wk * k.x, g.y + wk * k.y));
-              v = cmulT(Q.get(e), cmk<C>(c1c * b.x + c2c * k.x, c1c * b.y + c2c * k.y));
-            } else {
+            if (s == 3) {
               const C g = acc.get(e), w = cmulT(cconjT(Q.get(e)), k);
               v = cmk<C>(e3 * (g.x + w.x), e3 * (g.y + w.y));
+            } else {
+              const C b = bv.get(e);
+              C g = cmk<C>(0.0, 0.0);
+              if (s == 0) k = cmulT(Q.get(e), k);
+              else g = acc.get(e);
+              acc.set(e, cmk<C>(g.x + wks * k.x, g.y + wks * k.y));
+              v = cmk<C>(c1s * b.x + c2s * k.x, c1s * b.y + c2s * k.y);
+              if (s == 2) v = cmulT(Q.get(e), v);
             }
             u[x][z] = v;
             if (NP > 1 && s < 3) at[NP - 1][x * SA + z * SB] = v;
@@ -843,10 +845,11 @@ int ocr_t(const OcrPlan* o, OcBatch* bt, double dt, cudaStream_t st) {
       return n;
     }
     int g = 0;
-    for (int b = 0; b < bt->nsys; ++b) {
+    for (int b = 0; b < (bt->many ? 0 : bt->nsys); ++b) {
       bt->cta0[b] = g;
       g += bt->s[b].C * o->a.ncta;
     }
+    if (bt->many) g = bt->nsys * bt->per;
     if (g > 0) k_ocr_fwd<R, DL, NQ><<<g, Lay<DL, NQ>::NT, o->smem, st>>>(o->a, dt, *bt);
     return 1;
   }

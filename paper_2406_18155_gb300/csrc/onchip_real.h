@@ -38,5 +38,20 @@ int ocr_groups(const OcrPlan* o);
 int ocr_densities(const OcrPlan* o, const void* u, const void* k, const void* coef, const double2* opd, const double* J,
                   int n0, int n1, double dt, bool ham, long long nstK, double* gF, double* acc, cudaStream_t st);
 
+// Many systems of one structure from their own start columns (FP32, one chunk each): per
+// system the flat operators and couplings, the coefficients (3N x K), the frame phases of
+// every step's middle (N x sumd), the half-step phases (D) and the columns (D x S, in and out).
+struct OcrMany {
+  const double2* opd;
+  const double* J;
+  const float* coef;
+  const float2 *ph, *half;
+  double2* psi;
+  long long opd_n, J_n;           // entries per system
+};
+// Bytes of the device array that ocr_many fills with the systems' descriptions.
+size_t ocr_many_bytes(int nsys);
+cudaError_t ocr_many(const OcrPlan* o, const OcrMany& m, int nsys, int N, double dt, void* table, cudaStream_t st);
+
 struct OcBatch;
 int ocr_forward(const OcrPlan* o, OcBatch& bt, double dt, cudaStream_t st);

@@ -97,3 +97,22 @@ def test_other_terms_keep_their_kernels(sgctx, monkeypatch, make):
     monkeypatch.setenv("SG_PATH", "gather")
     ref = s.evolve(wl["T"], wl["dt"], precision="fp64", col_index=wl["col_index"]).cpu().numpy()
     assert np.max(np.abs(psi - ref)) <= 1e-10
+
+
+@pytest.mark.parametrize("odd_one_out", [False, True])
+def test_batch_of_pairs(sgctx, odd_one_out):
+    # one structure: the on-chip kernel, a warp per system; a system with its coupling written
+    # the other way round: the tensor-core kernel for all
+    from paper_2406_18155_gb300.api import System, evolve_batch
+    wls = [W.fluxonium_pair_multipath(seed=s, T=0.3, levels=4) for s in range(3)]
+    if odd_one_out:
+        c = wls[1]["couplings"][0]
+        c["a"], c["b"] = c["b"], c["a"]
+    cols = [3, 0, 15, 1, 4, 5, 2, 7, 8, 14, 6, 9, 10, 13, 12, 11]
+    systems = [System.from_workload(sgctx, wl) for wl in wls]
+    for s in systems:
+        s.prepare()
+    psi = evolve_batch(systems, 0.3, 0.01, cols).cpu().numpy()
+    for p, s in zip(psi, systems):
+        ref = s.evolve(0.3, 0.01, precision="fp64", col_index=cols).cpu().numpy()
+        assert np.max(np.abs(p - ref)) <= 1e-5
