@@ -310,45 +310,57 @@ __global__ void k_ops_z(TabArgs a, Z* __restrict__ zo, int zpar, int DL) {
 // ---------------------------------------------------------------------------
 // exp(A) of a small complex matrix (n x n, row-major) by scaling and squaring of
 // the Taylor series (Moler and Van Loan's method 3): A / 2^s with |A / 2^s|_1 <= 1/2,
-// 18 Taylor terms (remainder below 1e-22 of the norm), then s squarings.  Serial,
-// one thread: R = exp(A); W1, W2 are n x n scratch.
-__device__ void expm_serial(const double2* A, int n, double2* R, double2* W1, double2* W2) {
-  double nrm = 0.0;
-  for (int c = 0; c < n; ++c) {
+// 18 Taylor terms (remainder below 1e-22 of the norm), then s squarings.  By a team of nt threads
+// (t: this one), each taking elements of the products; sync orders the team's shared-memory
+// accesses.  R = exp(A); W1, W2 are n x n scratch, red n values.  (One thread per matrix with
+// its arrays in local memory took 34.6 ms for the ten 16 x 16 coupling exponentials of a
+// six-mode chain and 21.6 ms for the gradient tables of 300 steps.)
+template <typename Sync>
+__device__ void expm_team(const double2* A, int n, double2* R, double2* W1, double2* W2, double* red, int t, int nt,
+                          Sync sync) {
+  for (int c = t; c < n; c += nt) {
     double col = 0.0;
     for (int r = 0; r < n; ++r) col += hypot(A[r * n + c].x, A[r * n + c].y);
-    nrm = fmax(nrm, col);
+    red[c] = col;
   }
+  for (int i = t; i < n * n; i += nt) R[i] = W1[i] = make_double2((i / n == i % n) ? 1.0 : 0.0, 0.0);
+  sync();
+  double nrm = 0.0;
+  for (int c = 0; c < n; ++c) nrm = fmax(nrm, red[c]);
   int sq = 0;
   while (nrm > 0.5 && sq < 60) { nrm *= 0.5; ++sq; }
   const double sc = ldexp(1.0, -sq);
-  for (int i = 0; i < n * n; ++i) {
-    W1[i] = make_double2((i / n == i % n) ? 1.0 : 0.0, 0.0);    // current term
-    R[i] = W1[i];
-  }
   for (int k = 1; k <= 18; ++k) {
-    for (int r = 0; r < n; ++r)                                 // W2 = W1 (A sc) / k
-      for (int c = 0; c < n; ++c) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int m = 0; m < n; ++m) acc = cfma(W1[r * n + m], A[m * n + c], acc);
-        W2[r * n + c] = make_double2(acc.x * sc / k, acc.y * sc / k);
-      }
-    for (int i = 0; i < n * n; ++i) {
-      W1[i] = W2[i];
+    for (int i = t; i < n * n; i += nt) {                       // W2 = W1 (A sc) / k
+      const int r = i / n, c = i - r * n;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int m = 0; m < n; ++m) acc = cfma(W1[r * n + m], A[m * n + c], acc);
+      W2[i] = make_double2(acc.x * sc / k, acc.y * sc / k);
       R[i].x += W2[i].x;
       R[i].y += W2[i].y;
     }
+    sync();
+    double2* x = W1; W1 = W2; W2 = x;
   }
+  double2* Q = R;
+  double2* T = W1;
   for (int q = 0; q < sq; ++q) {
-    for (int r = 0; r < n; ++r)
-      for (int c = 0; c < n; ++c) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int m = 0; m < n; ++m) acc = cfma(R[r * n + m], R[m * n + c], acc);
-        W2[r * n + c] = acc;
-      }
-    for (int i = 0; i < n * n; ++i) R[i] = W2[i];
+    for (int i = t; i < n * n; i += nt) {
+      const int r = i / n, c = i - r * n;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int m = 0; m < n; ++m) acc = cfma(Q[r * n + m], Q[m * n + c], acc);
+      T[i] = acc;
+    }
+    sync();
+    double2* x = Q; Q = T; T = x;
+  }
+  if (Q != R) {
+    for (int i = t; i < n * n; i += nt) R[i] = Q[i];
+    sync();
   }
 }
+struct WarpSync { __device__ void operator()() const { __syncwarp(); } };
+struct BlockSync { __device__ void operator()() const { __syncthreads(); } };
 
 // Drive coefficient f_k = E(t) cos(omega t + phase) at the complex time t = tr + i ti
 // inside step n: Gaussian and cosine envelopes and the carrier continued analytically,
@@ -372,67 +384,68 @@ __device__ double2 coef_complex(const DriveDev& dr, const double* amps, int n, d
 }
 
 // U_i(m) = exp(A), A = -i c_j (dt/2) H_i(t_n + tau_j dt) for sub-step m = J n + j,
-// H_i = diag(E) + sum_{drives k on i} f_k O_k.  A is left in A.
-__device__ void q2_onebody(const TabArgs& a, int i, int m, double2* U, double2* A, double2* W1, double2* W2) {
+// H_i = diag(E) + sum_{drives k on i} f_k O_k, by one warp in shared memory.  A is left in A.
+struct Q2Work {
+  double2 U[SG_MAXD * SG_MAXD], A[SG_MAXD * SG_MAXD], W1[SG_MAXD * SG_MAXD], W2[SG_MAXD * SG_MAXD];
+  double2 f[SG_MAXDRIVE];
+  double red[2 * SG_MAXD];
+};
+__device__ void q2_onebody(const TabArgs& a, int i, int m, Q2Work& w, int lane) {
   const int d = a.dims[i];
   const int n = m / a.nsub, j = m - n * a.nsub;
   const double tr = (double)(2 * n + 1) * a.dt * 0.5 + (a.tau[j].x - 0.5) * a.dt;
   const double ti = a.tau[j].y * a.dt;
-  for (int x = 0; x < d * d; ++x) A[x] = make_double2(0.0, 0.0);
-  for (int x = 0; x < d; ++x) A[x * d + x].x = a.E[a.eoff[i] + x];
-  for (int k = 0; k < a.K; ++k) {
-    const DriveDev& dr = a.drives[k];
-    if (dr.mode != i) continue;
-    const double2 f = coef_complex(dr, a.amps, n, tr, ti);
-    const double2* O = a.opd + a.opd_off[i] + dr.op * d * d;
-    for (int x = 0; x < d * d; ++x) A[x] = cfma(f, O[x], A[x]);
-  }
+  for (int k = lane; k < a.K; k += 32)
+    if (a.drives[k].mode == i) w.f[k] = coef_complex(a.drives[k], a.amps, n, tr, ti);
+  __syncwarp();
   const double h = a.q1 ? a.dt : a.dt * 0.5;        // Q1: the full step
-  for (int x = 0; x < d * d; ++x) {
-    const double2 cH = cmul(a.sc[j], A[x]);
-    A[x] = make_double2(h * cH.y, -h * cH.x);                                     // -i c H dt/2 (Q1: dt)
+  for (int x = lane; x < d * d; x += 32) {
+    double2 v = make_double2(x % (d + 1) == 0 ? a.E[a.eoff[i] + x / (d + 1)] : 0.0, 0.0);
+    for (int k = 0; k < a.K; ++k)
+      if (a.drives[k].mode == i) v = cfma(w.f[k], a.opd[a.opd_off[i] + a.drives[k].op * d * d + x], v);
+    const double2 cH = cmul(a.sc[j], v);
+    w.A[x] = make_double2(h * cH.y, -h * cH.x);                                   // -i c H dt/2 (Q1: dt)
   }
-  expm_serial(A, d, U, W1, W2);
+  __syncwarp();
+  expm_team(w.A, d, w.U, w.W1, w.W2, w.red, lane, 32, WarpSync());
 }
 
 // Row m < M - 1 (M = J N sub-steps): V_i(m) = U_i(m+1) U_i(m) (the second half of
 // sub-step m followed by the first of sub-step m + 1); row M - 1: U_i(M - 1); row M:
-// U_i(0).  One thread per (row, mode).
-__global__ void k_q2_onebody(TabArgs a, int DL, double2* __restrict__ rows) {
+// U_i(0).  One warp per (row, mode).
+constexpr int kQ2Warps = 4;
+__global__ void __launch_bounds__(32 * kQ2Warps) k_q2_onebody(TabArgs a, int DL, double2* __restrict__ rows) {
+  __shared__ Q2Work work[kQ2Warps];
+  __shared__ double2 first[kQ2Warps][SG_MAXD * SG_MAXD];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  Q2Work& w = work[wi];
+  double2* const U0 = first[wi];
   const int M = a.N * a.nsub, nrow = M + 1;
-  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nrow * a.nq; x += gridDim.x * blockDim.x) {
+  for (int x = blockIdx.x * kQ2Warps + wi; x < nrow * a.nq; x += gridDim.x * kQ2Warps) {
     const int m = x / a.nq, i = x - m * a.nq, d = a.dims[i];
-    double2 U0[SG_MAXD * SG_MAXD], U1[SG_MAXD * SG_MAXD], A[SG_MAXD * SG_MAXD];
-    double2 W1[SG_MAXD * SG_MAXD], W2[SG_MAXD * SG_MAXD];
     double2* out = rows + ((size_t)m * a.nq + i) * DL * DL;
-    if (m == M) {
-      q2_onebody(a, i, 0, U0, A, W1, W2);
-      for (int y = 0; y < d * d; ++y) out[y] = U0[y];
+    if (a.q1 && m == M - 1) {
+      for (int y = lane; y < d * d; y += 32) out[y] = make_double2(y % (d + 1) == 0 ? 1.0 : 0.0, 0.0);
       continue;
     }
-    if (a.q1) {
-      // Q1: row M is step 0's 1-body factor, applied first; row m < M - 1 step m + 1's,
-      // applied after step m's couplings; row M - 1 the identity
-      if (m == M - 1) {
-        for (int y = 0; y < d * d; ++y) out[y] = make_double2(y % (d + 1) == 0 ? 1.0 : 0.0, 0.0);
-      } else {
-        q2_onebody(a, i, m + 1, U0, A, W1, W2);
-        for (int y = 0; y < d * d; ++y) out[y] = U0[y];
-      }
+    // Q1: row M is step 0's 1-body factor, applied first; row m < M - 1 step m + 1's,
+    // applied after step m's couplings; row M - 1 the identity
+    q2_onebody(a, i, m == M ? 0 : a.q1 ? m + 1 : m, w, lane);
+    if (a.q1 || m >= M - 1) {
+      for (int y = lane; y < d * d; y += 32) out[y] = w.U[y];
+      __syncwarp();
       continue;
     }
-    q2_onebody(a, i, m, U0, A, W1, W2);
-    if (m == M - 1) {
-      for (int y = 0; y < d * d; ++y) out[y] = U0[y];
-      continue;
+    for (int y = lane; y < d * d; y += 32) U0[y] = w.U[y];
+    __syncwarp();
+    q2_onebody(a, i, m + 1, w, lane);
+    for (int y = lane; y < d * d; y += 32) {
+      const int r = y / d, c = y - r * d;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int q = 0; q < d; ++q) acc = cfma(w.U[r * d + q], U0[q * d + c], acc);
+      out[y] = acc;
     }
-    q2_onebody(a, i, m + 1, U1, A, W1, W2);
-    for (int r = 0; r < d; ++r)
-      for (int c = 0; c < d; ++c) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int q = 0; q < d; ++q) acc = cfma(U1[r * d + q], U0[q * d + c], acc);
-        out[r * d + c] = acc;
-      }
+    __syncwarp();
   }
 }
 
@@ -441,17 +454,20 @@ __global__ void k_q2_onebody(TabArgs a, int DL, double2* __restrict__ rows) {
 // at matrices (s ne + e) 2 + {0, 1}; for the pull-back of the gradient, from matrix
 // 2 ne nset on, per (s, e) four: the inverses G_half^-1, G_full^-1 (the states) and the
 // adjoints G_half^dag, G_full^dag (the co-states), equal pairs when c_s is real.  One
-// thread per (set, coupling).
-__global__ void k_q2_edges(TabArgs a, int DL, double2* __restrict__ mats, double2* __restrict__ scratch) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+// block per (set, coupling), n <= 25.
+constexpr int kQ2EdgeN = 25;
+__global__ void __launch_bounds__(256) k_q2_edges(TabArgs a, int DL, double2* __restrict__ mats) {
+  extern __shared__ __align__(16) unsigned char esm[];
+  __shared__ double red[kQ2EdgeN];
+  const int x = blockIdx.x, t = threadIdx.x, nt = blockDim.x;
   const int ne = a.p.ne;
-  if (x >= ne * a.nset) return;
   const int sidx = x / ne, e = x - sidx * ne;
   const int ia = a.p.e_a[e], ib = a.p.e_b[e], da = a.dims[ia], db = a.dims[ib], n = da * db;
   const double2* Aop = a.opd + a.opd_off[ia] + a.e_opa[e] * da * da;
   const double2* Bop = a.opd + a.opd_off[ib] + a.e_opb[e] * db * db;
-  double2* M = scratch + (size_t)x * 3 * n * n;
-  double2* W1 = M + n * n;
+  double2* M = reinterpret_cast<double2*>(esm);
+  double2* R = M + n * n;
+  double2* W1 = R + n * n;
   double2* W2 = W1 + n * n;
   const size_t D4 = (size_t)DL * DL * DL * DL;
   double2* Gh = mats + (size_t)x * 2 * D4;
@@ -462,33 +478,30 @@ __global__ void k_q2_edges(TabArgs a, int DL, double2* __restrict__ mats, double
   double2* Gfd = Ghd + D4;
   const double h = a.J[e] * a.dt * 0.5;
   const double2 c = a.setc[sidx];
-  for (int xx = 0; xx < da; ++xx)
-    for (int z = 0; z < db; ++z)
-      for (int p = 0; p < da; ++p)
-        for (int q = 0; q < db; ++q) {
-          const double2 v = cmul(c, cmul(Aop[xx * da + p], Bop[z * db + q]));
-          M[(xx * db + z) * n + p * db + q] = make_double2(h * v.y, -h * v.x);   // -i c J (A x B) dt/2
-        }
-  expm_serial(M, n, Gh, W1, W2);
-  for (int r = 0; r < n; ++r)
-    for (int q = 0; q < n; ++q) {
+  for (int i = t; i < n * n; i += nt) {
+    const int r = i / n, q = i - r * n;
+    const double2 v = cmul(c, cmul(Aop[r / db * da + q / db], Bop[r % db * db + q % db]));
+    M[i] = make_double2(h * v.y, -h * v.x);                                      // -i c J (A x B) dt/2
+  }
+  __syncthreads();
+  for (int inv = 0; inv < 2; ++inv) {                                            // then exp(+i c J (A x B) dt/2)
+    expm_team(M, n, R, W1, W2, red, t, nt, BlockSync());
+    double2* H = inv ? Ghi : Gh;
+    double2* F = inv ? Gfi : Gf;
+    for (int i = t; i < n * n; i += nt) {
+      const int r = i / n, q = i - r * n;
       double2 acc = make_double2(0.0, 0.0);
-      for (int m = 0; m < n; ++m) acc = cfma(Gh[r * n + m], Gh[m * n + q], acc);
-      Gf[r * n + q] = acc;
+      for (int m = 0; m < n; ++m) acc = cfma(R[r * n + m], R[m * n + q], acc);
+      H[i] = R[i];
+      F[i] = acc;
+      if (!inv) {
+        Ghd[q * n + r] = cconj(R[i]);
+        Gfd[q * n + r] = cconj(acc);
+      }
+      M[i] = make_double2(-M[i].x, -M[i].y);
     }
-  for (int r = 0; r < n; ++r)
-    for (int q = 0; q < n; ++q) {
-      Ghd[r * n + q] = cconj(Gh[q * n + r]);
-      Gfd[r * n + q] = cconj(Gf[q * n + r]);
-    }
-  for (int i = 0; i < n * n; ++i) M[i] = make_double2(-M[i].x, -M[i].y);
-  expm_serial(M, n, Ghi, W1, W2);                                                // exp(+i c J (A x B) dt/2)
-  for (int r = 0; r < n; ++r)
-    for (int q = 0; q < n; ++q) {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int m = 0; m < n; ++m) acc = cfma(Ghi[r * n + m], Ghi[m * n + q], acc);
-      Gfi[r * n + q] = acc;
-    }
+    __syncthreads();
+  }
 }
 
 // Gradient tables (pulse parameters), rows [J N][2 nq + K][d^2]: per sub-step m the
@@ -498,48 +511,61 @@ __global__ void k_q2_edges(TabArgs a, int DL, double2* __restrict__ mats, double
 // M_k(m) = U_i(m)^-1 L_k(m) with L_k(m) = L(A, -i c_j (dt/2) O_k) the Frechet derivative
 // of expm at A = -i c_j (dt/2) H_i(t_n + tau_j dt), the top-right block of
 // exp([[A, E], [0, A]]) (Sec. 2.5: dU/df_k).  Q1: the step's full-step factor, dt for
-// dt/2 throughout.  One thread per (m, row).
+// dt/2 throughout.  One warp per (m, row).
 constexpr int kQ2MaxD = 5;
-__global__ void k_q2_gradtabs(TabArgs a, int DL, double2* __restrict__ rows) {
+struct Q2GradWork {
+  Q2Work w;
+  double2 Ui[SG_MAXD * SG_MAXD];
+  double2 Z[4 * kQ2MaxD * kQ2MaxD], RZ[4 * kQ2MaxD * kQ2MaxD], Z1[4 * kQ2MaxD * kQ2MaxD], Z2[4 * kQ2MaxD * kQ2MaxD];
+};
+__global__ void __launch_bounds__(32 * kQ2Warps) k_q2_gradtabs(TabArgs a, int DL, double2* __restrict__ rows) {
+  extern __shared__ __align__(16) unsigned char gsm[];
   const int per = 2 * a.nq + a.K, M = a.N * a.nsub;
-  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < M * per; x += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  Q2GradWork& g = reinterpret_cast<Q2GradWork*>(gsm)[wi];
+  for (int x = blockIdx.x * kQ2Warps + wi; x < M * per; x += gridDim.x * kQ2Warps) {
     const int m = x / per, r = x - m * per;
-    double2 U[SG_MAXD * SG_MAXD], A[SG_MAXD * SG_MAXD], W1[SG_MAXD * SG_MAXD], W2[SG_MAXD * SG_MAXD];
-    double2 Ui[SG_MAXD * SG_MAXD];
     double2* out = rows + ((size_t)m * per + r) * DL * DL;
     if (r < 2 * a.nq) {
       const int i = r < a.nq ? r : r - a.nq, d = a.dims[i];
-      q2_onebody(a, i, m, U, A, W1, W2);
+      q2_onebody(a, i, m, g.w, lane);
       if (r >= a.nq) {
-        for (int p = 0; p < d; ++p)
-          for (int c = 0; c < d; ++c) out[p * d + c] = cconj(U[c * d + p]);
+        for (int y = lane; y < d * d; y += 32) out[y] = cconj(g.w.U[y % d * d + y / d]);
       } else {
-        for (int p = 0; p < d * d; ++p) A[p] = make_double2(-A[p].x, -A[p].y);
-        expm_serial(A, d, Ui, W1, W2);
-        for (int p = 0; p < d * d; ++p) out[p] = Ui[p];
+        for (int p = lane; p < d * d; p += 32) g.w.A[p] = make_double2(-g.w.A[p].x, -g.w.A[p].y);
+        __syncwarp();
+        expm_team(g.w.A, d, g.Ui, g.w.W1, g.w.W2, g.w.red, lane, 32, WarpSync());
+        for (int p = lane; p < d * d; p += 32) out[p] = g.Ui[p];
       }
+      __syncwarp();
       continue;
     }
     const DriveDev& dr = a.drives[r - 2 * a.nq];
     const int i = dr.mode, d = a.dims[i], mm = 2 * d;
     if (d > kQ2MaxD) continue;                      // the on-chip Suzuki-Trotter plan has d <= 5
-    q2_onebody(a, i, m, U, A, W1, W2);              // U_i(m), and A = -i c (dt/2) H_i on return
-    constexpr int MM = 4 * kQ2MaxD * kQ2MaxD;
-    double2 Z[MM], RZ[MM], Z1[MM], Z2[MM];
+    q2_onebody(a, i, m, g.w, lane);                 // U_i(m), and A = -i c (dt/2) H_i on return
+    double2* const A = g.w.A;
+    double2* const Ui = g.Ui;
+    double2* const RZ = g.RZ;
     const double2* O = a.opd + a.opd_off[i] + dr.op * d * d;
     const double h = a.q1 ? a.dt : a.dt * 0.5;       // Q1: full-step factors
     const double2 c = a.sc[m % a.nsub];
-    for (int p = 0; p < mm * mm; ++p) Z[p] = make_double2(0.0, 0.0);
-    for (int p = 0; p < d; ++p)
-      for (int q = 0; q < d; ++q) {
-        Z[p * mm + q] = A[p * d + q];
-        Z[(p + d) * mm + q + d] = A[p * d + q];
-        const double2 cO = cmul(c, O[p * d + q]);
-        Z[p * mm + q + d] = make_double2(h * cO.y, -h * cO.x);                 // -i c (dt/2) O (Q1: dt)
+    for (int y = lane; y < mm * mm; y += 32) {
+      const int p = y / mm, q = y - p * mm;
+      double2 v = make_double2(0.0, 0.0);
+      if ((p < d) == (q < d)) {
+        v = A[p % d * d + q % d];
+      } else if (p < d) {
+        const double2 cO = cmul(c, O[p * d + q - d]);
+        v = make_double2(h * cO.y, -h * cO.x);                                   // -i c (dt/2) O (Q1: dt)
       }
-    expm_serial(Z, mm, RZ, Z1, Z2);
-    for (int p = 0; p < d * d; ++p) A[p] = make_double2(-A[p].x, -A[p].y);
-    expm_serial(A, d, Ui, W1, W2);                  // U^-1 = exp(-A)
+      g.Z[y] = v;
+    }
+    __syncwarp();
+    expm_team(g.Z, mm, RZ, g.Z1, g.Z2, g.w.red, lane, 32, WarpSync());
+    for (int p = lane; p < d * d; p += 32) A[p] = make_double2(-A[p].x, -A[p].y);
+    __syncwarp();
+    expm_team(A, d, Ui, g.w.W1, g.w.W2, g.w.red, lane, 32, WarpSync());          // U^-1 = exp(-A)
     // df_k/dtheta = z (a segment or amplitude indicator): z = carrier x envelope shape at
     // the sub-step time (complex for Q4j), folded in here so that the real part the
     // adjoint takes is Re(<psibar, L psi> df/dtheta)
@@ -559,12 +585,13 @@ __global__ void k_q2_gradtabs(TabArgs a, int DL, double2* __restrict__ rows) {
     }
     const double wa = dr.omega * tr + dr.phase, wb = dr.omega * ti;
     z = cmul(z, make_double2(cos(wa) * cosh(wb), -(sin(wa) * sinh(wb))));
-    for (int p = 0; p < d; ++p)                     // M = z U^-1 L
-      for (int q = 0; q < d; ++q) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int w = 0; w < d; ++w) acc = cfma(Ui[p * d + w], RZ[w * mm + q + d], acc);
-        out[p * d + q] = cmul(z, acc);
-      }
+    for (int y = lane; y < d * d; y += 32) {        // M = z U^-1 L
+      const int p = y / d, q = y - p * d;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int w = 0; w < d; ++w) acc = cfma(Ui[p * d + w], RZ[w * mm + q + d], acc);
+      out[y] = cmul(z, acc);
+    }
+    __syncwarp();
   }
 }
 
@@ -1841,10 +1868,12 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
     const size_t nrow = (size_t)(M + 1) * s.nq * DL * DL, nedge = (size_t)6 * ne1 * nset * D4;
     double2* rows = sv.ar.get<double2>(nrow);
     double2* edges = sv.ar.get<double2>(nedge);
-    double2* scratch = sv.ar.get<double2>((size_t)ne1 * nset * 3 * D4);
-    if (!rows || !edges || !scratch) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the Q2 tables failed");
-    k_q2_onebody<<<grid_for((M + 1) * s.nq), kT, 0, st>>>(ta, DL, rows);
-    if (s.p.ne) k_q2_edges<<<(s.p.ne * nset + 31) / 32, 32, 0, st>>>(ta, DL, edges, scratch);
+    if (!rows || !edges) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the Q2 tables failed");
+    auto q2_grid = [](long long tasks) {
+      return (unsigned)std::max<long long>(1, std::min<long long>((tasks + kQ2Warps - 1) / kQ2Warps, 152ll * 32));
+    };
+    k_q2_onebody<<<q2_grid((M + 1) * s.nq), 32 * kQ2Warps, 0, st>>>(ta, DL, rows);
+    if (s.p.ne) k_q2_edges<<<s.p.ne * nset, 256, 4 * D4 * sizeof(double2), st>>>(ta, DL, edges);
     sv.launches += 2;
     sv.q2rows = rows;
     sv.q2edges = edges;
@@ -1853,7 +1882,10 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
     if (grad) {
       gtab = sv.ar.get<double2>(ngr);
       if (!gtab) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the Q2 gradient tables failed");
-      k_q2_gradtabs<<<grid_for(M * (2 * s.nq + s.K)), 64, 0, st>>>(ta, DL, gtab);
+      static const cudaError_t gattr = cudaFuncSetAttribute(k_q2_gradtabs, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                            (int)(kQ2Warps * sizeof(Q2GradWork)));
+      SG_CUDA_TRY(ctx, gattr);
+      k_q2_gradtabs<<<q2_grid(M * (2 * s.nq + s.K)), 32 * kQ2Warps, kQ2Warps * sizeof(Q2GradWork), st>>>(ta, DL, gtab);
       ++sv.launches;
       sv.q2grad = gtab;
     }

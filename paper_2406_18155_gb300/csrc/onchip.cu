@@ -552,6 +552,7 @@ struct Q2Factor {
   Phase P;
   int kind;
   int mat;                        // kind 2: index of the d^4 matrix in the edge table
+  int spar;                       // kind 2: both factors parity-odd (block_dense)
 };
 struct Q2Args {
   int nf0;                        // 1-body factors (applied first with the initial row,
@@ -570,7 +571,8 @@ __device__ __forceinline__ void q2_apply(const Q2Factor& F, int mat, const OcArg
   for (int b = threadIdx.x; b < oa.nbt; b += blockDim.x) {
     const int c = b / oa.nbc;
     const int pb = blk_pos<DL>(P, b - c * oa.nbc) + c * oa.CS;
-    if (F.kind == 2) block_dense<DL>(edges + (size_t)mat * DL * DL * DL * DL, ys, ks, pb, P.psa, P.psb);
+    if (F.kind == 2 && F.spar) block_dense<DL, true>(edges + (size_t)mat * DL * DL * DL * DL, ys, ks, pb, P.psa, P.psb);
+    else if (F.kind == 2) block_dense<DL>(edges + (size_t)mat * DL * DL * DL * DL, ys, ks, pb, P.psa, P.psb);
     else phase_block<DL, false>(P, M, ys, ks, pb, true);
   }
   __syncthreads();
@@ -675,6 +677,7 @@ struct Q2AdjArgs {
   int setoff[3];                  // first matrix of sub-step j's pull-back coupling set: 4 ne set(j)
   int row;                        // (nq + K) d^2: U_i(n)^dag then M_k(n)
   unsigned driven;                // bit i: a drive acts on mode i
+  unsigned spar;                  // bit e: both factors of coupling e parity-odd (block_dense)
   Phase one[SG_MAXQ / 2 + 1];     // pairs (offL, offR) and an odd last mode (offA)
   Phase mode[SG_MAXQ];            // cross-density block layout of mode i
   Phase edge[32];
@@ -739,8 +742,13 @@ k_oc_q2_adj(SlabPass sp, OcArgs oa, Q2AdjArgs qa, const typename CT<R>::T* __res
           for (int b = threadIdx.x; b < oa.nbt; b += blockDim.x) {
             const int c = b / oa.nbc;
             const int pb = blk_pos<DL>(P, b - c * oa.nbc) + c * oa.CS;
-            block_dense<DL>(Gi, xs, t1, pb, P.psa, P.psb);
-            block_dense<DL>(Gd, xb, t2, pb, P.psa, P.psb);
+            if ((qa.spar >> e) & 1u) {
+              block_dense<DL, true>(Gi, xs, t1, pb, P.psa, P.psb);
+              block_dense<DL, true>(Gd, xb, t2, pb, P.psa, P.psb);
+            } else {
+              block_dense<DL>(Gi, xs, t1, pb, P.psa, P.psb);
+              block_dense<DL>(Gd, xb, t2, pb, P.psa, P.psb);
+            }
           }
           __syncthreads();
           C* tmp = xs; xs = t1; t1 = tmp;
@@ -1535,6 +1543,7 @@ sg_status onchip_q2_forward(const OnchipPlan* oc, const KPlan& p, const void* ro
     F.P = make_phase(sp, DL, p.e_a[e], p.e_b[e]);
     F.kind = 2;
     F.mat = 2 * e;                // per set and coupling: half, full
+    F.spar = ((p.parL >> e) & 1ull) && ((p.parR >> e) & 1ull);
   }
   qa.J = J;
   qa.q1 = q1 ? 1 : 0;
@@ -1607,7 +1616,10 @@ sg_status onchip_q2_pulse_adjoint(const OnchipPlan* oc, const KPlan& p, const in
     }
   }
   for (int i = 0; i < p.nq; ++i) qa.mode[i] = make_phase(sp, DL, i, i == 0 ? 1 : 0);
-  for (int e = 0; e < p.ne; ++e) qa.edge[e] = make_phase(sp, DL, p.e_a[e], p.e_b[e]);
+  for (int e = 0; e < p.ne; ++e) {
+    qa.edge[e] = make_phase(sp, DL, p.e_a[e], p.e_b[e]);
+    if (((p.parL >> e) & 1ull) && ((p.parR >> e) & 1ull)) qa.spar |= 1u << e;
+  }
   for (int k = 0; k < K; ++k) {
     qa.drv_mode[k] = drv_mode[k];
     qa.driven |= 1u << drv_mode[k];

@@ -177,8 +177,10 @@ __device__ __forceinline__ void blk_apply(const Phase& P, const C* __restrict__ 
 }
 
 // o[x][z] = sum_{a,c} G[(x d + z), (a d + c)] y[a][c] over one block (digits ka, kb): a
-// dense two-mode factor (the Suzuki-Trotter coupling unitaries).
-template <int DL, typename C>
+// dense two-mode factor (the Suzuki-Trotter coupling unitaries).  PAR: exp of A (x) B with A and
+// B parity-odd, so output (x, z) takes only inputs with a + c = x + z mod 2 (the others' elements
+// are zero); the kept terms go to the same sums in the same order.
+template <int DL, bool PAR = false, typename C>
 __device__ __forceinline__ void block_dense(const C* __restrict__ G, const C* __restrict__ ys, C* __restrict__ ks,
                                             int pb, int psa, int psb) {
   C y[DL][DL];
@@ -186,20 +188,35 @@ __device__ __forceinline__ void block_dense(const C* __restrict__ G, const C* __
   for (int a = 0; a < DL; ++a)
 #pragma unroll
     for (int c = 0; c < DL; ++c) y[a][c] = ys[pb + a * psa + c * psb];
-  // one output per iteration (a runtime loop keeps the d^4 code small)
+#pragma unroll
+  for (int par = 0; par < (PAR ? 2 : 1); ++par) {
+    // one output per iteration (a runtime loop keeps the d^4 code small)
 #pragma unroll 1
-  for (int xz = 0; xz < DL * DL; ++xz) {
-    const C* g = G + xz * DL * DL;
-    C acc0 = cmk<C>(0.0, 0.0), acc1 = cmk<C>(0.0, 0.0);       // two chains for latency
-#pragma unroll
-    for (int a = 0; a < DL; ++a)
-#pragma unroll
-      for (int c = 0; c < DL; ++c) {
-        if ((a * DL + c) & 1) acc1 = cfma(g[a * DL + c], y[a][c], acc1);
-        else acc0 = cfma(g[a * DL + c], y[a][c], acc0);
+    for (int k = 0; k < (PAR ? (DL * DL + 1 - par) / 2 : DL * DL); ++k) {
+      // PAR: the k-th (x, z) of parity par, in row order
+      int x, z;
+      if (!PAR) {
+        x = k / DL;
+        z = k - x * DL;
+      } else if (DL & 1) {
+        x = (2 * k + par) / DL;
+        z = 2 * k + par - x * DL;
+      } else {
+        x = k / (DL / 2);
+        z = 2 * (k - x * (DL / 2)) + ((x + par) & 1);
       }
-    const int x = xz / DL, z = xz - x * DL;
-    ks[pb + x * psa + z * psb] = cmk<C>(acc0.x + acc1.x, acc0.y + acc1.y);
+      const C* g = G + (x * DL + z) * DL * DL;
+      C acc0 = cmk<C>(0.0, 0.0), acc1 = cmk<C>(0.0, 0.0);       // two chains for latency
+#pragma unroll
+      for (int a = 0; a < DL; ++a)
+#pragma unroll
+        for (int c = 0; c < DL; ++c) {
+          if (PAR && ((a + c) & 1) != par) continue;
+          if ((a * DL + c) & 1) acc1 = cfma(g[a * DL + c], y[a][c], acc1);
+          else acc0 = cfma(g[a * DL + c], y[a][c], acc0);
+        }
+      ks[pb + x * psa + z * psb] = cmk<C>(acc0.x + acc1.x, acc0.y + acc1.y);
+    }
   }
 }
 
