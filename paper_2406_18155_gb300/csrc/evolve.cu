@@ -1695,7 +1695,10 @@ struct KTimer {
 struct OcChunks {
   bool prop = false, par = false;
   bool direct = false;            // one chunk whose serial passes keep every stage input
-  void *segU = nullptr;           // direct: the stage inputs of all steps
+  void *segU = nullptr, *segK = nullptr;   // direct: the stage inputs of all steps
+  // serial passes side by side: the co-states are sums over the computational rows j of
+  // barc[j][s] times the pulled-back unit vectors e_j, which need no forward result
+  bool basis = false;
   int L = 1, C = 1, R = 1;
   int G = 1, NG = 1;              // prop: chunks per group of the two-level product, groups
   double2 *ck = nullptr, *lam = nullptr;   // states before, co-states after each chunk
@@ -1740,6 +1743,7 @@ struct Solve {
   bool real_oc = false;           // terms real up to the frame phases (rterms), interaction frame
   OcrTerms rterms;
   void* half = nullptr;           // onchip_half_step
+  const double2* barc = nullptr;  // co-states on the computational rows (Dc x S), product basis
   ~Solve() {
     slab_plan_destroy(slab);
     onchip_plan_destroy(oc);
@@ -1798,8 +1802,46 @@ void fill_terms(const Setup& s, const TabArgs& ta, OcrTerms& rt) {
   for (int u = 0; u <= s.p.n1; ++u) rt.drv_start[u] = ta.drv_of_slot_start[u];
   for (int k = 0; k < s.K; ++k) { rt.drv_list[k] = ta.drv_list[k]; rt.drv_op[k] = s.drives[k].op; }
   for (int e = 0; e < s.p.ne; ++e) {
-    rt.e_opa[e] = ta.e_opa[e]; rt.e_opb[e] = ta.e_opb[e]; rt.e_part[e] = ta.e_zpart[e];
+    rt.e_opa[e] = ta.e_opa[e]; rt.e_opb[e] = ta.e_opb[e]; rt.e_pa[e] = rt.e_pb[e] = ta.e_zpart[e];
   }
+}
+
+// The parts of the couplings' factors and a choice of modes to turn (OcrTerms::flip) that
+// makes every drive real and both factors of every coupling real or both imaginary; false if
+// there is none.  Turning a mode exchanges the parts of its parity-odd operators (the on-chip plan
+// takes no others).
+bool real_gauge(const sg_system* sys, const Setup& s, OcrTerms& rt) {
+  std::vector<int> f(s.nq, -1);
+  for (const HostDrive& hd : sys->drives) {
+    const int part = op_part(sys, hd.mode, hd.op);
+    if (part < 0 || (f[hd.mode] >= 0 && f[hd.mode] != part)) return false;
+    f[hd.mode] = part;
+  }
+  for (int e = 0; e < s.p.ne; ++e) {
+    const HostCoupling& c = sys->couplings[e];
+    rt.e_pa[e] = op_part(sys, c.a, c.op_a);
+    rt.e_pb[e] = op_part(sys, c.b, c.op_b);
+    if (rt.e_pa[e] < 0 || rt.e_pb[e] < 0) return false;
+  }
+  // settled modes settle their neighbours; an unsettled component starts from its first mode
+  for (int start = 0; start < s.nq;) {
+    bool moved = false;
+    for (int e = 0; e < s.p.ne; ++e) {
+      const int a = sys->couplings[e].a, b = sys->couplings[e].b, x = rt.e_pa[e] ^ rt.e_pb[e];
+      if (f[a] >= 0 && f[b] >= 0) {
+        if ((f[a] ^ f[b]) != x) return false;
+      } else if (f[a] >= 0 || f[b] >= 0) {
+        (f[a] >= 0 ? f[b] : f[a]) = (f[a] >= 0 ? f[a] : f[b]) ^ x;
+        moved = true;
+      }
+    }
+    if (moved) continue;
+    while (start < s.nq && f[start] >= 0) ++start;
+    if (start < s.nq) f[start] = 0;
+  }
+  rt.flip = 0;
+  for (int i = 0; i < s.nq; ++i) rt.flip |= (unsigned)f[i] << i;
+  return true;
 }
 
 sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, bool grad) {
@@ -1810,9 +1852,9 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
   // a solve goes before its first kernel (see dcopy)
   sv.mixed = o->precision == SG_MIXED;
   const int pc = path_choice();
-  sv.real_oc = !s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows && real_terms(sys, s, s.ta);
-  if (sv.real_oc) {
+  if (!s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows) {
     fill_terms(s, s.ta, sv.rterms);
+    sv.real_oc = real_gauge(sys, s, sv.rterms);
   }
   if (pc == 0)
     sv.oc = onchip_plan_create(s.p, sv.mixed, s.K, s.sumd, st, sv.real_oc ? &sv.rterms : nullptr, sv.two_rows);
@@ -2055,7 +2097,12 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     const int nD = sv.ocp && onchip_forward_ok(sv.ocp) ? onchip_fwd_ctas(sv.ocp) : 0;
     const int most = nD ? 152 * onchip_fwd_resident(sv.ocp) / nD : 0;
     if (most >= kMinSide) {
-      c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + most - 1) / most);
+      // A gradient's chunks are also recomputed and pulled back with S columns, which take fewer CTAs:
+      // more chunks than propagators fit at once (whole rounds of them, up to 8) until those fill
+      // the SMs.  D = 64 FP64, 4 columns: 57 chunks 26.5 ms (2 x 8.1 ms of passes with 57 CTAs), 456
+      // chunks 14.1 ms.
+      const int rounds = grad ? std::max(1, std::min(8, slots / most)) : 1;
+      c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + rounds * most - 1) / (rounds * most));
       c.C = (N + c.L - 1) / c.L;
       c.prop = c.par = c.C > 1;
       c.R = grad ? fit_rounds(c.C, c.L) : 1;
@@ -2074,13 +2121,20 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     }
   }
   if (!grad) return;
+  // The two serial passes run side by side when the SMs hold both and every computational row has
+  // an image column: D = 3125 with 32 columns takes 32 CTAs each way (1000 steps with their
+  // gradient: 62 -> 40.6 ms, of which the sums over the basis take 3.5).
+  const bool basis = real && sv.barc && onchip_mix_ok(sv.oc, s.Dc) &&
+                     2 * onchip_fwd_ctas(sv.oc) <= 152 * onchip_fwd_resident(sv.oc);
   // real operators: the two serial passes keep all stage inputs when there is room
   if (real && ckpt <= 0 && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
     c.direct = true;
+    c.basis = basis;
     return;
   }
   // boundary states by serial passes; segments of L steps
   if (slots > 1 && N > kMinChunk) {
+    c.basis = basis;
     if (ckpt > 0) {
       c.L = std::min(ckpt, N);
     } else {
@@ -2108,7 +2162,8 @@ sg_status alloc_chunks(sg_ctx* ctx, Solve& sv, int ckpt) {
   if (sv.ch.direct) {
     const size_t n = (size_t)4 * sv.s.N * onchip_state_elems(sv.oc);
     sv.ch.segU = sv.mixed ? (void*)sv.ar.get<float2>(n) : (void*)sv.ar.get<double2>(n);
-    if (!sv.ch.segU) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the stage inputs failed");
+    sv.ch.segK = sv.mixed ? (void*)sv.ar.get<float2>(n) : (void*)sv.ar.get<double2>(n);
+    if (!sv.ch.segU || !sv.ch.segK) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the stage inputs failed");
   }
   return SG_OK;
 }
@@ -2142,6 +2197,19 @@ void chunk_products(Solve& sv, const double2* start, double2* states, double2* l
 }
 
 // sv.psi evolved in place; with sv.ch.ck, the states before every chunk kept.
+FrameArgs frame_args(const Setup& s, const double* E_dev, double sign);
+CompArgs comp_args(const Setup& s);
+
+__global__ void k_unit(int n, double2* u) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * n; i += gridDim.x * blockDim.x)
+    u[i] = make_double2(i % (n + 1) == 0 ? 1.0 : 0.0, 0.0);
+}
+// API layout (D x S) -> columns of D entries
+__global__ void k_columns(long long D, int S, const double2* __restrict__ api, double2* __restrict__ col) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < D * S; i += (long long)gridDim.x * blockDim.x)
+    col[i] = api[(i % D) * S + i / D];
+}
+
 template <typename R>
 OnchipRealTables real_tables(const Solve& sv) {
   OnchipRealTables r;
@@ -2167,7 +2235,37 @@ sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
     f.ck_out = c.direct ? nullptr : c.ck;
     f.segY = c.segU;
     f.K = c.L;
-    sv.launches += onchip_forward(sv.oc, f, 0, s.N, s.N, s.dt, st);
+    if (c.basis && (c.par || c.direct)) {
+      // unit vectors on the computational rows, in the frame, as co-states at the end
+      const long long n = s.D * s.S, ns = onchip_state_elems(sv.oc);
+      double2* unit = sv.ar.get<double2>((size_t)s.Dc * s.Dc);
+      double2* api = sv.ar.get<double2>((size_t)s.D * s.Dc);
+      double2* img = sv.ar.get<double2>((size_t)ns);
+      if (!c.direct) c.lam = sv.ar.get<double2>((size_t)c.C * ns);
+      if (!unit || !api || !img || (!c.direct && !c.lam))
+        return sg_fail(ctx, SG_E_NOMEM, "device allocation of the co-state basis failed");
+      (void)n;
+      SG_CUDA_TRY(ctx, cudaMemsetAsync(api, 0, (size_t)s.D * s.Dc * sizeof(double2), st));
+      SG_CUDA_TRY(ctx, cudaMemsetAsync(img, 0, (size_t)ns * sizeof(double2), st));
+      CompArgs ca = comp_args(s);
+      ca.S = s.Dc;
+      FrameArgs fr = frame_args(s, sv.E_dev, +1.0);
+      fr.S = s.Dc;
+      k_unit<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(s.Dc, unit);
+      k_scatter_comp<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(ca, unit, api);
+      k_frame<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(fr, api);
+      k_columns<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(s.D, s.Dc, api, img);
+      OnchipForward b;
+      b.rt = f.rt;
+      b.rev = true;
+      b.img_in = img;
+      b.segY = c.segK;
+      b.ck_out = c.direct ? nullptr : c.lam;
+      b.K = c.L;
+      sv.launches += 4 + onchip_forward_pair(sv.oc, f, b, s.N, s.dt, st);
+    } else {
+      sv.launches += onchip_forward(sv.oc, f, 0, s.N, s.N, s.dt, st);
+    }
     SG_CUDA_TRY(ctx, cudaGetLastError());
     return SG_OK;
   }
@@ -2318,10 +2416,11 @@ sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc ac
   const size_t naccd = (size_t)blocks * onchip_acc_doubles(oc), nseg = (size_t)4 * c.R * c.L * ns;
   double2* pimg = sv.ar.get<double2>(ns);
   C* segU = c.direct ? static_cast<C*>(c.segU) : sv.ar.get<C>(nseg);
-  C* segK = sv.ar.get<C>(nseg);
+  C* segK = c.direct ? static_cast<C*>(c.segK) : sv.ar.get<C>(nseg);
   double* gFc = sv.ar.get<double>((size_t)groups * nstK);
   double* accc = sv.ar.get<double>(naccd);
-  c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
+  const bool basis = c.basis && (c.par || c.direct);
+  if (!(basis && c.par)) c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
   double2* gimg = c.prop ? sv.ar.get<double2>((size_t)c.NG * ns) : pimg;
   if (!pimg || !segU || !segK || !gFc || !accc || !c.lam || !gimg)
     return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
@@ -2333,7 +2432,12 @@ sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc ac
   f.rt = real_tables<R>(sv);
   OnchipForward b = f;
   b.rev = true;
-  if (c.prop) {
+  if (basis) {
+    // the pulled-back basis becomes the co-states: their stage inputs, or their boundary values
+    SG_CUDA_TRY(ctx, onchip_mix(oc, c.direct ? (void*)segK : (void*)c.lam, c.direct && sizeof(R) == 4,
+                                c.direct ? 4ll * s.N : c.C, sv.barc, s.Dc, st));
+    ++sv.launches;
+  } else if (c.prop) {
     chunk_products(sv, pimg, c.lam, nullptr, gimg, true, st);
   } else if (c.par) {
     b.img_in = pimg;
@@ -2352,7 +2456,7 @@ sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc ac
     b.img_in = c.par ? c.lam + (size_t)c0 * ns : pimg;
     b.img_out = c.par ? nullptr : pimg;                 // one after the other: handed on
     b.segY = segK;
-    sv.launches += onchip_forward(oc, b, n0, n1, c.L, s.dt, st);
+    if (!(basis && c.direct)) sv.launches += onchip_forward(oc, b, n0, n1, c.L, s.dt, st);
     if (c0 == 0) onchip_batcher_release();              // the solve's last on-chip launch is issued
     sv.launches += ocr_densities(rp, segU, segK, f.rt.coef, sv.opd_dev, sv.J_dev, n0, n1, s.dt, sv.want_ham, nstK, gFc,
                                  accc, st);
@@ -2896,6 +3000,7 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
   // checkpoints
   int K = 0;
   std::vector<double2*> ckpts;
+  if (grad && !dressed) sv.barc = barc;
   if (!grad && !s.q2 && sv.onchip(false)) plan_chunks(sv, false, 0, ctx->work_limit);
   if (grad && !s.q2) {             // the Q2 adjoint recomputes the states by inverse factors
     K = ckpt > 0 ? ckpt : std::max(1, (int)std::lround(std::sqrt((double)s.N)));

@@ -832,6 +832,56 @@ __global__ void k_oc_api(OcArgs oa, const double2* __restrict__ img, double2* __
   }
 }
 
+// Images of columns j -> images of columns s, out_s = sum_j W[j][s] in_j, in place: a block owns
+// kMixT entries of all columns of one image, read into shared memory before it writes.  A thread
+// takes two entries and four columns at a time, so 32 multiply-adds share six loads.
+constexpr int kMixT = 64, kMixMax = 64;      // entries per block; columns at most
+template <typename C>
+__global__ void __launch_bounds__(256) k_oc_mix(C* __restrict__ img, const double2* __restrict__ W, int nin, int nout,
+                                                int cols, int D) {
+  typedef decltype(C().x) R;
+  extern __shared__ __align__(16) unsigned char msm[];
+  C* const in = reinterpret_cast<C*>(msm);               // nin x kMixT
+  C* const w = in + nin * kMixT;                         // nin x out4
+  const int out4 = (nout + 3) / 4 * 4, tid = threadIdx.x;
+  C* const base = img + (size_t)blockIdx.y * cols * D;
+  const int t0 = blockIdx.x * kMixT, nt = min(kMixT, D - t0);
+  for (int i = tid; i < nin * out4; i += blockDim.x) {
+    const int j = i / out4, s = i - j * out4;
+    const double2 v = s < nout ? W[(size_t)j * nout + s] : make_double2(0.0, 0.0);
+    w[i] = cmk<C>(v.x, v.y);
+  }
+  for (int i = tid; i < nin * kMixT; i += blockDim.x) {
+    const int j = i / kMixT, t = i - j * kMixT;
+    in[i] = t < nt ? base[(size_t)j * D + t0 + t] : cmk<C>(0.0, 0.0);
+  }
+  __syncthreads();
+  const int lane = tid & 31, g = tid >> 5, ng = blockDim.x >> 5;
+  for (int s0 = 4 * g; s0 < cols; s0 += 4 * ng) {
+    C a[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k][0] = a[k][1] = cmk<C>(0.0, 0.0);
+    if (s0 < nout)
+      for (int j = 0; j < nin; ++j) {
+        const C x0 = in[j * kMixT + lane], x1 = in[j * kMixT + lane + 32];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const C v = w[j * out4 + s0 + k];
+          a[k][0] = cfma(v, x0, a[k][0]);
+          a[k][1] = cfma(v, x1, a[k][1]);
+        }
+      }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int t = lane + 32 * e;
+        if (s0 + k < cols && t < nt) base[(size_t)(s0 + k) * D + t0 + t] = a[k][e];
+      }
+  }
+  (void)sizeof(R);
+}
+
 // FP64 -> FP32 copy of the per-stage phase and coefficient tables and the operators.
 __global__ void k_oc_f32(const double* __restrict__ src, float* __restrict__ dst, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -1417,7 +1467,9 @@ int submit(const OcPending& p, cudaStream_t st) {
 
 }  // namespace
 
-int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st) {
+namespace {
+
+OcPending forward_of(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt) {
   OcPending p{};
   p.kind = oc->real && !f.rows ? 2 : 0;
   p.oc = oc;
@@ -1441,7 +1493,24 @@ int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1,
   p.d.C = (n1 - n0 + p.d.L - 1) / p.d.L;
   p.d.ident = f.ident ? 1 : 0;
   p.d.rev = f.rev ? 1 : 0;
-  return submit(p, st);
+  return p;
+}
+
+}  // namespace
+
+int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st) {
+  return submit(forward_of(oc, f, n0, n1, L, dt), st);
+}
+
+int onchip_forward_pair(const OnchipPlan* oc, const OnchipForward& f, const OnchipForward& b, int N, double dt,
+                        cudaStream_t st) {
+  const OcPending p = forward_of(oc, f, 0, N, N, dt), q = forward_of(oc, b, 0, N, N, dt);
+  if (tl_batcher) return submit(p, st) + submit(q, st);
+  OcBatch bt{};
+  bt.nsys = 2;
+  bt.s[0] = p.d;
+  bt.s[1] = q.d;
+  return oc_launch(oc, p.kind, bt, dt, nullptr, st);
 }
 
 int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* lam, int n0, int n1,
@@ -1653,6 +1722,24 @@ void onchip_to_image(const OnchipPlan* oc, const double2* api, double2* img, cud
 
 void onchip_from_image(const OnchipPlan* oc, const double2* img, double2* api, cudaStream_t st) {
   k_oc_api<<<grid_of((long long)oc->oa.S * oc->oa.D), 256, 0, st>>>(oc->oa, img, api);
+}
+
+bool onchip_mix_ok(const OnchipPlan* oc, int nin) {
+  return nin <= kMixMax && oc->oa.S <= kMixMax && nin <= oc->oa.ncta * oc->oa.Sc;
+}
+
+cudaError_t onchip_mix(const OnchipPlan* oc, void* img, bool f32, long long nimg, const double2* W, int nin,
+                       cudaStream_t st) {
+  const int D = oc->oa.D, S = oc->oa.S, cols = oc->oa.ncta * oc->oa.Sc, out4 = (S + 3) / 4 * 4;
+  const size_t smem = (size_t)nin * (kMixT + out4) * (f32 ? sizeof(float2) : sizeof(double2));
+  smem_limit_once<k_oc_mix<float2>>();
+  smem_limit_once<k_oc_mix<double2>>();
+  for (long long i = 0; i < nimg; i += 65535) {                 // the grid's second dimension
+    const dim3 grid((D + kMixT - 1) / kMixT, (unsigned)std::min<long long>(65535, nimg - i));
+    if (f32) k_oc_mix<<<grid, 256, smem, st>>>(static_cast<float2*>(img) + i * cols * D, W, nin, S, cols, D);
+    else k_oc_mix<<<grid, 256, smem, st>>>(static_cast<double2*>(img) + i * cols * D, W, nin, S, cols, D);
+  }
+  return cudaGetLastError();
 }
 
 int onchip_columns(const OnchipPlan* oc) { return oc->oa.ncta * oc->oa.Sc; }

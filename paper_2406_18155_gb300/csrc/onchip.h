@@ -69,6 +69,15 @@ struct OnchipForward {
   bool rows = false;              // the complex-row kernels, also where the plan is real
 };
 int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1, int L, double dt, cudaStream_t st);
+// f and b over all N steps side by side in one launch (serial passes that do not wait for one
+// another: the states, and co-states of a basis).
+int onchip_forward_pair(const OnchipPlan* oc, const OnchipForward& f, const OnchipForward& b, int N, double dt,
+                        cudaStream_t st);
+// nimg images of nin columns -> of the plan's columns in place, out_s = sum_j W[j][s] in_j (W: nin x
+// S, device; padding columns become zero); f32: complex64 images, else complex128.
+bool onchip_mix_ok(const OnchipPlan* oc, int nin);
+cudaError_t onchip_mix(const OnchipPlan* oc, void* img, bool f32, long long nimg, const double2* W, int nin,
+                       cudaStream_t st);
 // CTAs of the forward (adjoint) launch that one SM holds at once.
 int onchip_fwd_resident(const OnchipPlan* oc);
 int onchip_adj_resident(const OnchipPlan* oc);

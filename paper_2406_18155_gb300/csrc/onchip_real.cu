@@ -60,15 +60,18 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
     P.mR = P.mL = P.expR = P.mR2 = P.mL2 = P.mE = P.expL = P.bA = P.bB = -1;
   }
   for (int i = 0; i < nq; ++i) a.eoff[i] = t.eoff[i];
+  a.flip = t.flip;
+  auto flip = [&](int mode) { return (int)((t.flip >> mode) & 1u); };
   auto matrix = [&](int mode, int op, int part, int J) {
     const int off = t.opd_off[mode] + op * DL * DL;
     for (int m = 0; m < a.nmat; ++m)
-      if (a.m_off[m] == off && a.m_part[m] == part && a.m_J[m] == J) return m;
+      if (a.m_off[m] == off && a.m_J[m] == J) return m;
     if (a.nmat == kRMat) return -1;
     a.m_off[a.nmat] = off;
     a.m_part[a.nmat] = part;
+    a.m_flip[a.nmat] = flip(mode);
     a.m_J[a.nmat] = J;
-    a.m_sign[a.nmat] = J >= 0 && part ? -1 : 1;     // i A (x) i B = -A (x) B
+    a.m_sign[a.nmat] = J >= 0 && (part ^ flip(mode)) ? -1 : 1;     // i A (x) i B = -A (x) B
     return a.nmat++;
   };
   auto phase_of = [&](int i, int j) {                // a phase that holds both modes, the last such
@@ -82,7 +85,8 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
     if (q < 0) continue;
     const bool fwd = p.e_a[e] == pm[q][0];
     const int opl = fwd ? t.e_opa[e] : t.e_opb[e], opr = fwd ? t.e_opb[e] : t.e_opa[e];
-    const int L = matrix(pm[q][0], opl, t.e_part[e], e), Rm = matrix(pm[q][1], opr, t.e_part[e], -1);
+    const int L = matrix(pm[q][0], opl, fwd ? t.e_pa[e] : t.e_pb[e], e);
+    const int Rm = matrix(pm[q][1], opr, fwd ? t.e_pb[e] : t.e_pa[e], -1);
     OcrPhase& P = a.ph[q];
     if (L < 0 || Rm < 0) return give_up();
     if (P.mR < 0) { P.mR = Rm; P.mL = L; }
@@ -113,7 +117,8 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
       if (src != q) continue;
       const int ms = a_first ? p.e_a[e] : p.e_b[e], md = a_first ? p.e_b[e] : p.e_a[e];
       const int ops = a_first ? t.e_opa[e] : t.e_opb[e], opd = a_first ? t.e_opb[e] : t.e_opa[e];
-      const int mat = matrix(ms, ops, t.e_part[e], -1), mJ = matrix(md, opd, t.e_part[e], e);
+      const int mat = matrix(ms, ops, a_first ? t.e_pa[e] : t.e_pb[e], -1);
+      const int mJ = matrix(md, opd, a_first ? t.e_pb[e] : t.e_pa[e], e);
       if (mat < 0 || mJ < 0) return give_up();
       const bool right = ms == pm[q][1];
       Need* n = nullptr;
@@ -163,6 +168,7 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
       if (pm[q][1] == p.s1_mode[u] && P.bB < 0) { P.bB = u; break; }
     }
     a.d_start[u] = t.drv_start[u];
+    a.d_flip[u] = flip(p.s1_mode[u]);
     for (int x = t.drv_start[u]; x < t.drv_start[u + 1]; ++x) {
       a.d_drv[x] = t.drv_list[x];
       a.d_off[x] = t.opd_off[p.s1_mode[u]] + t.drv_op[t.drv_list[x]] * DL * DL;
@@ -222,8 +228,9 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
     if (g.nmat == kRMat) { fits = false; return 0; }
     g.m_off[g.nmat] = t.opd_off[mode] + op * DL * DL;
     g.m_part[g.nmat] = part;
+    g.m_flip[g.nmat] = flip(mode);
     g.m_J[g.nmat] = J;
-    g.m_sign[g.nmat] = part ? -1 : 1;
+    g.m_sign[g.nmat] = part ^ flip(mode) ? -1 : 1;
     return g.nmat++;
   };
   for (int u = 0; u < p.n1 && fits; ++u)
@@ -234,6 +241,7 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
       S->drv = t.drv_list[x];
       S->mslot = u;
       S->off = t.opd_off[i] + t.drv_op[S->drv] * DL * DL;
+      S->part = S->flip = flip(i);
       lay(*S, i, i ? i - 1 : 1);
     }
   const int ndrv = g.nslot;
@@ -245,10 +253,11 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
       S->kind = 1;
       S->edge = e;
       S->side = side;
-      S->part = t.e_part[e];
-      S->sign = S->part ? -1 : 1;
+      S->part = side ? t.e_pb[e] : t.e_pa[e];
+      S->flip = flip(i);
+      S->sign = S->part ^ S->flip ? -1 : 1;
       S->off = t.opd_off[i] + (side ? t.e_opb[e] : t.e_opa[e]) * DL * DL;
-      S->mat = dmat(j, side ? t.e_opa[e] : t.e_opb[e], t.e_part[e], side ? e : -1);
+      S->mat = dmat(j, side ? t.e_opa[e] : t.e_opb[e], side ? t.e_pa[e] : t.e_pb[e], side ? e : -1);
       lay(*S, i, j);
     }
   if (fits) {
@@ -285,7 +294,7 @@ void ocr_signature(const OcrPlan* o, std::vector<long long>& sig) {
   const OcrArgs& a = o->a;
   sig.push_back(a.nmat);
   for (int m = 0; m < a.nmat; ++m) {
-    sig.push_back(a.m_off[m]); sig.push_back(a.m_part[m]); sig.push_back(a.m_J[m]);
+    sig.push_back(a.m_off[m]); sig.push_back(a.m_part[m]); sig.push_back(a.m_flip[m]); sig.push_back(a.m_J[m]);
   }
   for (int u = 0; u < a.n1; ++u)
     for (int x = a.d_start[u]; x < a.d_start[u + 1]; ++x) { sig.push_back(a.d_drv[x]); sig.push_back(a.d_off[x]); }

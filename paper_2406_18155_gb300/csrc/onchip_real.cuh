@@ -3,7 +3,9 @@
 //
 // In the interaction picture H_I(t) = P(t) H(t) P(t)^dag with P = diag exp(i E t) and
 // H(t) = sum_k f_k(t) O_k + sum_e J_e A_e (x) B_e, whose matrices are real and constant (a
-// coupling of two imaginary factors is -J Im A (x) Im B).  The complex-row kernels
+// coupling of two imaginary factors is -J Im A (x) Im B; where a real factor meets an imaginary
+// one, as a transmon's charge and a fluxonium's, turning the odd levels of one mode by i makes
+// them alike, OcrTerms::flip).  The complex-row kernels
 // (onchip.cu) form every matrix of H_I(t) per stage and multiply complex by complex.  Here
 // the stage inputs are kept as u = P(t)^dag y: between two half steps P changes by the constant
 // diagonal Q = exp(-i E h/2), so one RK4 step from psi (interaction picture, P_m = P at the
@@ -111,10 +113,11 @@ struct OcrArgs {
   int K, sumd, sumdA, n1, nmat;
   OcrPhase ph[3];
   int eoff[SG_MAXQ];              // level offsets of the modes in a phase row
+  unsigned flip;                  // modes whose odd levels are turned by i
   // constant matrices: element (x, c) is part of opd[off + x d + c], times sign, times J
-  int m_off[kRMat], m_part[kRMat], m_sign[kRMat], m_J[kRMat];
+  int m_off[kRMat], m_part[kRMat], m_flip[kRMat], m_sign[kRMat], m_J[kRMat];
   // one-body slots: drives and their operators
-  int d_start[SG_MAXQ + 1], d_drv[SG_MAXDRIVE], d_off[SG_MAXDRIVE];
+  int d_start[SG_MAXQ + 1], d_drv[SG_MAXDRIVE], d_off[SG_MAXDRIVE], d_flip[SG_MAXQ];
   // shared-memory byte offsets
   int s_img, s_psi, s_b, s_acc, s_Q, s_mat, s_one, s_ph;
 };
@@ -123,7 +126,7 @@ constexpr int kRSlot = 16;        // slots per CTA (warps)
 struct OcdSlot {
   int kind;                       // 0 one-body, 1 side of a coupling
   int drv, mslot, edge, side;     // kind 0: drive and 1-body slot; kind 1: coupling and side
-  int off, part, sign;            // the slot's own operator: opd offset, part; sign of i A (x) i B
+  int off, part, flip, sign;      // the slot's own operator: opd offset, part; sign of i A (x) i B
   int mat;                        // kind 1: the other factor's matrix (J included on side 1)
   int s1, s2;                     // image strides of the slot's digit and of its partner
   int no, pst[4];
@@ -133,7 +136,7 @@ struct OcdArgs {
   int nslot, nmat, ni;            // slots; matrices; images per load (1, or whole steps)
   long long accd, nstK;
   OcdSlot slot[kRSlot];
-  int m_off[kRMat], m_part[kRMat], m_sign[kRMat], m_J[kRMat];
+  int m_off[kRMat], m_part[kRMat], m_flip[kRMat], m_sign[kRMat], m_J[kRMat];
   int s_img, s_mat, s_g;
 };
 struct OcdJob {
@@ -177,6 +180,13 @@ namespace {
 // the columns of row x that a parity-odd matrix keeps: c = zc(x, 0 .. zn(x) - 1)
 template <int DL> __host__ __device__ constexpr int zn(int x) { return x & 1 ? (DL + 1) / 2 : DL / 2; }
 __host__ __device__ constexpr int zc(int x, int j) { return 2 * j + (x & 1 ? 0 : 1); }
+
+// The real matrix element in row x of an operator whose `part` holds it, in a basis turned by
+// g = i on the odd levels (flip): conj(g_x) X_xc g_c for a parity-odd X = m or i m.
+__device__ __forceinline__ double r_sign(int part, int flip, int x) { return flip && ((x & 1) ^ part) ? -1.0 : 1.0; }
+__device__ __forceinline__ double r_elem(double2 o, int part, int flip, int x) {
+  return r_sign(part, flip, x) * (part ? o.y : o.x);
+}
 
 __device__ __forceinline__ float2 zdup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ double zdup(double v) { return v; }
@@ -306,7 +316,8 @@ __device__ __forceinline__ void one_body(const OcrArgs& a, const R* __restrict__
   R v = f0 * o0;
   if (j < zn<DL>(x))
     for (int k = a.d_start[u] + 1; k < a.d_start[u + 1]; ++k)
-      v += coef[(size_t)q * a.K + a.d_drv[k]] * (R)opd[a.d_off[k] + x * DL + zc(x, j)].x;
+      v += coef[(size_t)q * a.K + a.d_drv[k]] *
+           (R)r_elem(opd[a.d_off[k] + x * DL + zc(x, j)], a.d_flip[u], a.d_flip[u], x);
   one[i] = zdup(v);
 }
 
@@ -383,7 +394,7 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
     double v = 0.0;
     if (j < zn<DL>(x)) {
       const double2 o = d.opd64[a.m_off[m] + x * DL + zc(x, j)];
-      v = a.m_part[m] ? o.y : o.x;
+      v = r_elem(o, a.m_part[m], a.m_flip[m], x);
       if (a.m_J[m] >= 0) v *= d.J[a.m_J[m]] * a.m_sign[m];
     }
     mat[i] = zdup((R)v);
@@ -402,7 +413,7 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
       const int k = a.d_start[u];
       if (k < a.d_start[u + 1] && j < zn<DL>(x)) {
         k0[e] = a.d_drv[k];
-        o0[e] = (R)d.opd64[a.d_off[k] + x * DL + zc(x, j)].x;
+        o0[e] = (R)r_elem(d.opd64[a.d_off[k] + x * DL + zc(x, j)], a.d_flip[u], a.d_flip[u], x);
       }
     }
   }
@@ -446,9 +457,19 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
   auto phases = [&](const C* row, C (&pa)[DL]) {
     C f = cmk<C>(1.0, 0.0);
 #pragma unroll
-    for (int j = 0; j < NO; ++j) f = cmulT(f, row[a.eoff[Y::other(NP - 1, j)] + dig[j]]);
+    for (int j = 0; j < NO; ++j) {
+      f = cmulT(f, row[a.eoff[Y::other(NP - 1, j)] + dig[j]]);
+      if (((a.flip >> Y::other(NP - 1, j)) & 1u) && (dig[j] & 1)) f = cmk<C>(-f.y, f.x);
+    }
 #pragma unroll
-    for (int x = 0; x < DL; ++x) pa[x] = cmulT(f, row[a.eoff[MA] + x]);
+    for (int x = 0; x < DL; ++x) {
+      pa[x] = cmulT(f, row[a.eoff[MA] + x]);
+      if ((x & 1) && ((a.flip >> MA) & 1u)) pa[x] = cmk<C>(-pa[x].y, pa[x].x);
+    }
+  };
+  auto phase_b = [&](const C* row, int z) {
+    const C p = row[a.eoff[MA + 1] + z];
+    return (z & 1) && ((a.flip >> (MA + 1)) & 1u) ? cmk<C>(-p.y, p.x) : p;
   };
   C u[DL][DL];
   // b = P_m^dag psi, u = Q^dag b
@@ -460,7 +481,7 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
 #pragma unroll
       for (int z = 0; z < DL; ++z) {
         const int e = x * DL + z;
-        const C p = cmulT(pa[x], row[a.eoff[MA + 1] + z]);
+        const C p = cmulT(pa[x], phase_b(row, z));
         const C b = cmulT(cconjT(p), ps.hi(e * nthr));
         bv.set(e, b);
         const C w = cmulT(cconjT(Q.get(e)), b);
@@ -551,7 +572,7 @@ k_ocr_fwd(const __grid_constant__ OcrArgs a, double dt, const __grid_constant__ 
           for (int x = 0; x < DL; ++x)
 #pragma unroll
             for (int z = 0; z < DL; ++z)
-              ps.add((x * DL + z) * nthr, cmulT(cmulT(pa[x], prow[a.eoff[MA + 1] + z]), u[x][z]));
+              ps.add((x * DL + z) * nthr, cmulT(cmulT(pa[x], phase_b(prow, z)), u[x][z]));
           if (i + 1 < nsteps) begin_step(pnext);
         }
       }
@@ -609,7 +630,7 @@ k_ocr_dens(const __grid_constant__ OcdArgs a, const __grid_constant__ OcdJob jb)
     double v = 0.0;
     if (j < zn<DL>(x)) {
       const double2 o = jb.opd[a.m_off[m] + x * DL + zc(x, j)];
-      v = a.m_part[m] ? o.y : o.x;
+      v = r_elem(o, a.m_part[m], a.m_flip[m], x);
       if (a.m_J[m] >= 0) v *= jb.J[a.m_J[m]] * a.m_sign[m];
     }
     mat[i] = zdup((R)v);
@@ -625,7 +646,7 @@ k_ocr_dens(const __grid_constant__ OcdArgs a, const __grid_constant__ OcdJob jb)
 #pragma unroll
       for (int j = 0; j < zn<DL>(x); ++j, ++p) {
         const double2 o = jb.opd[S.off + x * DL + zc(x, j)];
-        own[p] = (R)(S.part ? o.y : o.x);
+        own[p] = (R)r_elem(o, S.part, S.flip, x);
       }
   }
   R aI[NPR], aR[NPR];
@@ -802,10 +823,10 @@ k_ocr_dens(const __grid_constant__ OcdArgs a, const __grid_constant__ OcdJob jb)
         for (int j = 0; j < zn<DL>(x); ++j, ++p) {
           const int y = zc(x, j);
           const double2 o = jb.opd[S.off + x * DL + y];
-          const double m = S.part ? o.y : o.x;
+          const double m = r_elem(o, S.part, S.flip, x);
           // side 1's matrix carries J and the sign already
           const double s1 = S.kind && S.side == 1 ? 1.0 : sc;
-          ob[2 * (x * SG_MAXD + y) + (S.part ? 1 : 0)] += s1 * eI[p];
+          ob[2 * (x * SG_MAXD + y) + (S.part ? 1 : 0)] += r_sign(S.part, S.flip, x) * s1 * eI[p];
           eb[x] += s1 * m * eR[p];
           eb[y] -= s1 * m * eR[p];
           dj += m * eI[p];

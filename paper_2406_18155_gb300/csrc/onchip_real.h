@@ -13,7 +13,12 @@ struct OcrTerms {
   int drv_start[SG_MAXQ + 1] = {0}, drv_list[SG_MAXDRIVE] = {0};   // drives of each 1-body slot
   int drv_op[SG_MAXDRIVE] = {0};
   int e_opa[SG_MAXEDGE] = {0}, e_opb[SG_MAXEDGE] = {0};
-  int e_part[SG_MAXEDGE] = {0};                      // 0: real factors, 1: imaginary factors
+  // Which part of an operator holds its real matrix (0 real, 1 imaginary), per coupling side,
+  // and the modes whose basis is turned by i on odd levels: a parity-odd operator then changes
+  // its part, so that drives are real and the two factors of a coupling alike (a drive's
+  // part is its mode's flip).
+  int e_pa[SG_MAXEDGE] = {0}, e_pb[SG_MAXEDGE] = {0};
+  unsigned flip = 0;
 };
 
 struct OcrPlan;   // opaque

@@ -83,8 +83,40 @@ def test_real_gradient_matches_the_general_kernels(sgctx, monkeypatch, name):
         assert np.max(np.abs(pulse[1] - gp)) <= 1e-8 * scale
 
 
+def _charge_driven():
+    # charge drives (imaginary on a fluxonium) on two of three modes, n (x) n and n (x) phi couplings
+    wl = _workload("triangle_l4", steps=9)
+    wl["couplings"][1]["op_b"] = "phi"
+    wl["couplings"] = wl["couplings"][:2]
+    for d in wl["drives"][:2]:
+        d["op"] = "n"
+    wl["drives"] = wl["drives"][:2]
+    return wl
+
+
+@pytest.mark.parametrize("make", [lambda: W.coupler_scheme(seed=2, kind="ftf", T=0.09),
+                                  lambda: W.coupler_scheme(seed=3, kind="ftf", T=0.09, levels=(3, 3, 3)),
+                                  _charge_driven])
+def test_turned_modes_match_the_general_kernels(sgctx, monkeypatch, make):
+    # a real factor against an imaginary one: a mode's odd levels are turned by i
+    from paper_2406_18155_gb300.api import System
+    wl = make()
+    s = System.from_workload(sgctx, wl)
+    s.prepare()
+    args = (wl["T"], wl["dt"], wl["target"], wl["col_index"])
+    got = {p: (s.evolve(wl["T"], wl["dt"], precision=p, col_index=wl["col_index"]).cpu().numpy(),
+               s.fidelity_grad(*args, kind="state", precision=p)) for p in ("fp64", "mixed")}
+    monkeypatch.setenv("SG_PATH", "gather")
+    ref = s.evolve(wl["T"], wl["dt"], precision="fp64", col_index=wl["col_index"]).cpu().numpy()
+    F, gp, gh = s.fidelity_grad(*args, kind="state", precision="fp64")
+    g = np.concatenate([gp, gh])
+    for p, (psi, (f, a, b)) in got.items():
+        ta, tg = (1e-10, 1e-8) if p == "fp64" else (1e-5, 1e-3)
+        assert np.max(np.abs(psi - ref)) <= ta and abs(f[1] - F[1]) <= ta, p
+        assert np.max(np.abs(np.concatenate([a, b]) - g)) <= tg * np.max(np.abs(g)), p
+
+
 @pytest.mark.parametrize("make", [
-    lambda: W.coupler_scheme(seed=2, kind="ftf", T=0.2),              # a real factor against an imaginary one
     lambda: W.local_op_pair(seed=3, T=0.2),                           # complex operators without parity
     lambda: dict(W.transmon_pair(seed=4, T=0.2), modes=[dict(m, ng=0.2) for m in W.transmon_pair(seed=4)["modes"]]),
 ])
