@@ -3704,7 +3704,7 @@ sg_status sg_evolve_batch_impl(sg_system* const* systems, int B, const sg_evolve
   // Pairs of modes that put at least half a warp of columns to work run on the real-operator
   // on-chip kernel, one warp per system with a thread per column, all systems in one launch:
   // its structured products are 1/8 of the dense ones' arithmetic and nothing is exchanged.  512
-  // transmon pairs (D = 16, 16 columns, 2000 steps): 36.3 ms dense, 12.0 ms.  Fewer columns
+  // transmon pairs (D = 16, 16 columns, 2000 steps): 36.3 ms dense, 10.5 to 13 ms here.  Fewer columns
   // leave lanes idle (D = 25, 4 columns: 4 of 32), and the tensor cores keep those.
   OcrPlan* rp = nullptr;
   struct PlanGuard { OcrPlan** p; ~PlanGuard() { ocr_plan_destroy(*p); } } guard{&rp};
