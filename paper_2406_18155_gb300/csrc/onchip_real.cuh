@@ -665,7 +665,8 @@ k_ocr_dens(const __grid_constant__ OcdArgs a, const __grid_constant__ OcdJob jb)
 #pragma unroll
   for (int p = 0; p < NPR; ++p) aI[p] = aR[p] = 0;
   // every kDensFlush images the warp's sums move to FP64, element p held by lane p (thousands of
-  // FP32 additions to one sum would cost digits that the next sums cancel against)
+  // FP32 additions to one sum would cost digits that the next sums cancel against; D = 3125, 1000
+  // steps: error of the Hamiltonian gradient 5.5e-7 -> 1.8e-7)
   double kI = 0.0, kR = 0.0;
   int since = 0;
   auto flush = [&]() {
