@@ -66,6 +66,7 @@ struct TabArgs {
   // its time-dependent terms at t_n + tau[j] dt (complex for Q4j) and its coupling
   // unitaries from set set_of[j]; set s has length setc[s] dt
   int nsub, nset;
+  int unit_ph;                // frame phases of modulus 1 on average (unit_cis32)
   int q1;                     // first-order product: full-step factors, each term once per step
   int set_of[3];
   double2 sc[3], tau[3], setc[3];
@@ -163,6 +164,24 @@ __device__ __forceinline__ float2 cis32(double theta) {
   return make_float2(cs, sn);
 }
 
+// |c|^2 - 1 of an FP32 cosine and sine, exact (p - 1 and its sum with small^2 are).  The two
+// FP32 functions give 1.8e-8 on average (2^24 arguments in [-pi, pi]), an error with one direction:
+// it adds up over the steps of a solve where it stays in the amplitudes or in the phases.
+__device__ __forceinline__ float cis_excess(float2 c) {
+  const float big = fmaxf(fabsf(c.x), fabsf(c.y)), small = fminf(fabsf(c.x), fabsf(c.y)), p = big * big;
+  return fmaf(small, small, p - 1.f) + fmaf(big, big, -p);
+}
+// exp(i theta) with modulus 1 on average, for the real-operator kernels, which turn the state by the
+// phases of all modes and back in every step.  The smaller part, whose rounding is finer, takes the
+// excess up; the angle moves by 2e-7 at most, either way.
+__device__ __forceinline__ float2 unit_cis32(double theta) {
+  const float2 c = cis32(theta);
+  const bool sw = fabsf(c.x) < fabsf(c.y);
+  const float big = sw ? c.y : c.x, small = sw ? c.x : c.y, m = cis_excess(c);
+  const float s = small - fminf(2e-7f, fmaxf(-2e-7f, small != 0.f ? 0.5f * m / small : 0.f));
+  return sw ? make_float2(s, big) : make_float2(big, s);
+}
+
 // Stage tables in FP32 only (mixed precision on the on-chip kernels, which read
 // nothing else): the same coefficients, phases and term rows as k_tables, with the
 // FP64 work cut to the envelope and the argument reduction.
@@ -175,12 +194,16 @@ __global__ void k_tables32(TabArgs a, float* __restrict__ coef32, float2* __rest
   for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
     const DriveDev dr = a.drives[k];
     const double E = envelope_dev(dr, a.amps, n, j, t);
-    const float v = (float)E * cis32(dr.omega * t + dr.phase).x;
+    // one rounding, of the product: the envelope's own would be constant over a segment
+    const float2 c = cis32(dr.omega * t + dr.phase);
+    const float v = (float)(E * (double)c.x * (1.0 - 0.5 * (double)cis_excess(c)));
     f[k] = v;
     coef32[(size_t)q * a.K + k] = v;
   }
   for (int i = threadIdx.x; i < a.sumd; i += blockDim.x) {
-    const float2 c = a.frame == SG_FRAME_INTERACTION ? cis32(a.E[i] * t) : make_float2(1.f, 0.f);
+    const float2 c = a.frame != SG_FRAME_INTERACTION ? make_float2(1.f, 0.f)
+                     : a.unit_ph                     ? unit_cis32(a.E[i] * t)
+                                                     : cis32(a.E[i] * t);
     ph[i] = c;
     ph32[(size_t)q * a.sumd + i] = c;
   }
@@ -1952,7 +1975,10 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
     // a forward evolution with real operators reads the coefficients and phases only
     const bool real = sv.onchip(grad) && onchip_real(sv.oc);
     TabArgs tt = ta;
-    if (real && (!grad || onchip_real_adjoint(sv.oc))) tt.p.n1 = tt.p.ne = 0;
+    if (real && (!grad || onchip_real_adjoint(sv.oc))) {
+      tt.p.n1 = tt.p.ne = 0;
+      tt.unit_ph = 1;
+    }
     if (f32only) k_tables32<<<(unsigned)nst, 64, 0, st>>>(tt, sv.coef32, sv.ph32);
     else k_tables<<<(unsigned)nst, 64, 0, st>>>(tt);
     if (real) {
@@ -3629,15 +3655,13 @@ __global__ void k_batch_phases(int B, int N, int sumd, double dt, const double* 
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long bn = i / sumd, b = bn / N;
     const int l = (int)(i - bn * sumd);
-    ph[i] = cis32(E[b * sumd + l] * ((double)(2 * (bn - b * N) + 1) * dt * 0.5));
+    ph[i] = unit_cis32(E[b * sumd + l] * ((double)(2 * (bn - b * N) + 1) * dt * 0.5));
   }
 }
 // e: composite energies, B x D
 __global__ void k_batch_half(long long n, double dt, const double* __restrict__ e, float2* __restrict__ half) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double sn, cs;
-    sincos(-0.5 * e[i] * dt, &sn, &cs);
-    half[i] = make_float2((float)cs, (float)sn);
+    half[i] = unit_phase32(-0.5 * e[i] * dt);
   }
 }
 // the lab frame: psi <- exp(-i e T) psi

@@ -12,9 +12,13 @@ __global__ void k_ocr_half(HalfArgs a, typename CT<R>::T* __restrict__ q) {
       e += a.E[a.eoff[i] + r % a.DL];
       r /= a.DL;
     }
-    double sn, cs;
-    sincos(-0.5 * e * a.dt, &sn, &cs);
-    q[t] = cmk<typename CT<R>::T>(cs, sn);
+    if constexpr (sizeof(R) == 4) {
+      q[t] = unit_phase32(-0.5 * e * a.dt);
+    } else {
+      double sn, cs;
+      sincos(-0.5 * e * a.dt, &sn, &cs);
+      q[t] = make_double2(cs, sn);
+    }
   }
 }
 
