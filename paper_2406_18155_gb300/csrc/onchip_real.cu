@@ -1,5 +1,7 @@
 // Real-operator on-chip solves: plans (how the terms are spread over the phases) and launches.
 #include "onchip_real.cuh"
+#include <cstring>
+#include <type_traits>
 
 namespace {
 
@@ -294,14 +296,12 @@ OcrPlan* ocr_plan_create(const KPlan& p, bool mixed, const OcrTerms& t, int cols
 void ocr_plan_destroy(OcrPlan* o) { delete o; }
 int ocr_ctas(const OcrPlan* o) { return o->a.ncta; }
 
+// Solves of equal signature share a launch, whose kernel reads the first one's arguments: all of them.
 void ocr_signature(const OcrPlan* o, std::vector<long long>& sig) {
-  const OcrArgs& a = o->a;
-  sig.push_back(a.nmat);
-  for (int m = 0; m < a.nmat; ++m) {
-    sig.push_back(a.m_off[m]); sig.push_back(a.m_part[m]); sig.push_back(a.m_flip[m]); sig.push_back(a.m_J[m]);
-  }
-  for (int u = 0; u < a.n1; ++u)
-    for (int x = a.d_start[u]; x < a.d_start[u + 1]; ++x) { sig.push_back(a.d_drv[x]); sig.push_back(a.d_off[x]); }
+  static_assert(std::has_unique_object_representations_v<OcrArgs> && sizeof(OcrArgs) % sizeof(int) == 0);
+  int v[sizeof(OcrArgs) / sizeof(int)];
+  std::memcpy(v, &o->a, sizeof v);
+  sig.insert(sig.end(), v, v + sizeof v / sizeof v[0]);
 }
 
 void ocr_half_step(const OcrPlan* o, const double* E, double dt, void* q, cudaStream_t st) {

@@ -1,0 +1,48 @@
+"""Solves that share a batched on-chip launch: what differs between them although their shapes are alike."""
+import numpy as np
+import pytest
+
+from paper_2406_18155_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+X = np.array([[0, 1, 0], [1, 0, 1.3], [0, 1.3, 0]], complex)
+Y = np.array([[0, -1j, 0], [1j, 0, -1.3j], [0, 1.3j, 0]], complex)
+
+
+def _system(ctx, op, seed):
+    """Two uncoupled transmons, each driven through a local operator: same shape for X and Y, but the
+    real-operator kernels turn the basis of a mode whose drive is imaginary."""
+    from paper_2406_18155_gb300.api import System
+    rng = np.random.Generator(np.random.PCG64(seed))
+    s = System(ctx)
+    for m in range(2):
+        s.add_transmon(2 * np.pi * (12 + m), 2 * np.pi * 0.3, levels=3)
+    for m in range(2):
+        k = s.add_local_op(m, op)
+        s.add_drive(m, k, "pwc", amps=rng.uniform(0.2, 0.6, 3), length=0.6, omega_mode=m)
+    s.prepare()
+    return s
+
+
+def test_packed_solves_keep_their_own_gauge(sgctx):
+    from paper_2406_18155_gb300.api import Server
+    T, dt, cols = 0.6, 0.01, W.comp_states([3, 3])
+    target = W.haar_unitary(4, np.random.Generator(np.random.PCG64(2)))
+    ops = [X, Y, Y, X]
+    alone = [_system(sgctx, op, i).fidelity_grad(T, dt, target, cols, precision="mixed") for i, op in enumerate(ops)]
+    srv = Server(sgctx, mem_budget_bytes=8 << 30, max_slots=1, max_batch=4)
+    # a first request holds the slot while the others queue up behind it
+    first = _system(sgctx, X, 9)
+    tickets = [srv.submit(first, 60.0, dt, target, cols)]
+    systems = [_system(sgctx, op, i) for i, op in enumerate(ops)]
+    tickets += [srv.submit(s, T, dt, target, cols) for s in systems]
+    res = [srv.wait(t) for t in tickets][1:]
+    assert srv.stats()["batched_requests"] >= 2
+    srv.close()
+    # a packed solve does the arithmetic of the lone one
+    for (F, gp, gh), r in zip(alone, res):
+        assert r["status"] == 0, r["error"]
+        assert abs(r["F"][0] - F[0]) <= 1e-12
+        assert np.max(np.abs(r["grad_pulse"] - gp)) <= 1e-12 * max(1.0, np.max(np.abs(gp)))
+        assert np.max(np.abs(r["grad_ham"] - gh)) <= 1e-12 * max(1.0, np.max(np.abs(gh)))
