@@ -1440,7 +1440,12 @@ struct Arena {
   std::vector<void*> ptrs;
   size_t bytes = 0;
   cudaStream_t st = nullptr;
-  ~Arena() { for (void* p : ptrs) cudaFreeAsync(p, st); }
+  ~Arena() { clear(); }
+  void clear() {
+    for (void* p : ptrs) cudaFreeAsync(p, st);
+    ptrs.clear();
+    bytes = 0;
+  }
   template <typename T> T* get(size_t n) {
     void* p = nullptr;
     size_t b = std::max<size_t>(n * sizeof(T), 16);
@@ -1724,8 +1729,15 @@ struct OcChunks {
   bool basis = false;
   int L = 1, C = 1, R = 1;
   int G = 1, NG = 1;              // prop: chunks per group of the two-level product, groups
+  // Buffers, all allocated with the plan (alloc_chunks):
   double2 *ck = nullptr, *lam = nullptr;   // states before, co-states after each chunk
   double2 *U = nullptr, *P = nullptr;      // chunk and group propagators
+  double2 *img = nullptr, *groups = nullptr;                     // products: columns in and out, before each group
+  double2 *unit = nullptr, *uapi = nullptr, *uimg = nullptr;     // the basis of co-states
+  double2* pimg = nullptr;        // a gradient's co-state,
+  void* segY = nullptr;           // stage inputs of a round on the complex rows,
+  void* colow = nullptr;          // low words of its co-states,
+  double *gF = nullptr, *acc = nullptr;    // and accumulators
 };
 
 struct Solve {
@@ -1763,6 +1775,7 @@ struct Solve {
   // on-chip: the solve's chunks of steps (plan_chunks)
   OnchipPlan* ocp = nullptr;      // propagator plan (D columns)
   OcChunks ch;
+  Arena car;                      // its buffers
   bool real_oc = false;           // terms real up to the frame phases (rterms), interaction frame
   OcrTerms rterms;
   void* half = nullptr;           // onchip_half_step
@@ -2092,6 +2105,8 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   Setup& s = sv.s;
   OcChunks& c = sv.ch;
   c = OcChunks{};
+  onchip_plan_destroy(sv.ocp);
+  sv.ocp = nullptr;
   const int N = s.N;
   c.L = N;
   const long long simg = onchip_state_elems(sv.oc);
@@ -2160,7 +2175,6 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   }
   // boundary states by serial passes; segments of L steps
   if (slots > 1 && N > kMinChunk) {
-    c.basis = basis;
     if (ckpt > 0) {
       c.L = std::min(ckpt, N);
     } else {
@@ -2171,6 +2185,7 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     c.C = (N + c.L - 1) / c.L;
     c.R = fit_rounds(c.C, c.L);
     c.par = c.C > 1;
+    c.basis = basis && c.par;
     if (!c.par || bytes(c.C, c.L, c.R, 0) <= work_limit) return;
     c = OcChunks{};
   }
@@ -2180,18 +2195,68 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   c.R = 1;
 }
 
-// A gradient solve's chunks and the states before them.
-sg_status alloc_chunks(sg_ctx* ctx, Solve& sv, int ckpt) {
-  plan_chunks(sv, true, ckpt, ctx->work_limit);
-  sv.ch.ck = sv.ar.get<double2>((size_t)sv.ch.C * onchip_state_elems(sv.oc));
-  if (!sv.ch.ck) return sg_fail(ctx, SG_E_NOMEM, "device allocation of checkpoints failed");
-  if (sv.ch.direct) {
-    const size_t n = (size_t)4 * sv.s.N * onchip_state_elems(sv.oc);
-    sv.ch.segU = sv.mixed ? (void*)sv.ar.get<float2>(n) : (void*)sv.ar.get<double2>(n);
-    sv.ch.segK = sv.mixed ? (void*)sv.ar.get<float2>(n) : (void*)sv.ar.get<double2>(n);
-    if (!sv.ch.segU || !sv.ch.segK) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the stage inputs failed");
+// The planned chunks' buffers; false if one cannot be allocated.
+bool chunk_buffers(Solve& sv, bool grad) {
+  const Setup& s = sv.s;
+  OcChunks& c = sv.ch;
+  Arena& ar = sv.car;
+  ar.st = sv.ar.st;
+  const size_t ns = (size_t)onchip_state_elems(sv.oc), DD = (size_t)s.D * s.D;
+  bool ok = true;
+  auto get = [&](double2*& p, size_t n) { ok = ok && (p = ar.get<double2>(n)); };
+  auto stage = [&](void*& p, size_t n) { ok = ok && (p = sv.mixed ? (void*)ar.get<float2>(n) : (void*)ar.get<double2>(n)); };
+  auto reals = [&](double*& p, size_t n) { ok = ok && (p = ar.get<double>(n)); };
+  if (c.prop) {
+    get(c.U, (size_t)c.C * onchip_columns(sv.ocp) * s.D);
+    get(c.P, c.NG > 1 ? (size_t)c.NG * DD : 1);
+    get(c.img, 2 * ns);
+    get(c.groups, (size_t)c.NG * ns);
   }
-  return SG_OK;
+  if (!grad) return ok;
+  const bool real = onchip_real_adjoint(sv.oc);
+  const size_t nstK = (size_t)3 * s.N * std::max(1, s.K);
+  get(c.ck, (size_t)c.C * ns);
+  get(c.pimg, ns);
+  if (c.basis) {
+    get(c.unit, (size_t)s.Dc * s.Dc);
+    get(c.uapi, (size_t)s.D * s.Dc);
+    get(c.uimg, ns);
+  }
+  if (c.par) get(c.lam, (size_t)c.C * ns);
+  else c.lam = c.pimg;
+  if (real) {
+    stage(c.segU, (size_t)4 * c.R * c.L * ns);
+    stage(c.segK, (size_t)4 * c.R * c.L * ns);
+    reals(c.gF, (size_t)ocr_groups(onchip_real_plan(sv.oc)) * nstK);
+    reals(c.acc, (size_t)ocr_blocks(onchip_real_plan(sv.oc)) * onchip_acc_doubles(sv.oc));
+  } else {
+    stage(c.segY, (size_t)4 * c.R * c.L * onchip_stage_elems(sv.oc));
+    if (onchip_colow_global(sv.oc)) ok = ok && (c.colow = ar.get<float2>((size_t)c.R * ns));
+    reals(c.gF, (size_t)onchip_ctas(sv.oc) * nstK);
+    reals(c.acc, (size_t)c.R * onchip_ctas(sv.oc) * onchip_acc_doubles(sv.oc));
+  }
+  return ok;
+}
+
+// An on-chip solve's chunks with their buffers, before its first launch.  Chunks side by side take up
+// to several GB (8 of stage inputs, the propagators) where one after the other take a few MB, so
+// a plan that does not fit beside what else holds memory is made again for half of what is
+// free once the pool's unused memory is given back, then for one chunk after the other.
+sg_status alloc_chunks(sg_ctx* ctx, Solve& sv, bool grad, int ckpt) {
+  size_t limit = ctx->work_limit;
+  for (int attempt = 0;; ++attempt) {
+    plan_chunks(sv, grad, ckpt, limit);
+    if (chunk_buffers(sv, grad)) return SG_OK;
+    sv.car.clear();
+    if (attempt == 2) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the chunks' buffers failed");
+    SG_CUDA_TRY(ctx, cudaStreamSynchronize(sv.ar.st));
+    cudaMemPool_t pool;
+    size_t free_b = 0, total_b = 0;
+    if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
+    cudaGetLastError();
+    limit = attempt == 0 ? std::min(limit, free_b / 2) : 0;
+  }
 }
 
 // The chunk propagators' products: columns `start` (a state image) through all chunks.
@@ -2222,7 +2287,6 @@ void chunk_products(Solve& sv, const double2* start, double2* states, double2* l
   sv.launches += onchip_chain(a, cols, c.NG, st);
 }
 
-// sv.psi evolved in place; with sv.ch.ck, the states before every chunk kept.
 FrameArgs frame_args(const Setup& s, const double* E_dev, double sign);
 CompArgs comp_args(const Setup& s);
 
@@ -2247,6 +2311,7 @@ OnchipRealTables real_tables(const Solve& sv) {
   return r;
 }
 
+// sv.psi evolved in place; with sv.ch.ck, the states before every chunk kept.
 template <typename R>
 sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
   sg_ctx* ctx = sys->ctx;
@@ -2259,33 +2324,25 @@ sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
   if (!c.prop) {
     f.psi_api = f.psi_out = sv.psi;
     f.ck_out = c.direct ? nullptr : c.ck;
-    f.segY = c.segU;
+    f.segY = c.direct ? c.segU : nullptr;
     f.K = c.L;
-    if (c.basis && (c.par || c.direct)) {
+    if (c.basis) {
       // unit vectors on the computational rows, in the frame, as co-states at the end
-      const long long n = s.D * s.S, ns = onchip_state_elems(sv.oc);
-      double2* unit = sv.ar.get<double2>((size_t)s.Dc * s.Dc);
-      double2* api = sv.ar.get<double2>((size_t)s.D * s.Dc);
-      double2* img = sv.ar.get<double2>((size_t)ns);
-      if (!c.direct) c.lam = sv.ar.get<double2>((size_t)c.C * ns);
-      if (!unit || !api || !img || (!c.direct && !c.lam))
-        return sg_fail(ctx, SG_E_NOMEM, "device allocation of the co-state basis failed");
-      (void)n;
-      SG_CUDA_TRY(ctx, cudaMemsetAsync(api, 0, (size_t)s.D * s.Dc * sizeof(double2), st));
-      SG_CUDA_TRY(ctx, cudaMemsetAsync(img, 0, (size_t)ns * sizeof(double2), st));
+      SG_CUDA_TRY(ctx, cudaMemsetAsync(c.uapi, 0, (size_t)s.D * s.Dc * sizeof(double2), st));
+      SG_CUDA_TRY(ctx, cudaMemsetAsync(c.uimg, 0, (size_t)onchip_state_elems(sv.oc) * sizeof(double2), st));
       CompArgs ca = comp_args(s);
       ca.S = s.Dc;
       FrameArgs fr = frame_args(s, sv.E_dev, +1.0);
       fr.S = s.Dc;
-      k_unit<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(s.Dc, unit);
-      k_scatter_comp<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(ca, unit, api);
-      k_frame<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(fr, api);
-      k_columns<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(s.D, s.Dc, api, img);
+      k_unit<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(s.Dc, c.unit);
+      k_scatter_comp<<<grid_for((long long)s.Dc * s.Dc), kT, 0, st>>>(ca, c.unit, c.uapi);
+      k_frame<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(fr, c.uapi);
+      k_columns<<<grid_for((long long)s.D * s.Dc), kT, 0, st>>>(s.D, s.Dc, c.uapi, c.uimg);
       OnchipForward b;
       b.rt = f.rt;
       b.rev = true;
-      b.img_in = img;
-      b.segY = c.segK;
+      b.img_in = c.uimg;
+      b.segY = c.direct ? c.segK : nullptr;
       b.ck_out = c.direct ? nullptr : c.lam;
       b.K = c.L;
       sv.launches += 4 + onchip_forward_pair(sv.oc, f, b, s.N, s.dt, st);
@@ -2297,12 +2354,7 @@ sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
   }
   const long long simg = onchip_state_elems(sv.oc), DD = (long long)s.D * s.D;
   const long long uimg = (long long)onchip_columns(sv.ocp) * s.D;
-  c.U = sv.ar.get<double2>((size_t)c.C * uimg);
-  c.P = sv.ar.get<double2>(c.NG > 1 ? (size_t)c.NG * DD : 1);
-  double2* img = sv.ar.get<double2>(2 * (size_t)simg);
-  double2* groups = sv.ar.get<double2>((size_t)c.NG * simg);
-  if (!c.U || !c.P || !img || !groups) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the chunk propagators failed");
-  onchip_to_image(sv.oc, sv.psi, img, st);
+  onchip_to_image(sv.oc, sv.psi, c.img, st);
   f.ident = true;
   f.img_out = c.U;
   sv.launches += 1 + onchip_forward(sv.ocp, f, 0, s.N, c.L, s.dt, st);
@@ -2312,8 +2364,8 @@ sg_status run_forward_onchip(sg_system* sys, Solve& sv) {
     a.last = c.P; a.last_stride = DD;
     sv.launches += onchip_chain(a, (int)s.D, c.NG, st);
   }
-  chunk_products(sv, img, c.ck, img + simg, groups, false, st);
-  onchip_from_image(sv.oc, img + simg, sv.psi, st);
+  chunk_products(sv, c.img, c.ck, c.img + simg, c.groups, false, st);
+  onchip_from_image(sv.oc, c.img + simg, sv.psi, st);
   ++sv.launches;
   SG_CUDA_TRY(ctx, cudaGetLastError());
   return SG_OK;
@@ -2439,17 +2491,12 @@ sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc ac
   const long long ns = onchip_state_elems(oc);
   const long long nst = 3ll * s.N, nstK = nst * std::max(1, s.K);
   const int groups = ocr_groups(rp), blocks = ocr_blocks(rp);
-  const size_t naccd = (size_t)blocks * onchip_acc_doubles(oc), nseg = (size_t)4 * c.R * c.L * ns;
-  double2* pimg = sv.ar.get<double2>(ns);
-  C* segU = c.direct ? static_cast<C*>(c.segU) : sv.ar.get<C>(nseg);
-  C* segK = c.direct ? static_cast<C*>(c.segK) : sv.ar.get<C>(nseg);
-  double* gFc = sv.ar.get<double>((size_t)groups * nstK);
-  double* accc = sv.ar.get<double>(naccd);
-  const bool basis = c.basis && (c.par || c.direct);
-  if (!(basis && c.par)) c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
-  double2* gimg = c.prop ? sv.ar.get<double2>((size_t)c.NG * ns) : pimg;
-  if (!pimg || !segU || !segK || !gFc || !accc || !c.lam || !gimg)
-    return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
+  const size_t naccd = (size_t)blocks * onchip_acc_doubles(oc);
+  double2* const pimg = c.pimg;
+  C* const segU = static_cast<C*>(c.segU);
+  C* const segK = static_cast<C*>(c.segK);
+  double *const gFc = c.gF, *const accc = c.acc;
+  const bool basis = c.basis;
   SG_CUDA_TRY(ctx, cudaMemsetAsync(gFc, 0, (size_t)groups * nstK * sizeof(double), st));
   SG_CUDA_TRY(ctx, cudaMemsetAsync(accc, 0, naccd * sizeof(double), st));
   onchip_to_image(oc, pbar, pimg, st);
@@ -2464,7 +2511,7 @@ sg_status run_backward_real(sg_system* sys, Solve& sv, double2* pbar, GradAcc ac
                                 c.direct ? 4ll * s.N : c.C, sv.barc, s.Dc, st));
     ++sv.launches;
   } else if (c.prop) {
-    chunk_products(sv, pimg, c.lam, nullptr, gimg, true, st);
+    chunk_products(sv, pimg, c.lam, nullptr, c.groups, true, st);
   } else if (c.par) {
     b.img_in = pimg;
     b.ck_out = c.lam;
@@ -2512,16 +2559,11 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc 
   const long long nst = 3ll * s.N;
   const int Kd = std::max(1, s.K);
   const size_t naccd = (size_t)c.R * ncta * onchip_acc_doubles(oc);
-  double2* pimg = sv.ar.get<double2>(ns);
-  C* segY = sv.ar.get<C>((size_t)4 * c.R * c.L * nstage);
-  double* gFc = sv.ar.get<double>((size_t)ncta * nst * Kd);
-  double* accc = sv.ar.get<double>(naccd);
+  double2* const pimg = c.pimg;
+  C* const segY = static_cast<C*>(c.segY);
+  double *const gFc = c.gF, *const accc = c.acc;
   int* err = sv.ar.get<int>(1);
-  void* colow = onchip_colow_global(oc) ? (void*)sv.ar.get<float2>((size_t)c.R * ns) : nullptr;
-  c.lam = c.par ? sv.ar.get<double2>((size_t)c.C * ns) : pimg;
-  double2* groups = c.prop ? sv.ar.get<double2>((size_t)c.NG * ns) : pimg;
-  if (!pimg || !segY || !gFc || !accc || !err || (onchip_colow_global(oc) && !colow) || !c.lam || !groups)
-    return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
+  if (!err) return sg_fail(ctx, SG_E_NOMEM, "device allocation of the on-chip adjoint buffers failed");
   SG_CUDA_TRY(ctx, cudaMemsetAsync(gFc, 0, (size_t)ncta * nst * Kd * sizeof(double), st));
   SG_CUDA_TRY(ctx, cudaMemsetAsync(accc, 0, naccd * sizeof(double), st));
   SG_CUDA_TRY(ctx, cudaMemsetAsync(err, 0, sizeof(int), st));
@@ -2541,7 +2583,7 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc 
     tb = OnchipTables{tab, atab, sv.coef32, sv.ph32, op32};
   }
   if (c.prop) {
-    chunk_products(sv, pimg, c.lam, nullptr, groups, true, st);
+    chunk_products(sv, pimg, c.lam, nullptr, c.groups, true, st);
   } else if (c.par) {
     OnchipForward b;
     b.tab = atab;
@@ -2561,7 +2603,7 @@ sg_status run_backward_onchip(sg_system* sys, Solve& sv, double2* pbar, GradAcc 
     f.rows = true;
     sv.launches += onchip_forward(oc, f, n0, n1, c.L, s.dt, st);
     sv.launches += onchip_adjoint(oc, tb, segY, c.par ? c.lam + (size_t)c0 * ns : pimg, n0, n1, c.L, s.dt, xa,
-                                  (int)nst, gFc, accc, err, colow, st);
+                                  (int)nst, gFc, accc, err, c.colow, st);
   }
   onchip_batcher_release();                       // the solve's last on-chip launch is issued
   onchip_reduce(oc, gFc, ncta, accc, c.R * ncta, nst, s.K, s.p.n1, s.p.ne, acc, st);
@@ -2876,7 +2918,10 @@ sg_status sg_evolve_impl(sg_system* sys, const sg_evolve_opts* o, void* psi_dev)
   rc = upload_and_tables(sys, o, sv, false);
   if (rc != SG_OK) return rc;
   sv.psi = static_cast<double2*>(psi_dev);
-  if (!s.q2 && sv.onchip(false)) plan_chunks(sv, false, 0, ctx->work_limit);
+  if (!s.q2 && sv.onchip(false)) {
+    rc = alloc_chunks(ctx, sv, false, 0);
+    if (rc != SG_OK) return rc;
+  }
   if (s.q2) rc = run_q2(sys, sv, cols_dev, !o->col_index);
   else rc = o->precision == SG_MIXED ? run_forward<float>(sys, sv, cols_dev, !o->col_index, 0, nullptr)
                                      : run_forward<double>(sys, sv, cols_dev, !o->col_index, 0, nullptr);
@@ -3027,13 +3072,16 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
   int K = 0;
   std::vector<double2*> ckpts;
   if (grad && !dressed) sv.barc = barc;
-  if (!grad && !s.q2 && sv.onchip(false)) plan_chunks(sv, false, 0, ctx->work_limit);
+  if (!grad && !s.q2 && sv.onchip(false)) {
+    rc = alloc_chunks(ctx, sv, false, 0);
+    if (rc != SG_OK) return rc;
+  }
   if (grad && !s.q2) {             // the Q2 adjoint recomputes the states by inverse factors
     K = ckpt > 0 ? ckpt : std::max(1, (int)std::lround(std::sqrt((double)s.N)));
     K = std::min(K, s.N);
     const int nck = (s.N + K - 1) / K;
     if (sv.onchip(true)) {
-      rc = alloc_chunks(ctx, sv, ckpt);
+      rc = alloc_chunks(ctx, sv, true, ckpt);
       if (rc != SG_OK) return rc;
       K = sv.ch.L;
     } else {
@@ -3103,7 +3151,7 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
   SG_CUDA_TRY(ctx, cudaGetLastError());
   cudaEventRecord(ev1, st);
   double Fh[2];
-  size_t peak = sv.ar.bytes;
+  size_t peak = sv.ar.bytes + sv.car.bytes;
   if (grad) {
     // accumulators
     const int ne = s.p.ne, n1 = s.p.n1;
@@ -3210,7 +3258,7 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
       if (grad_pulse) for (int k = 0; k < s.n_pulse; ++k) grad_pulse[k] = g[k];
       for (int k = 0; k < nh; ++k) grad_ham[k] = g[s.n_pulse + k];
     }
-    peak = sv.ar.bytes;
+    peak = sv.ar.bytes + sv.car.bytes;
   } else {
     cudaEventRecord(ev2, st);
     SG_CUDA_TRY(ctx, cudaStreamSynchronize(st));
@@ -3327,7 +3375,7 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
   const int nck = (s.N + K - 1) / K;
   std::vector<double2*> ckpts;
   if (sv.onchip(true)) {
-    rc = alloc_chunks(ctx, sv, ckpt);
+    rc = alloc_chunks(ctx, sv, true, ckpt);
     if (rc != SG_OK) return rc;
     K = sv.ch.L;
   } else {
@@ -3472,7 +3520,7 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
   cudaEventElapsedTime(&bwd_ms, ev1, ev2);
   sys->last_stats[0] = fwd_ms;
   sys->last_stats[1] = bwd_ms;
-  sys->last_stats[2] = (double)(sv.ar.bytes + sva.ar.bytes);
+  sys->last_stats[2] = (double)(sv.ar.bytes + sv.car.bytes + sva.ar.bytes);
   sys->last_stats[3] = K;
   sv.kt.finish(sys->ktimes);
   sys->last_stats[4] = sv.launches + (double)(sv.kt.total[0] + sv.kt.total[1] + sv.kt.total[2]);
