@@ -46,3 +46,34 @@ def test_gradient_fits_beside_another_user(sgctx, nq, levels, cols, steps, ckpt,
     r = subprocess.run([sys.executable, "-c", _SOLVE] + [str(v) for v in (nq, levels, cols, steps, ckpt, left)],
                        cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr[-2000:]
+
+
+_BATCH = """
+import numpy as np, torch
+from paper_2406_18155_gb300 import workloads as W
+from paper_2406_18155_gb300.api import Context, System, evolve_batch
+ctx, dt, steps = Context(0), 0.005, 20000
+systems = []
+for i in range(256):
+    s = System.from_workload(ctx, W.transmon_pair(seed=i, T=steps * dt, dt=dt))
+    s.prepare()
+    systems.append(s)
+cols = list(range(16))
+evolve_batch(systems[:2], 4 * dt, dt, cols)                     # kernels loaded
+other = torch.empty(torch.cuda.mem_get_info()[0] - (250 << 20), dtype=torch.uint8, device="cuda")
+out = []
+for _ in range(2):
+    out.append((evolve_batch(systems, steps * dt, dt, cols).cpu().numpy(), systems[0].last_stats()["launches"]))
+    del other
+    torch.cuda.empty_cache()
+    other = None
+(a, n), (b, m) = out
+print("launches", n, m)
+assert n < m and np.max(np.abs(a - b)) < 1e-5
+"""
+
+
+def test_batch_fits_beside_another_user(sgctx):
+    # 256 pairs of 20,000 steps: 330 MB of frame phases with room, the dense kernel without
+    r = subprocess.run([sys.executable, "-c", _BATCH], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr[-2000:]
