@@ -3782,6 +3782,7 @@ sg_status sg_evolve_batch_impl(sg_system* const* systems, int B, const sg_evolve
   struct PlanGuard { OcrPlan** p; ~PlanGuard() { ocr_plan_destroy(*p); } } guard{&rp};
   std::vector<double2> opds;
   std::vector<double> Es, Js;
+  std::vector<int> parts;                      // of the couplings' factors, system after system (TabArgs::e_zpart)
   TabArgs ta0;
   // per system: dense real [C; O_1..O_K] (R x Dp), composite energies, drives
   std::vector<double> A, E((size_t)B * D, 0.0), amps;
@@ -3811,6 +3812,7 @@ sg_status sg_evolve_batch_impl(sg_system* const* systems, int B, const sg_evolve
       drv[(size_t)b * K + k] = dd;
     }
     for (double v : ss.amps) amps.push_back(v);
+    parts.insert(parts.end(), ta.e_zpart, ta.e_zpart + ss.p.ne);
     if (b == 0) {
       ta0 = ta;
       if (real) {
@@ -3879,20 +3881,16 @@ sg_status sg_evolve_batch_impl(sg_system* const* systems, int B, const sg_evolve
     }
   }
   A.assign((size_t)B * R * Dp, 0.0);
+  size_t at = 0;
   for (int b = 0; b < B; ++b) {
     sg_system* sy = systems[b];
-    Setup ss;
-    rc = build_setup(sy, o, ss);
-    if (rc != SG_OK) return rc;
-    TabArgs ta = ss.ta;
-    real_terms(sy, ss, ta);
     double* Ab = A.data() + (size_t)b * R * Dp;
-    if (ss.frame == SG_FRAME_LAB)
+    if (s.frame == SG_FRAME_LAB)
       for (int i = 0; i < D; ++i) Ab[(size_t)i * Dp + i] += E[(size_t)b * D + i];
     // couplings: J A (x) B on modes (a, b), the other digits equal
-    for (int e = 0; e < ss.p.ne; ++e) {
+    for (size_t e = 0; e < sy->couplings.size(); ++e) {
       const HostCoupling& c = sy->couplings[e];
-      const int part = ta.e_zpart[e];
+      const int part = parts[at++];
       const double J = part ? -c.J : c.J;
       for (int i = 0; i < D; ++i)
         for (int j = 0; j < D; ++j) {
