@@ -7,7 +7,7 @@
 // with its own tables, buffers and step range.  A host thread bound to a batcher
 // (onchip_batcher_bind) hands its on-chip launches to the batcher instead of
 // launching them: the batcher waits until every thread that has joined it has handed
-// over one launch, then issues them as batched launches on its own stream (ordered
+// over its next launch (or two that do not wait for one another), then issues them as batched launches on its own stream (ordered
 // after each thread's earlier work by events) and makes each thread's stream wait
 // for the launch that holds its CTAs.  Each CTA does exactly the arithmetic of the
 // unbatched launch, so results do not depend on the batching.

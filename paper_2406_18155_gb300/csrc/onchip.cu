@@ -1357,6 +1357,7 @@ struct OcBatcher {
   std::condition_variable cv;
   int participants = 0;
   std::vector<OcPending*> subs;
+  int waiting = 0;                // threads that have handed over their launches of this round
   unsigned long long gen = 0;
   long long launches = 0, members = 0;
 
@@ -1382,22 +1383,27 @@ struct OcBatcher {
       members += bt.nsys;
     }
     subs.clear();
+    waiting = 0;
     ++gen;
     cv.notify_all();
   }
 
-  int submit(const OcPending& p0, cudaStream_t user) {
-    OcPending p = p0;
-    p.ready = tl_ready;
-    p.done = tl_done;
-    cudaEventRecord(p.ready, user);
+  // n launches of one thread that do not wait for one another (they share its events: the
+  // batches of a round follow one another on st, so the last record covers all).
+  int submit(OcPending* p, int n, cudaStream_t user) {
+    for (int i = 0; i < n; ++i) {
+      p[i].ready = tl_ready;
+      p[i].done = tl_done;
+    }
+    cudaEventRecord(tl_ready, user);
     std::unique_lock<std::mutex> lk(mu);
-    subs.push_back(&p);
+    for (int i = 0; i < n; ++i) subs.push_back(p + i);
+    ++waiting;
     const unsigned long long g = gen;
-    if ((int)subs.size() >= participants) launch_round();
+    if (waiting >= participants) launch_round();
     else cv.wait(lk, [&] { return gen != g; });
     lk.unlock();
-    cudaStreamWaitEvent(user, p.done, 0);
+    cudaStreamWaitEvent(user, tl_done, 0);
     return 1;
   }
 };
@@ -1438,7 +1444,7 @@ void onchip_batcher_release() {
   {
     std::lock_guard<std::mutex> lk(b->mu);
     --b->participants;
-    if (!b->subs.empty() && (int)b->subs.size() >= b->participants) b->launch_round();
+    if (!b->subs.empty() && b->waiting >= b->participants) b->launch_round();
   }
   cudaEventDestroy(tl_ready);
   cudaEventDestroy(tl_done);
@@ -1456,8 +1462,8 @@ void onchip_batcher_stats(const OcBatcher* b, long long* launches, long long* me
 namespace {
 
 // One launch, through the thread's batcher when it has one.
-int submit(const OcPending& p, cudaStream_t st) {
-  if (tl_batcher) return tl_batcher->submit(p, st);
+int submit(OcPending p, cudaStream_t st) {
+  if (tl_batcher) return tl_batcher->submit(&p, 1, st);
   OcBatch bt{};
   bt.nsys = 1;
   bt.s[0] = p.d;
@@ -1504,13 +1510,13 @@ int onchip_forward(const OnchipPlan* oc, const OnchipForward& f, int n0, int n1,
 
 int onchip_forward_pair(const OnchipPlan* oc, const OnchipForward& f, const OnchipForward& b, int N, double dt,
                         cudaStream_t st) {
-  const OcPending p = forward_of(oc, f, 0, N, N, dt), q = forward_of(oc, b, 0, N, N, dt);
-  if (tl_batcher) return submit(p, st) + submit(q, st);
+  OcPending p[2] = {forward_of(oc, f, 0, N, N, dt), forward_of(oc, b, 0, N, N, dt)};
+  if (tl_batcher) return tl_batcher->submit(p, 2, st);
   OcBatch bt{};
   bt.nsys = 2;
-  bt.s[0] = p.d;
-  bt.s[1] = q.d;
-  return oc_launch(oc, p.kind, bt, dt, nullptr, st);
+  bt.s[0] = p[0].d;
+  bt.s[1] = p[1].d;
+  return oc_launch(oc, p[0].kind, bt, dt, nullptr, st);
 }
 
 int onchip_adjoint(const OnchipPlan* oc, const OnchipTables& tb, const void* segY, double2* lam, int n0, int n1,

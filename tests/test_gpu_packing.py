@@ -46,3 +46,38 @@ def test_packed_solves_keep_their_own_gauge(sgctx):
         assert abs(r["F"][0] - F[0]) <= 1e-12
         assert np.max(np.abs(r["grad_pulse"] - gp)) <= 1e-12 * max(1.0, np.max(np.abs(gp)))
         assert np.max(np.abs(r["grad_ham"] - gh)) <= 1e-12 * max(1.0, np.max(np.abs(gh)))
+
+
+def test_packed_serial_passes_share_one_launch(sgctx):
+    """Beyond D = 256 the states and the basis of co-states are serial passes that do not wait for one
+    another: a pack issues them together, so each batch is one round of launches."""
+    from paper_2406_18155_gb300.api import Server, System
+    wls = []
+    for i in range(4):
+        wl = W.serving_request(np.random.Generator(np.random.PCG64(i)), nq=4, kind="fluxonium", levels=5)
+        wl["T"] = 3000 * wl["dt"] if i == 0 else 12 * wl["dt"]
+        for d in wl["drives"]:
+            d["length"] = wl["T"]
+        wls.append(wl)
+
+    def system(wl):
+        s = System.from_workload(sgctx, wl)
+        s.prepare()
+        return s
+
+    args = lambda wl: (wl["T"], wl["dt"], wl["target"], wl["col_index"])  # noqa: E731
+    alone = [system(wl).fidelity_grad(*args(wl), kind=wl["fid_kind"], precision="mixed") for wl in wls[1:]]
+    srv = Server(sgctx, mem_budget_bytes=32 << 30, max_slots=1, max_batch=4)
+    systems = [system(wl) for wl in wls]
+    # the first request holds the slot while the others queue up behind it
+    tickets = [srv.submit(s, *args(wl), kind=wl["fid_kind"], precision="mixed") for s, wl in zip(systems, wls)]
+    res = [srv.wait(t) for t in tickets][1:]
+    st = srv.stats()
+    srv.close()
+    assert st["batches"] == 1 and st["batched_requests"] == 3
+    assert st["batched_launches"] == 1 and st["batched_launch_members"] == 6
+    for (F, gp, gh), r in zip(alone, res):
+        assert r["status"] == 0, r["error"]
+        assert abs(r["F"][0] - F[0]) <= 1e-12
+        assert np.max(np.abs(r["grad_pulse"] - gp)) <= 1e-12 * max(1.0, np.max(np.abs(gp)))
+        assert np.max(np.abs(r["grad_ham"] - gh)) <= 1e-12 * max(1.0, np.max(np.abs(gh)))
