@@ -87,6 +87,17 @@ size_t estimate_bytes(const sg_system* sys, const sg_evolve_opts& o, int want_gr
   return b;
 }
 
+// What a gradient on the on-chip kernels holds beyond that with its chunks one after the other:
+// stage inputs of the states and of the co-states, and the density accumulators.
+size_t onchip_extra_bytes(const sg_system* sys, const sg_evolve_opts& o, int want_grad) {
+  double D = 1;
+  for (const HostMode& m : sys->modes) D *= m.d;
+  if (!want_grad || D > 4096 || sys->modes.size() < 2) return 0;
+  const double image = D * (o.ncols + 16) * sizeof(double2);
+  const double acc = 130.0 * sys->drives.size() + 290.0 * sys->couplings.size() + 10.0 * sys->modes.size();
+  return (size_t)(4 * std::sqrt(o.T / o.dt) * image + 304 * acc * sizeof(double));
+}
+
 }  // namespace
 
 struct sg_server {
@@ -331,8 +342,12 @@ sg_status sg_server_submit(sg_server* srv, const sg_request* req, uint64_t* tick
     ++srv->rejected;
     return sg_fail(srv->ctx, SG_E_NOMEM_RETRY, "request alone exceeds the memory budget");
   }
-  // a budget too small for the chunks side by side leaves them to run one after the other
-  r->chunk_mem = std::min(sg_chunk_bytes(req->sys, &r->opts, req->want_grad != 0), srv->budget - r->mem);
+  r->mem = std::min(srv->budget, r->mem + onchip_extra_bytes(req->sys, r->opts, req->want_grad));
+  // Memory for the chunks side by side makes a solve faster but is not needed: up to an equal share of
+  // the budget, so that every slot and every member of its pack finds room (without it the chunks run one
+  // after the other).  The share does not depend on what else runs, and so neither do the results.
+  const size_t share = srv->budget / ((size_t)srv->max_slots * srv->max_batch);
+  r->chunk_mem = std::min(sg_chunk_bytes(req->sys, &r->opts, req->want_grad != 0), share > r->mem ? share - r->mem : 0);
   r->mem += r->chunk_mem;
   srv->inflight[req->sys] = 1;
   r->ticket = srv->next_ticket++;

@@ -81,3 +81,41 @@ def test_packed_serial_passes_share_one_launch(sgctx):
         assert abs(r["F"][0] - F[0]) <= 1e-12
         assert np.max(np.abs(r["grad_pulse"] - gp)) <= 1e-12 * max(1.0, np.max(np.abs(gp)))
         assert np.max(np.abs(r["grad_ham"] - gh)) <= 1e-12 * max(1.0, np.max(np.abs(gh)))
+
+
+@pytest.mark.parametrize("slots,batch", [(1, 4), (4, 1)])
+def test_small_budget_still_runs_requests_together(sgctx, slots, batch):
+    """64 MiB hold the needs of many D = 27 requests: what each may take to run its chunks side by side
+    must not fill the budget."""
+    from paper_2406_18155_gb300.api import Server, System
+    wls = []
+    for i in range(5):
+        wl = W.serving_request(np.random.Generator(np.random.PCG64(i)), nq=3, kind="fluxonium", levels=3)
+        # the first request of one slot holds it while the others queue up
+        wl["T"] = (1000 if i == 0 or slots > 1 else 60) * wl["dt"]
+        for d in wl["drives"]:
+            d["length"] = wl["T"]
+        wls.append(wl)
+
+    def system(wl):
+        s = System.from_workload(sgctx, wl)
+        s.prepare()
+        return s
+
+    args = lambda wl: (wl["T"], wl["dt"], wl["target"], wl["col_index"])  # noqa: E731
+    alone = [system(wl).fidelity_grad(*args(wl), kind=wl["fid_kind"], precision="fp64") for wl in wls]
+    srv = Server(sgctx, mem_budget_bytes=64 << 20, max_slots=slots, max_batch=batch)
+    systems = [system(wl) for wl in wls]
+    tickets = [srv.submit(s, *args(wl), kind=wl["fid_kind"], precision="fp64") for s, wl in zip(systems, wls)]
+    res = [srv.wait(t) for t in tickets]
+    st = srv.stats()
+    srv.close()
+    for (F, gp, gh), r in zip(alone, res):
+        assert r["status"] == 0, r["error"]
+        assert abs(r["F"][0] - F[0]) <= 1e-10
+        g = np.concatenate([gp, gh])
+        assert np.max(np.abs(np.concatenate([r["grad_pulse"], r["grad_ham"]]) - g)) <= 1e-8 * np.max(np.abs(g))
+    if slots == 1:
+        assert st["batched_requests"] == 4
+    else:
+        assert sorted(r["start_s"] for r in res)[1] < min(r["done_s"] for r in res)
