@@ -3208,7 +3208,10 @@ sg_status sg_fidelity_impl(sg_system* sys, const sg_evolve_opts* o, const double
       int np_max = 1;
       for (auto& d : s.drives) np_max = std::max(np_max, d.kind == SG_ENV_PWC ? d.nseg : 1);
       rc = launch_pulse_chain(sv, acc.gF, np_max, poff, gpulse, omega_bar, s.q2 ? s.ta.nsub : 0);
-    if (rc != SG_OK) return rc;
+      if (rc != SG_OK) {
+        cudaEventDestroy(ev0); cudaEventDestroy(ev1); cudaEventDestroy(ev2);
+        return sg_fail(ctx, rc, "device allocation of the pulse gradient's shares failed");
+      }
     } else {
       SG_CUDA_TRY(ctx, cudaMemsetAsync(omega_bar, 0, sizeof(double), st));
     }
@@ -3451,7 +3454,7 @@ sg_status sg_gate_fidelity_open_grad_impl(sg_system* sys, const sg_evolve_opts* 
     int np_max = 1;
     for (auto& d : s.drives) np_max = std::max(np_max, d.kind == SG_ENV_PWC ? d.nseg : 1);
     rc = launch_pulse_chain(sv, acc.gF, np_max, poff, gpulse, omega_bar, 0);
-    if (rc != SG_OK) return done(rc);
+    if (rc != SG_OK) return done(sg_fail(ctx, rc, "device allocation of the pulse gradient's shares failed"));
     ++sv.launches;
   }
   double* gdev = nullptr;
