@@ -906,8 +906,10 @@ struct OcChainArgs {
   OnchipChain a;
   int ncols, rows, parts;
 };
+// Threads at most: entries held in registers (E > 0) come with D <= 64 only, and so with 512 (onchip_chain).
+constexpr int chain_threads(int E) { return E ? 512 : 768; }
 template <bool ADJ, int E>
-__global__ void k_oc_chain(const __grid_constant__ OcChainArgs k) {
+__global__ void __launch_bounds__(chain_threads(E)) k_oc_chain(const __grid_constant__ OcChainArgs k) {
   extern __shared__ __align__(16) unsigned char sm[];
   const OnchipChain& a = k.a;
   const int D = a.D, s = blockIdx.x, g = blockIdx.y;
@@ -1758,7 +1760,7 @@ int onchip_chain(const OnchipChain& a, int ncols, int ngroups, cudaStream_t st) 
   // threads: D rows (padded to whole warps) times parts of the sum
   const int rows = D <= 16 ? 16 : (D + 31) / 32 * 32;
   k.rows = rows;
-  k.parts = std::max(1, std::min((D > 64 ? 768 : 512) / rows, (D + 3) / 4));
+  k.parts = std::max(1, std::min((D > 64 ? chain_threads(0) : chain_threads(4)) / rows, (D + 3) / 4));
   const int threads = (rows * k.parts + 31) / 32 * 32;
   const int each = (D + k.parts - 1) / k.parts;
   const size_t smem = (size_t)(D + rows * k.parts) * sizeof(double2);
