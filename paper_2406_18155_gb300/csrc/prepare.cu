@@ -46,9 +46,9 @@ __device__ void jacobi_eigen(double* A, double* V, int M, double* cs, int* pairs
     double dia_tot = red[0];
     __syncthreads();
     if (off_tot <= 1e-32 * dia_tot || off_tot == 0.0) break;
-    // entries too small to keep the test above from passing (M^2 of them add up to less than
-    // a third of its bound) are not rotated: where parity splits the matrix that is half of them
-    const double small = 1e-18 * sqrt(dia_tot);
+    // entries too small to keep the test above from passing (M^2 of them add up to a third of its
+    // bound at most) are not rotated: where parity splits the matrix that is half of them
+    const double small = 5.7e-17 / M * sqrt(dia_tot);
     for (int round = 0; round < Mp - 1; ++round) {
       // pairing of this round (circle method): position 0 holds player 0,
       // position i >= 1 holds 1 + (i - 1 + round) mod (Mp - 1)
