@@ -1888,7 +1888,10 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
   // a solve goes before its first kernel (see dcopy)
   sv.mixed = o->precision == SG_MIXED;
   const int pc = path_choice();
-  if (!s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows) {
+  // A mixed evolution of a few steps on a small system is one serial launch (plan_chunks), where complex rows
+  // have less to set up: D = 25, four steps 0.14 ms, real operators 0.18; D = 125, eight steps 0.23 and 0.28
+  const bool few = !grad && sv.mixed && (s.D <= 64 ? s.N < 10 : s.p.dims[0] == 5 && s.D <= 125 && s.N < 16);
+  if (!s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows && !few) {
     fill_terms(s, s.ta, sv.rterms);
     sv.real_oc = real_gauge(sys, s, sv.rterms);
   }
@@ -2155,6 +2158,15 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
       c.G = c.C;
       if (two < one) c.G = G;
       c.NG = (c.C + c.G - 1) / c.G;
+      // An evolution alone trades N steps for L of every column, a few launches (35 us) and C products
+      // that wait for one another (130 us each at D = 256, 85 at 243, 27 at 125).  In mixed steps of the serial
+      // evolution, 8 us with real operators (five levels 16) and 14 us on complex rows, which take twice as
+      // long with every column; FP64 steps are ten times as long.  D = 256, 16 columns, 32 steps: 1.04 ms in
+      // chunks, 0.45 serially; 300 steps 1.49 against 2.5.
+      const double q = (D / 256) * (D / 256), dl = s.p.dims[0];
+      const double cost = onchip_real(sv.ocp) ? (sv.mixed ? c.L + 4 + c.C * (dl == 5 ? 8 : 14) * q : c.L + c.C * q)
+                                              : 2 * c.L + 2 + c.C * (sv.mixed ? 8 : 1) * q;
+      if (!grad && cost >= N) c.prop = false;
       const size_t nprop = (size_t)s.D * onchip_columns(sv.ocp) + (c.NG > 1 ? (size_t)s.D * s.D / c.G + 1 : 0);
       if (c.prop && bytes(grad ? c.C : 0, c.L, grad ? c.R : 0, 0) + c.C * nprop * sizeof(double2) <= work_limit) return;
       c = OcChunks{};
