@@ -53,7 +53,7 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 // exp(i theta) as an FP32 pair of modulus nearer to 1 (|z|^2 - 1: 1e-8 rms over the levels of
 // transmon and fluxonium pairs at 10 ps, the nearest pair's 3e-8), at the price of an angle off by up to
-// 1e-6: steps the larger part by one unit in the last place at most and solves for the smaller one,
+// 2e-7 (short solves see it, long ones the modulus): steps the larger part by one unit in the last place at most and solves for the smaller one,
 // whose own rounding is finer.
 __device__ __forceinline__ float2 unit_phase32(double theta) {
   double sn, cs;
@@ -66,7 +66,7 @@ __device__ __forceinline__ float2 unit_phase32(double theta) {
   for (int i = -1; i <= 1; ++i) {
     const double b = fma((double)i, 5.9604644775390625e-08, b0);      // 2^-24: the spacing in [0.5, 1)
     if (fabs(b) > 1.0) continue;
-    const double s = (double)(float)(small + fmin(1e-6, fmax(-1e-6, slope * (b - big))));
+    const double s = (double)(float)(small + fmin(2e-7, fmax(-2e-7, slope * (b - big))));
     const double r = fabs(fma(b, b, -1.0) + s * s);
     if (r < best) {
       best = r;

@@ -34,10 +34,11 @@
 // modulus 1 (unit_phase32): an error of its angle turns the terms of stages 1 and 4 by
 // opposite angles, which cancel from step to step, an error of its modulus does not.  The phases
 // P_m, which turn the state and its increment back, have modulus 1 on average (unit_cis32).
-// Against 64 bits, D = 25 pair, 10,000 steps, worst of five inputs: pulse gradient 5.5e-7 -> 1.4e-7
-// (complex rows 6.5e-7), Hamiltonian gradient 9.6e-7 -> 2.5e-7 (2.1e-6); four modes of three levels, 2560
-// steps: state 1.3e-7 -> 5e-8; at the same speed (1.57 ms, 6-mode chain 106 ms).  psi stays in the interaction
-// picture, so no phase error accumulates in it: P_m is read from the phase table every step.
+// Against 64 bits, D = 25 pair, 10,000 steps, worst of five inputs: pulse gradient 5.5e-7 -> 1.5e-7
+// (complex rows 6.5e-7), Hamiltonian gradient 9.6e-7 -> 2.8e-7 (2.1e-6); five modes of four levels, 2560
+// steps: state 1.2e-7 -> 9e-8; at the same speed (1.57 ms, 6-mode chain 106 ms).
+//
+// psi stays in the interaction picture, so no phase error accumulates in it: P_m is read from the phase table every step.
 // Real times complex halves the multiply-adds (one packed FP32x2 FMA each), and the
 // matrices stay in shared memory for the whole run; a stage reads K drive coefficients
 // from memory instead of a row of term matrices.
@@ -323,7 +324,7 @@ template <int N, typename C> struct Own<false, N, C> {
 // rounding and the remainder (f h + f l): an element rounded alone is a constant error of H that
 // adds up over the steps, where the product's rounding changes with f.  Against FP64 over 6000
 // steps of a 6-mode chain, largest gradient error over the largest component, with the constants of
-// the step as above: 1.4e-4 (7.6e-4 on the complex-row kernels).
+// the step as above: 1.3e-4 (rounded alone 1.1e-3, complex-row kernels 7.6e-4).
 template <typename R> struct OpEl {
   R h = 0, l = 0;
   OpEl() = default;
