@@ -2137,6 +2137,11 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     if (R > slots) R = R / slots * slots;               // whole waves
     return (int)std::min<long long>(R, C);
   };
+  // The two serial passes run side by side when the SMs hold both and every computational row has
+  // an image column: D = 3125 with 32 columns takes 32 CTAs each way (1000 steps with their
+  // gradient: 62 -> 40.6 ms, of which the sums over the basis take 3.5).
+  const bool basis = real && sv.barc && onchip_mix_ok(sv.oc, s.Dc) &&
+                     2 * onchip_fwd_ctas(sv.oc) <= 152 * onchip_fwd_resident(sv.oc);
   if (s.D <= 256 && N >= 2 * kMinChunk) {
     KPlan pd = s.p;
     pd.S = (int)s.D;
@@ -2144,32 +2149,47 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     const int nD = sv.ocp && onchip_forward_ok(sv.ocp) ? onchip_fwd_ctas(sv.ocp) : 0;
     const int most = nD ? 152 * onchip_fwd_resident(sv.ocp) / nD : 0;
     if (most >= kMinSide) {
-      // A gradient's chunks are also recomputed and pulled back with S columns, which take fewer CTAs:
-      // more chunks than propagators fit at once (whole rounds of them, up to 8) until those fill
-      // the SMs.  D = 64 FP64, 4 columns: 57 chunks 26.5 ms (2 x 8.1 ms of passes with 57 CTAs), 456
-      // chunks 14.1 ms.
-      const int rounds = grad ? std::max(1, std::min(8, slots / most)) : 1;
-      c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + rounds * most - 1) / (rounds * most));
-      c.C = (N + c.L - 1) / c.L;
-      c.prop = c.par = c.C > 1;
-      c.R = grad ? fit_rounds(c.C, c.L) : 1;
-      // The product's order.  One level: C dependent matrix-times-column products.  Two: the
-      // C - 1 products of every group with D columns (over the SMs), then C/G + G dependent ones.
-      const double D = (double)s.D, one = c.C;
-      int G = std::max(1, (int)std::lround(std::sqrt((double)c.C)));
-      const double two = c.C * D / 152.0 + 2.0 * G + c.C / (double)G;
-      c.G = c.C;
-      if (two < one) c.G = G;
-      c.NG = (c.C + c.G - 1) / c.G;
-      // An evolution alone trades N steps for L of every column, a few launches (35 us) and C products
-      // that wait for one another (130 us each at D = 256, 85 at 243, 27 at 125).  In mixed steps of the serial
-      // evolution, 8 us with real operators (five levels 16) and 14 us on complex rows, which take twice as
-      // long with every column; FP64 steps are ten times as long.  D = 256, 16 columns, 32 steps: 1.04 ms in
+      // Chunks trade the N steps of a serial pass for steps of every column, a few launches (35 us) and
+      // C products that wait for one another (130 us each at D = 256, 85 at 243, 27 at 125), which
+      // are measured here in steps of the serial pass: mixed 8 us with real operators (five levels
+      // 16) and 14 us on complex rows, which take twice as long with every column; FP64 ten times as long.
+      //   Evolution, as many chunks as fit at once: L steps.  D = 256, 16 columns, 32 steps: 1.04 ms in
       // chunks, 0.45 serially; 300 steps 1.49 against 2.5.
-      const double q = (D / 256) * (D / 256), dl = s.p.dims[0];
-      const double cost = onchip_real(sv.ocp) ? (sv.mixed ? c.L + 4 + c.C * (dl == 5 ? 8 : 14) * q : c.L + c.C * q)
-                                              : 2 * c.L + 2 + c.C * (sv.mixed ? 8 : 1) * q;
-      if (!grad && cost >= N) c.prop = false;
+      //   Gradient: the propagators, the recompute and the pull-back of a chunk, products both ways.  The
+      // latter two run with S columns, which take fewer CTAs: up to eight rounds of propagators make
+      // more and shorter chunks (D = 64 FP64, 4 columns: 57 chunks 26.5 ms, 456 chunks 14.1).
+      // Without chunks: the serial passes each way, or side by side.  D = 256, 16 columns, 64 steps: 4.28 ms
+      // in chunks, 2.40 serially (6.3 before there were chunks); 1000 steps 18.1 in 250 chunks, 6.9 in 7.
+      const bool realp = onchip_real(sv.ocp);
+      const double D = (double)s.D, q = (D / 256) * (D / 256);
+      const double wait = sv.mixed ? (realp ? (s.p.dims[0] == 5 ? 8 : 14) : 8) * q : q;
+      const double all = realp ? 1 : 2, over = sv.mixed ? (realp ? 4 : 2) : 0;
+      double best = !grad ? N : real ? (basis ? 1.0 : 2.0) * N : 2.0 * N + 4.0 * std::max(kMinChunk, N / slots);
+      OcChunks b;
+      const int rounds = grad ? std::max(1, std::min(8, slots / most)) : 1;
+      // mixed: the best number of rounds; FP64 and complex rows have steps so long that the most are
+      for (int r = sv.mixed && realp ? 1 : rounds; r <= rounds; ++r) {
+        c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + r * most - 1) / (r * most));
+        c.C = (N + c.L - 1) / c.L;
+        // The product's order.  One level: C dependent matrix-times-column products.  Two: the
+        // C - 1 products of every group with D columns (over the SMs), then C/G + G dependent ones.
+        const double one = c.C;
+        int G = std::max(1, (int)std::lround(std::sqrt((double)c.C)));
+        const double two = c.C * D / 152.0 + 2.0 * G + c.C / (double)G;
+        c.G = two < one ? G : c.C;
+        c.NG = (c.C + c.G - 1) / c.G;
+        const int waves = (c.C + most - 1) / most;
+        const double cost = all * waves * c.L + over + (grad ? 2 : 1) * std::min(one, two) * wait +
+                            (grad ? (real ? 2.0 : 4.0) * c.L + over : 0.0);
+        if (c.C > 1 && cost < best) {
+          best = cost;
+          b = c;
+        }
+        if (grad && ckpt > 0) break;
+      }
+      c = b;
+      c.prop = c.par = b.C > 1;
+      c.R = grad && c.prop ? fit_rounds(c.C, c.L) : 1;
       const size_t nprop = (size_t)s.D * onchip_columns(sv.ocp) + (c.NG > 1 ? (size_t)s.D * s.D / c.G + 1 : 0);
       if (c.prop && bytes(grad ? c.C : 0, c.L, grad ? c.R : 0, 0) + c.C * nprop * sizeof(double2) <= work_limit) return;
       c = OcChunks{};
@@ -2177,13 +2197,9 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     }
   }
   if (!grad) return;
-  // The two serial passes run side by side when the SMs hold both and every computational row has
-  // an image column: D = 3125 with 32 columns takes 32 CTAs each way (1000 steps with their
-  // gradient: 62 -> 40.6 ms, of which the sums over the basis take 3.5).
-  const bool basis = real && sv.barc && onchip_mix_ok(sv.oc, s.Dc) &&
-                     2 * onchip_fwd_ctas(sv.oc) <= 152 * onchip_fwd_resident(sv.oc);
-  // real operators: the two serial passes keep all stage inputs when there is room
-  if (real && ckpt <= 0 && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
+  // real operators: the two serial passes keep all stage inputs when there is room, and one requested
+  // chunk of all steps keeps them anyway
+  if (real && (ckpt <= 0 || ckpt >= N) && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
     c.direct = true;
     c.basis = basis;
     return;

@@ -26,16 +26,18 @@ def _system(ctx, op, seed):
 
 
 def test_packed_solves_keep_their_own_gauge(sgctx):
-    from paper_2406_18155_gb300.api import Server
+    from paper_2406_18155_gb300.api import Server, System
     T, dt, cols = 0.6, 0.01, W.comp_states([3, 3])
     target = W.haar_unitary(4, np.random.Generator(np.random.PCG64(2)))
     ops = [X, Y, Y, X]
     alone = [_system(sgctx, op, i).fidelity_grad(T, dt, target, cols, precision="mixed") for i, op in enumerate(ops)]
     srv = Server(sgctx, mem_budget_bytes=8 << 30, max_slots=1, max_batch=4)
     # a first request holds the slot while the others queue up behind it
-    first = _system(sgctx, X, 9)
-    tickets = [srv.submit(first, 60.0, dt, target, cols)]
+    wl = W.fluxonium_chain(seed=1, nq=4, levels=4, T=10.0, dt=dt)
+    first = System.from_workload(sgctx, wl)
+    first.prepare()
     systems = [_system(sgctx, op, i) for i, op in enumerate(ops)]
+    tickets = [srv.submit(first, wl["T"], dt, wl["target"], wl["col_index"], kind="state", precision="fp64")]
     tickets += [srv.submit(s, T, dt, target, cols) for s in systems]
     res = [srv.wait(t) for t in tickets][1:]
     assert srv.stats()["batched_requests"] >= 2
