@@ -843,36 +843,34 @@ k_ocr_dens(const __grid_constant__ OcdArgs a, const __grid_constant__ OcdJob jb)
   double* const geR = geL + (long long)a.ne * SG_MAXD;
   double* const gjb = geR + (long long)a.ne * SG_MAXD;
   const double Je = S.kind ? jb.J[S.edge] : 1.0;
-  // side 0: C without J; the co-gradient of A and the energies take it, dF/dJ does not
-  const double sc = S.kind && S.side == 0 ? Je * S.sign : (S.kind ? (double)S.sign : 1.0);
+  // side 0: C without J; the co-gradient of A and the energies take it, dF/dJ does not.  Side 1's matrix
+  // carries J and the sign already.
+  const double s1 = !S.kind || S.side ? 1.0 : Je * S.sign;
   double* const ob = S.kind == 0 ? gD + 2ll * S.drv * MD2 : (S.side ? gR : gL) + 2ll * S.edge * MD2;
   double* const eb = S.kind == 0 ? geB + S.mslot * SG_MAXD : (S.side ? geR : geL) + S.edge * SG_MAXD;
-  double dj = 0.0, eI[NPR], eR[NPR];
-#pragma unroll
-  for (int i = 0; i < NPR; ++i) {
-    eI[i] = hs * __shfl_sync(0xffffffffu, kI, i);
-    eR[i] = hs * __shfl_sync(0xffffffffu, kR, i);
+  // lane p has element p's sums; lane x gathers level x (one lane for all took 12 to 36 dependent
+  // accesses to memory per slot, slot after slot: 0.2 ms of a launch)
+  double eR = 0.0, dj = 0.0;
+  int x = 0, y = 0;
+  if (on && lane < NPR) {
+    int r = lane;
+    while (r >= zn<DL>(x)) r -= zn<DL>(x++);
+    y = zc(x, r);
+    const double m = r_elem(jb.opd[S.off + x * DL + y], S.part, S.flip, x);
+    ob[2 * (x * SG_MAXD + y) + (S.part ? 1 : 0)] += r_sign(S.part, S.flip, x) * s1 * (hs * kI);
+    eR = s1 * m * (hs * kR);
+    dj = m * (hs * kI);
+  }
+  dj = warp_sum(dj);
+  if (on && S.kind && S.side == 0 && lane == 0) gjb[S.edge] += S.sign * dj;
+  double mine = 0.0;
+  for (int l = 0; l < DL; ++l) {
+    const double v = warp_sum(lane < NPR ? (x == l ? eR : 0.0) - (y == l ? eR : 0.0) : 0.0);
+    if (lane == l) mine = v;
   }
   // one warp after the other: drives of one mode add to the same energies
   for (int turn = 0; turn < a.nslot; ++turn) {
-    if (w == turn && lane == 0) {
-      int p = 0;
-#pragma unroll
-      for (int x = 0; x < DL; ++x)
-#pragma unroll
-        for (int j = 0; j < zn<DL>(x); ++j, ++p) {
-          const int y = zc(x, j);
-          const double2 o = jb.opd[S.off + x * DL + y];
-          const double m = r_elem(o, S.part, S.flip, x);
-          // side 1's matrix carries J and the sign already
-          const double s1 = S.kind && S.side == 1 ? 1.0 : sc;
-          ob[2 * (x * SG_MAXD + y) + (S.part ? 1 : 0)] += r_sign(S.part, S.flip, x) * s1 * eI[p];
-          eb[x] += s1 * m * eR[p];
-          eb[y] -= s1 * m * eR[p];
-          dj += m * eI[p];
-        }
-      if (S.kind && S.side == 0) gjb[S.edge] += S.sign * dj;
-    }
+    if (on && w == turn && lane < DL) eb[lane] += mine;
     __syncthreads();
   }
 }

@@ -43,4 +43,4 @@ def test_sizes_at_the_slot_limit(sgctx, monkeypatch, nq, levels, ring, driven, o
             assert m != n, (steps, p, m, n)
     if on_chip:
         for p in ("fp64", "mixed"):
-            assert out[21][p][3] <= out[9][p][3] + 4, (out[9][p][3], out[21][p][3])
+            assert out[21][p][3] < out[9][p][3] + 12, (out[9][p][3], out[21][p][3])     # a launch a step
