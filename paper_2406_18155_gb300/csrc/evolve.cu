@@ -1719,6 +1719,8 @@ struct KTimer {
   }
 };
 
+constexpr int kMinChunk = 4;      // steps of a chunk at least: below this the products outweigh the steps saved
+
 // An on-chip solve's steps in C chunks of L.  prop: every chunk's propagator is computed
 // (all chunks side by side) and the states and co-states at the chunk boundaries follow by
 // products; otherwise one serial pass each writes them.  par: the gradient's chunks run
@@ -1891,9 +1893,12 @@ sg_status upload_and_tables(sg_system* sys, const sg_evolve_opts* o, Solve& sv, 
   // a solve goes before its first kernel (see dcopy)
   sv.mixed = o->precision == SG_MIXED;
   const int pc = path_choice();
-  // A mixed evolution of a few steps on a small system is one serial launch (plan_chunks), where complex rows
+  // An evolution of a few steps on a small system is one serial launch (plan_chunks), where complex rows
   // have less to set up: D = 25, four steps 0.14 ms, real operators 0.18; D = 125, eight steps 0.23 and 0.28
-  const bool few = !grad && sv.mixed && (s.D <= 64 ? s.N < 10 : s.p.dims[0] == 5 && s.D <= 125 && s.N < 16);
+  // (FP64: D = 9, four steps 0.22 and 0.26)
+  const bool few = !grad && (!sv.mixed   ? s.D <= 9 && s.N < 2 * kMinChunk
+                             : s.D <= 64 ? s.N < 10
+                                         : s.p.dims[0] == 5 && s.D <= 125 && s.N < 16);
   if (!s.q2 && s.frame == SG_FRAME_INTERACTION && !sv.two_rows && !few) {
     fill_terms(s, s.ta, sv.rterms);
     sv.real_oc = real_gauge(sys, s, sv.rterms);
@@ -2103,7 +2108,6 @@ void dcopy(double2* dst, const double2* src, long long n, cudaStream_t st) {
 // at the level counts here).  Beyond that the boundary states come from one serial pass
 // each way.
 constexpr int kMinSide = 4;
-constexpr int kMinChunk = 4;      // steps: below this the products outweigh the steps saved
 constexpr size_t kSegBytes = 1ull << 30;      // stage inputs of one round of chunks
 constexpr size_t kDirectBytes = 8ull << 30;   // of a whole solve (real operators, no propagators)
 
@@ -2198,8 +2202,8 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   }
   if (!grad) return;
   // real operators: the two serial passes keep all stage inputs when there is room, and one requested
-  // chunk of all steps keeps them anyway
-  if (real && (ckpt <= 0 || ckpt >= N) && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
+  // chunk of all steps keeps them anyway, as a few steps always may
+  if (real && (ckpt <= 0 || ckpt >= N || N <= kMinChunk) && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
     c.direct = true;
     c.basis = basis;
     return;
