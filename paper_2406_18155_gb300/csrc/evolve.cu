@@ -2146,6 +2146,10 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
   // gradient: 62 -> 40.6 ms, of which the sums over the basis take 3.5).
   const bool basis = real && sv.barc && onchip_mix_ok(sv.oc, s.Dc) &&
                      2 * onchip_fwd_ctas(sv.oc) <= 152 * onchip_fwd_resident(sv.oc);
+  // real operators: the two serial passes keep all stage inputs when there is room, and one requested
+  // chunk of all steps keeps them anyway, as a few steps always may
+  const bool direct = real && (ckpt <= 0 || ckpt >= N || N <= kMinChunk) && (size_t)N * 4 * stage <= kDirectBytes &&
+                      bytes(1, N, 1, 0) <= work_limit;
   if (s.D <= 256 && N >= 2 * kMinChunk) {
     KPlan pd = s.p;
     pd.S = (int)s.D;
@@ -2168,7 +2172,8 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
       const double D = (double)s.D, q = (D / 256) * (D / 256);
       const double wait = sv.mixed ? (realp ? (s.p.dims[0] == 5 ? 8 : 14) : 8) * q : q;
       const double all = realp ? 1 : 2, over = sv.mixed ? (realp ? 4 : 2) : 0;
-      double best = !grad ? N : real ? (basis ? 1.0 : 2.0) * N : 2.0 * N + 4.0 * std::max(kMinChunk, N / slots);
+      const int Ls = ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, N / slots);      // their chunks, if any
+      double best = !grad ? N : real ? (basis ? 1.0 : 2.0) * N + (direct ? 0.0 : 2.0 * Ls) : 2.0 * N + 4.0 * Ls;
       OcChunks b;
       const int rounds = grad ? std::max(1, std::min(8, slots / most)) : 1;
       // mixed: the best number of rounds; FP64 and complex rows have steps so long that the most are
@@ -2201,9 +2206,7 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
     }
   }
   if (!grad) return;
-  // real operators: the two serial passes keep all stage inputs when there is room, and one requested
-  // chunk of all steps keeps them anyway, as a few steps always may
-  if (real && (ckpt <= 0 || ckpt >= N || N <= kMinChunk) && (size_t)N * 4 * stage <= kDirectBytes && bytes(1, N, 1, 0) <= work_limit) {
+  if (direct) {
     c.direct = true;
     c.basis = basis;
     return;
