@@ -296,8 +296,8 @@ sg_status sg_gate_fidelity_open(sg_system* sys, const sg_evolve_opts* opts, cons
  * eigen-derivatives (the collapse operators are held fixed in the truncated
  * eigenbasis).  Exact derivative of the discrete map: the Dc^2 columns are pulled back
  * through each RK4 step by the adjoint of the non-Hermitian generator (stage rows of
- * H_eff^dag), from segment checkpoints every ckpt steps (0: round(sqrt(N))).  opts: T,
- * dt, precision, frame (ncols and col_index ignored; RK4 only). */
+ * H_eff^dag), from chunks of ckpt steps (0: the library's choice, see sg_fidelity_grad).
+ * opts: T, dt, precision, frame (ncols and col_index ignored; RK4 only). */
 sg_status sg_gate_fidelity_open_grad(sg_system* sys, const sg_evolve_opts* opts, const double* target_re_im,
                                      int kind, double* F_out, double* grad_pulse, double* grad_ham, int ckpt);
 
@@ -311,7 +311,10 @@ sg_status sg_gate_fidelity_open_grad(sg_system* sys, const sg_evolve_opts* opts,
  * phases, form the constant operand [C; O_1; ...; O_K] of tcgen05 TF32 matrix
  * products with the state z = P^dag y (P the frame phases), each product split into
  * three TF32 products (3xTF32, about FP32 accuracy, accumulated in FP32 in tensor
- * memory); the RK4 stage math is FP32 and the state float-float.  Requires
+ * memory); the RK4 stage math is FP32 and the state float-float.  Pairs of modes with 16
+ * columns and one structure run on the on-chip kernel of real operators instead, with the
+ * coefficients (12 bytes per drive) and frame phases (8 per level) of every system and step in
+ * device memory, where there is room for them.  Requires
  * opts->precision == SG_MIXED and the RK4 solver; S = ncols in {4, 8, 16};
  * (1 + drives) x D, with D rounded up to a multiple of 8, at most 128 (for
  * example D = 16 with one drive: 4 systems per CTA; D = 25: 2); D <= 64; every
@@ -334,8 +337,13 @@ sg_status sg_fidelity(sg_system* sys, const sg_evolve_opts* opts, const double* 
                       double* F_out, double* Ucomp_out);
 
 /* F (of `kind`) and dF/dtheta by the exact discrete adjoint of RK4, with the forward
- * states recomputed per segment from checkpoints every `ckpt_interval` steps (0 =
- * about sqrt(N)).  grad_pulse / grad_ham are host arrays of sg_param_counts sizes.
+ * states recomputed in chunks of `ckpt_interval` steps from the states at their starts.
+ * 0: the library's choice.  Systems of one tile (D <= 4096, one level count) then run
+ * their chunks side by side, or keep the stage inputs of all steps: up to 8 GiB of them,
+ * else 1 GiB at a time, the states at the chunks' ends and, for D <= 256, the chunks'
+ * propagators (16 D^2 bytes each).  Where that much memory is not to be had the chunks run one
+ * after the other, about sqrt(N) steps each (half as long where a stage keeps states and
+ * co-states), as they do on other systems.  grad_pulse / grad_ham are host arrays of sg_param_counts sizes.
  * grad_ham may be NULL: the Hamiltonian-parameter gradient is then not computed,
  * which skips the cross-densities of the coupling terms (the pulse gradient needs
  * only those of the driven terms) and gives the same grad_pulse.
@@ -423,8 +431,10 @@ typedef struct {
  * free and the device memory they need fits `mem_budget_bytes`; each admitted
  * request runs as one fidelity(+gradient) solve on its slot's stream, so the
  * kernels of all admitted requests overlap on the device, and a request that
- * arrives while others run starts as soon as a slot and memory free up.
- * Results do not depend on what else runs (each solve has its own buffers and
+ * arrives while others run starts as soon as a slot and memory free up.  A request
+ * takes what its solve needs and, to run its chunks of steps side by side, up to an equal
+ * share of the budget (mem_budget_bytes / (max_slots max_batch), less what it needs);
+ * with less its chunks run one after the other.  Results do not depend on what else runs (each solve has its own buffers and
  * fixed-order reductions).  gpu_busy_frac in sg_stats is the fraction of the
  * server's wall time with at least one request running, not a device occupancy. */
 sg_status sg_server_create(sg_ctx* ctx, size_t mem_budget_bytes, int max_slots, sg_server** out);

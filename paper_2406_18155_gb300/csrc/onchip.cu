@@ -839,7 +839,6 @@ constexpr int kMixT = 64, kMixMax = 64;      // entries per block; columns at mo
 template <typename C>
 __global__ void __launch_bounds__(256) k_oc_mix(C* __restrict__ img, const double2* __restrict__ W, int nin, int nout,
                                                 int cols, int D) {
-  typedef decltype(C().x) R;
   extern __shared__ __align__(16) unsigned char msm[];
   C* const in = reinterpret_cast<C*>(msm);               // nin x kMixT
   C* const w = in + nin * kMixT;                         // nin x out4
@@ -879,7 +878,6 @@ __global__ void __launch_bounds__(256) k_oc_mix(C* __restrict__ img, const doubl
         if (s0 + k < cols && t < nt) base[(size_t)(s0 + k) * D + t0 + t] = a[k][e];
       }
   }
-  (void)sizeof(R);
 }
 
 // FP64 -> FP32 copy of the per-stage phase and coefficient tables and the operators.

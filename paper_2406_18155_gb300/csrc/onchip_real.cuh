@@ -38,9 +38,9 @@
 // (complex rows 6.5e-7), Hamiltonian gradient 9.6e-7 -> 2.8e-7 (2.1e-6); five modes of four levels, 2560
 // steps: state 1.2e-7 -> 9e-8; at the same speed (1.57 ms, 6-mode chain 106 ms).
 //
-// psi stays in the interaction picture, so no phase error accumulates in it: P_m is read from the phase table every step.
-// Real times complex halves the multiply-adds (one packed FP32x2 FMA each), and the
-// matrices stay in shared memory for the whole run; a stage reads K drive coefficients
+// psi stays in the interaction picture, so no phase error accumulates in it: P_m is read from the
+// phase table every step.  Real times complex halves the multiply-adds (one packed FP32x2 FMA
+// each), and the matrices stay in shared memory for the whole run; a stage reads K drive coefficients
 // from memory instead of a row of term matrices.
 //
 // Work split.  A thread owns one d x d block over two modes at a time.  The modes are
