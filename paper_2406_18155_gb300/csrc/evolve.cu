@@ -2820,9 +2820,9 @@ size_t sg_chunk_bytes(const sg_system* sys, const sg_evolve_opts* o, bool grad) 
     C = std::max(C, std::min(N / kMinChunk + 1, 152.0 * 8 * waves / std::max(1.0, S * D / (d * d) / 256)));
     const double blocks = 152.0 * 32 * std::max(1.0, S * D / (d * d) / 128);      // accumulators
     const double acc = 8.0 * (130.0 * sys->drives.size() + 290.0 * sys->couplings.size() + 10.0 * sys->modes.size());
-    // all stage inputs where plan_chunks keeps them (S columns or more; beyond D = 256, or where FP64
-    // propagators of D near it are too few), else a round's
-    const bool direct = 8 * N * D * S * cs <= (double)kDirectBytes && (D > 256 || (cs == 16 && D > 125));
+    // all stage inputs where plan_chunks may keep them (S columns or more; for smaller D propagators are
+    // shorter at any N that makes them many), else a round's
+    const bool direct = 8 * N * D * S * cs <= (double)kDirectBytes && D > 64;
     b += 2 * C * image + std::min(seg, direct ? (double)kDirectBytes : 1.5 * (double)kSegBytes) + std::min(N, blocks) * acc;
   }
   return (size_t)(1.25 * b) + (32u << 20);
