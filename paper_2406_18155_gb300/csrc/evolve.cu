@@ -2175,10 +2175,12 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
       const int Ls = ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, N / slots);      // their chunks, if any
       double best = !grad ? N : real ? (basis ? 1.0 : 2.0) * N + (direct ? 0.0 : 2.0 * Ls) : 2.0 * N + 4.0 * Ls;
       OcChunks b;
+      // one requested chunk of all steps leaves the complex rows free to choose (real operators keep its inputs)
+      const bool fixed = grad && ckpt > 0 && (real || ckpt < N);
       const int rounds = grad ? std::max(1, std::min(8, slots / most)) : 1;
       // mixed: the best number of rounds; FP64 and complex rows have steps so long that the most are
       for (int r = sv.mixed && realp ? 1 : rounds; r <= rounds; ++r) {
-        c.L = grad && ckpt > 0 ? std::min(ckpt, N) : std::max(kMinChunk, (N + r * most - 1) / (r * most));
+        c.L = fixed ? std::min(ckpt, N) : std::max(kMinChunk, (N + r * most - 1) / (r * most));
         c.C = (N + c.L - 1) / c.L;
         // The product's order.  One level: C dependent matrix-times-column products.  Two: the
         // C - 1 products of every group with D columns (over the SMs), then C/G + G dependent ones.
@@ -2194,7 +2196,7 @@ void plan_chunks(Solve& sv, bool grad, int ckpt, size_t work_limit) {
           best = cost;
           b = c;
         }
-        if (grad && ckpt > 0) break;
+        if (fixed) break;
       }
       c = b;
       c.prop = c.par = b.C > 1;
